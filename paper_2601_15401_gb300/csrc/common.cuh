@@ -1,10 +1,9 @@
 // Device-side modular arithmetic and launch descriptors shared by the kernels.
 //
-// Residues are uint64 in [0, q) with every modulus q < 2^61, so lazy values up
-// to 4q fit a 64-bit word. Three multiplications are used:
-//   * Shoup (constant operand w with companion w' = floor(w 2^64 / q)):
-//     x w - floor(x w' / 2^64) q lies in [0, 2q) for any x < 2^64 (Shoup's
-//     precomputed-quotient method, as used in Harvey's NTT butterflies);
+// Residues are uint64 in [0, q) with every modulus q < 2^61. Three
+// multiplications are used:
+//   * Shoup (constant operand, arith.cuh): signed lazy values in the NTT,
+//     canonical ones elsewhere;
 //   * Montgomery REDC with R = 2^64 for variable products and for 128-bit
 //     dot products: for T = hi 2^64 + lo with hi < q,
 //     m = lo q^-1 mod 2^64 gives T R^-1 = hi - floor(m q / 2^64) (mod q),
@@ -14,46 +13,19 @@
 #include <cstdint>
 #include <cuda_runtime.h>
 
-typedef unsigned long long u64;
-typedef long long i64;
+#include "arith.cuh"
 
 #define CKKS_MAX_PRIMES 64
 #define CKKS_MAX_TUPLE 13   // k <= 12 inputs give at most 13 polynomials
 
-struct ModQ {
-    u64 q;      // modulus
-    u64 qinv;   // q^-1 mod 2^64 (Montgomery)
+struct __align__(16) ModQ {
+    u64 q;        // modulus
+    u64 qinv;     // q^-1 mod 2^64 (Montgomery)
+    Canon canon;  // reduction of small multiples of q (arith.cuh)
+    u64 pad;
 };
 
 __device__ __forceinline__ u64 mulhi64(u64 a, u64 b) { return __umul64hi(a, b); }
-
-// x * w mod q in [0, 2q), w < q, wp = floor(w 2^64 / q), any x < 2^64.
-__device__ __forceinline__ u64 shoup_lazy(u64 x, u64 w, u64 wp, u64 q) {
-    return x * w - mulhi64(x, wp) * q;
-}
-
-// The same for a modulus q = 1 (mod 2^32), q = qh 2^32 + 1: with
-// h = floor(x w'/2^64), h q = h + h qh 2^32, so modulo 2^64 the quotient
-// product needs only the low 32 bits of h qh (one 32-bit multiply instead of
-// a 64 x 64-bit low product).
-__device__ __forceinline__ u64 shoup_lazy_q1(u64 x, u64 w, u64 wp, uint32_t qh) {
-    const u64 h = mulhi64(x, wp);
-    const uint32_t t = (uint32_t)h * qh;
-    return x * w - h - ((u64)t << 32);
-}
-
-__device__ __forceinline__ u64 reduce2(u64 x, u64 q) { return x >= q ? x - q : x; }
-
-__device__ __forceinline__ u64 shoup(u64 x, u64 w, u64 wp, u64 q) {
-    return reduce2(shoup_lazy(x, w, wp, q), q);
-}
-
-// [0, 4q) -> [0, q)
-__device__ __forceinline__ u64 reduce4(u64 x, u64 q) {
-    u64 q2 = q << 1;
-    x = x >= q2 ? x - q2 : x;
-    return x >= q ? x - q : x;
-}
 
 __device__ __forceinline__ u64 add_mod(u64 a, u64 b, u64 q) {
     u64 s = a + b;
@@ -91,17 +63,6 @@ __device__ __forceinline__ u64 redc_q1(u64 hi, u64 lo, u64 q) {
 
 // The modular products in two forms selected at compile time: Q1 = true for
 // contexts whose primes are all 1 (mod 2^32).
-template <bool Q1>
-__device__ __forceinline__ u64 shoup_lazy_t(u64 x, u64 w, u64 wp, u64 q) {
-    if constexpr (Q1) return shoup_lazy_q1(x, w, wp, (uint32_t)(q >> 32));
-    else return shoup_lazy(x, w, wp, q);
-}
-
-template <bool Q1>
-__device__ __forceinline__ u64 shoup_t(u64 x, u64 w, u64 wp, u64 q) {
-    return reduce2(shoup_lazy_t<Q1>(x, w, wp, q), q);
-}
-
 template <bool Q1>
 __device__ __forceinline__ u64 redc_t(u64 hi, u64 lo, ModQ m) {
     if constexpr (Q1) return redc_q1(hi, lo, m.q);
@@ -155,11 +116,6 @@ struct Acc128Lazy {
     // the same calls as Acc128 (the modulus is not needed)
     __device__ __forceinline__ void mac(u64 a, u64 b, u64) { mac(a, b); }
     __device__ __forceinline__ void add(u64 vhi, u64 vlo, u64) { add(vhi, vlo); }
-};
-
-// Shoup constant pair.
-struct Shoup {
-    u64 w, wp;
 };
 
 // Addressing of a set of limbs: limb (b, p, l) of a [batch][poly][limb][N]

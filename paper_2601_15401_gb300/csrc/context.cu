@@ -2,7 +2,8 @@
 //
 // Host arithmetic uses unsigned __int128. Tables (all per prime index x,
 // Q primes first):
-//   twiddles      psi^brv(k) and psi^-brv(k) with Shoup companions (NTT)
+//   twiddles      psi^brv(k) and psi^-brv(k) with Shoup companions, in the
+//                 order the NTT's passes read them (twiddle_slot)
 //   N^-1          Shoup constants (INTT)
 //   ModUp BConv   per level and digit: N^-1 [(Q_beta/q_j)^-1]_{q_j} (applied
 //                 in the INTT epilogue) and [(Q_beta/q_j) mod x] R (Eq. 4)
@@ -31,12 +32,7 @@ static u64 h_pow(u64 b, u64 e, u64 q) {
     return r;
 }
 static u64 h_inv(u64 a, u64 q) { return h_pow(a % q, q - 2, q); }
-static Shoup h_shoup(u64 w, u64 q) {
-    Shoup s;
-    s.w = w % q;
-    s.wp = (u64)(((u128)s.w << 64) / q);
-    return s;
-}
+static Shoup h_shoup(u64 w, u64 q) { return make_shoup(w % q, q); }
 static u64 h_mont_qinv(u64 q) {
     u64 x = q;  // Newton iteration for q^-1 mod 2^64 (q odd)
     for (int i = 0; i < 6; ++i) x *= 2 - q * x;
@@ -136,10 +132,14 @@ int context_build(Context &C, const uint32_t log_n, const uint32_t L, const uint
     std::vector<Shoup> pscale(C.K);
     std::vector<Shoup> pgadget((size_t)C.dnum * NP);
     std::vector<u64> powt(N);
+    std::vector<int> slot(N);  // table position of twiddle k
+    for (int k = 0; k < N; ++k) slot[k] = twiddle_slot(C.log_n, k);
     for (int x = 0; x < NP; ++x) {
         const u64 m = C.primes[x];
         mods[x].q = m;
         mods[x].qinv = h_mont_qinv(m);
+        mods[x].canon = make_canon(m);
+        mods[x].pad = 0;
         const u64 psi = h_min_psi(m, N);
         if (!psi) return -1;
         // forward: psi^brv(k); inverse: psi^-brv(k)
@@ -147,16 +147,16 @@ int context_build(Context &C, const uint32_t log_n, const uint32_t L, const uint
         for (int e = 1; e < N; ++e) powt[e] = h_mul(powt[e - 1], psi, m);
         for (int k = 0; k < N; ++k) {
             u64 w = powt[brv(k, C.log_n)];
-            Shoup s = h_shoup(w, m);
-            twf[(size_t)x * N + k] = make_ulonglong2(s.w, s.wp);
+            Shoup s = make_twiddle(w, m);
+            twf[(size_t)x * N + slot[k]] = make_ulonglong2(s.w, s.wp);
         }
         const u64 psi_inv = h_inv(psi, m);
         powt[0] = 1;
         for (int e = 1; e < N; ++e) powt[e] = h_mul(powt[e - 1], psi_inv, m);
         for (int k = 0; k < N; ++k) {
             u64 w = powt[brv(k, C.log_n)];
-            Shoup s = h_shoup(w, m);
-            twi[(size_t)x * N + k] = make_ulonglong2(s.w, s.wp);
+            Shoup s = make_twiddle(w, m);
+            twi[(size_t)x * N + slot[k]] = make_ulonglong2(s.w, s.wp);
         }
         ninv[x] = h_shoup(h_inv((u64)N % m, m), m);
         one[x] = h_shoup(1, m);

@@ -40,7 +40,7 @@ __global__ void pk_kernel(const u64 *S, const u64 *E, const u64 *a, u64 *pk, int
 
 // Garner lift of (x0 mod q0, x1 mod q1) to [0, q0 q1), centred, as double.
 __global__ void crt2_kernel(const u64 *P, double *out, int limbs, int N, u64 q0, u64 q1, Shoup q0inv_mod_q1,
-                            u64 one_q1) {
+                            Shoup one_q1) {
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= N) return;
     P += (i64)blockIdx.y * limbs * N;  // batch element
@@ -51,7 +51,7 @@ __global__ void crt2_kernel(const u64 *P, double *out, int limbs, int N, u64 q0,
         return;
     }
     const u64 x1 = P[N + i];
-    const u64 x0r = shoup(x0, 1, one_q1, q1);  // x0 mod q1
+    const u64 x0r = shoup(x0, one_q1.w, one_q1.wp, q1);  // x0 mod q1
     const u64 t = shoup(sub_mod(x1, x0r, q1), q0inv_mod_q1.w, q0inv_mod_q1.wp, q1);
     // x = x0 + q0 t < q0 q1 < 2^122
     unsigned __int128 x = (unsigned __int128)q0 * t + x0;
@@ -283,12 +283,10 @@ int ckks_decrypt_batch(ckks_context *ctx, const ckks_tuple *ct, uint32_t batch, 
     }
     if (err == cudaSuccess) {
         const u64 q0 = C.primes[0], q1 = limbs > 1 ? C.primes[1] : 1;
-        Shoup inv{0, 0};
-        u64 one_q1 = 0;
+        Shoup inv{0, 0}, one_q1{0, 0};
         if (limbs > 1) {
-            inv.w = host_inv(q0 % q1, q1);
-            inv.wp = (u64)(((unsigned __int128)inv.w << 64) / q1);
-            one_q1 = (u64)(((unsigned __int128)1 << 64) / q1);
+            inv = make_shoup(host_inv(q0 % q1, q1), q1);
+            one_q1 = make_shoup(1, q1);
         }
         count_kernel(C);
         crt2_kernel<<<dim3(blocks(N), batch), kThr, 0, st>>>(P, out, limbs, C.N, q0, q1, inv, one_q1);

@@ -34,7 +34,7 @@ enum OpCounter {
 
 struct NttPhase {
     int N, N1, N2;
-    int sub_per_tile, log_sub, log_n2;
+    int log_n2;
     const ModQ *mods;
     const ulonglong2 *tw_fwd;
     const ulonglong2 *tw_inv;
@@ -140,7 +140,7 @@ struct Context {
     Profiler prof;
     // launch tunables
     int tune_ntt_tile_cols = 4096;    // elements per CTA tile, column phases
-    int tune_ntt_tile_blocks = 4096;  // elements per CTA tile, block phases
+    int tune_ntt_tile_blocks = 4096;  // elements per CTA tile, block phases (at most kBlockTile are used)
     int tune_bconv_threads = 256;
     int tune_mac_threads = 256;
     // forms of the rescaling (same results; for measuring the paper's
@@ -194,6 +194,7 @@ inline void count_kernel(const Context &C) { count_op(C, OP_KERNELS, 1); }
 
 // ntt.cu
 void ntt_geometry(int logN, int &log_n1, int &log_n2);
+int twiddle_slot(int logN, int k);  // table position of twiddle k
 // phase launch over a device table of NttJob (ntt_launch.cu); jobs: device
 // array of n_jobs entries
 cudaError_t launch_ntt_phase_table(const Context &C, bool fwd, bool cols, const NttJob *jobs, int n_jobs,

@@ -2,53 +2,94 @@
 // described in ntt_kernel.cuh): phase geometry, algorithmic byte and Shoup
 // product counts for the timing hook, and the two-phase transform with fused
 // first load / last store.
+#include <algorithm>
+
 #include "common.cuh"
 #include "internal.h"
 #include "ntt_kernel.cuh"
 
 namespace ckks {
 
-// Geometry of the two phases for a given log N.
+// Geometry of the phases for a given log N: log_n1 = 0 (one phase) up to
+// N = 2^12, the largest limb one CTA holds.
 void ntt_geometry(int logN, int &log_n1, int &log_n2) {
-    if (logN <= 8) { log_n1 = 0; log_n2 = logN; }
+    if (logN <= kWholeMax) { log_n1 = 0; log_n2 = logN; }
     else { log_n1 = logN / 2; log_n2 = logN - log_n1; }
 }
 
-// Tile shape of one phase: sub-problems per CTA from the context's tile
-// tunables, CTAs per limb, threads and shared memory per CTA.
+// Table position of forward / inverse twiddle k (psi^(+-)brv(k)) in the order
+// the passes read it (ntt_kernel.cuh): k = m_glob + i, m_glob = 2^s, is stage s
+// of the transform; its first log_n1 stages run in the column phase, the
+// others in the block phase, in passes of up to CKKS_NTT_RMAX stages.
+int twiddle_slot(int logN, int k) {
+    if (k == 0) return 0;
+    int log_n1, log_n2;
+    ntt_geometry(logN, log_n1, log_n2);
+    int s = 0;
+    while ((k >> (s + 1)) != 0) ++s;
+    const bool cols = s < log_n1;
+    const int logn = cols ? log_n1 : log_n2;
+    const int ls = cols ? s : s - log_n1;          // stage within the phase
+    const int m_loc = 1 << ls;
+    const int i = cols ? k - m_loc : k & (m_loc - 1);  // group within the sub-problem
+    const int b = cols ? 0 : (k >> ls) - (1 << log_n1);  // k = m_loc (N1 + b) + i
+    // the pass of stage ls (Pass<LOGN, P> of the kernels)
+    const int np = (logn + CKKS_NTT_RMAX - 1) / CKKS_NTT_RMAX, base = logn / np, extra = logn % np;
+    int p = 0, start = 0, len = base + (0 < extra ? 1 : 0);
+    while (ls >= start + len) {
+        start += len;
+        ++p;
+        len = base + (p < extra ? 1 : 0);
+    }
+    const int ep = ls - start, g = i >> ep, j = i & ((1 << ep) - 1);
+    const int n_sub = cols ? 1 : 1 << log_n1;
+    return (n_sub << start) + ((b * ((1 << len) - 1) + (1 << ep) - 1 + j) << start) + g;
+}
+
+// Elements per CTA of the block phases, at most. Their warps do not wait for
+// each other, so a CTA is only the unit in which shared memory is given out:
+// two-warp CTAs start as soon as two warps have ended (forward / inverse block
+// phase of 384 limbs at N = 2^16: 143 / 145 us with 64 threads, 144 / 146 with
+// 128, 163 / 156 with 256).
+constexpr int kBlockTile = 1024;
+
+// Geometry of one phase: CTAs per limb, threads and shared memory per CTA. A
+// thread takes 16 points; the tile tunables set the elements per CTA (at
+// least one group of 16 columns or one warp of blocks, at most 256 threads
+// for columns and kBlockTile elements for blocks).
 static int phase_geometry(const Context &C, bool cols, NttPhase &P, PhaseLaunch &G) {
     int log_n1, log_n2;
     ntt_geometry(C.log_n, log_n1, log_n2);
     P.N = C.N;
     P.N1 = 1 << log_n1;
     P.N2 = 1 << log_n2;
+    P.log_n2 = log_n2;
     P.mods = C.d_mods;
     P.tw_fwd = C.d_tw_fwd;
     P.tw_inv = C.d_tw_inv;
-    int logn, n_sub;
-    if (cols) {
-        logn = log_n1;
-        int n = 1 << logn;
-        n_sub = C.tune_ntt_tile_cols / n;
-        if (n_sub > P.N2) n_sub = P.N2;
-        G.tiles = P.N2 / n_sub;
-        G.smem = (size_t)n * n_sub * sizeof(u64) + (CKKS_NTT_COL_TW_SMEM ? (size_t)n * sizeof(ulonglong2) : 0);
+    const int logn = cols ? log_n1 : log_n2, n = 1 << logn;
+    const int sets = n >= 16 ? n / 16 : 1;  // threads per sub-problem
+    G.shape = cols ? COLS : logn > 8 ? WHOLE : BLOCKS;
+    if (G.shape == COLS) {
+        const int group = 16 * sets;
+        int groups = C.tune_ntt_tile_cols / (16 * n);
+        groups = std::max(1, std::min(groups, std::min(256 / group, P.N2 / 16)));
+        G.tiles = P.N2 / 16 / groups;
+        G.threads = groups * group;
+        G.smem = (size_t)groups * 16 * n * sizeof(u64) + (size_t)n * sizeof(ulonglong2);
+    } else if (G.shape == WHOLE) {
+        G.tiles = 1;
+        G.threads = sets;
+        G.smem = (size_t)(n + n / 16) * sizeof(u64) + (size_t)(n - 1) * sizeof(ulonglong2);
     } else {
-        logn = log_n2;
-        int n = 1 << logn;
-        n_sub = C.tune_ntt_tile_blocks / n;
-        if (n_sub < 1) n_sub = 1;
-        if (n_sub > P.N1) n_sub = P.N1;
-        G.tiles = P.N1 / n_sub;
-        G.smem = (size_t)n_sub * (n + n / 16) * sizeof(u64);
+        int threads = std::min(C.tune_ntt_tile_blocks, kBlockTile) / 16;
+        threads = std::max(32, std::min(threads, P.N1 * sets));
+        const int blocks = threads / sets;
+        G.tiles = (P.N1 + blocks - 1) / blocks;
+        G.threads = threads;
+        // per warp: its blocks (one pad word per 16) and their n - 1 twiddles each (Geo::warp_bytes)
+        G.smem = (size_t)blocks * ((n + n / 16) * sizeof(u64) + (n - 1) * sizeof(ulonglong2));
     }
-    P.sub_per_tile = n_sub;
-    P.log_sub = 0;
-    while ((1 << P.log_sub) < n_sub) ++P.log_sub;
-    P.log_n2 = log_n2;
-    int per_sub = (1 << logn) >= (1 << CKKS_NTT_RMAX) ? (1 << logn) >> CKKS_NTT_RMAX : 1;  // point sets per sub-problem
-    int threads = ((n_sub * per_sub + 31) / 32) * 32;
-    G.threads = threads > 256 ? 256 : threads;
     return logn;
 }
 
@@ -82,14 +123,11 @@ cudaError_t launch_ntt_phase(const Context &C, bool fwd, bool cols, const LimbJo
     if (S.mode == ST_SCALE || S.mode == ST_MODDOWN || S.mode == ST_MRS) ops += jobs_d * (double)C.N;
     ProfScope ps(C, fwd ? (cols ? KC_NTT_FWD_COLS : KC_NTT_FWD_BLOCKS) : (cols ? KC_NTT_INV_COLS : KC_NTT_INV_BLOCKS),
                  bytes, st, ops);
-    if (C.q1()) {
-        bool found;
-        const cudaError_t e = fwd ? ntt_dispatch_q1_uniform_fwd(cols, logn, P, J, L, S, G, found)
-                                  : ntt_dispatch_q1_uniform_inv(cols, logn, P, J, L, S, G, found);
-        if (found) return e;
-    }
-    return fwd ? ntt_dispatch_uniform_fwd(cols, logn, P, J, L, S, G)
-               : ntt_dispatch_uniform_inv(cols, logn, P, J, L, S, G);
+    if (P.N1 == 1)
+        return fwd ? ntt_whole_uf(logn, P, &J, nullptr, 0, L, S, G) : ntt_whole_ui(logn, P, &J, nullptr, 0, L, S, G);
+    if (C.q1() && C.log_n >= 14)
+        return fwd ? ntt_two_uf1(logn, P, &J, nullptr, 0, L, S, G) : ntt_two_ui1(logn, P, &J, nullptr, 0, L, S, G);
+    return fwd ? ntt_two_uf(logn, P, &J, nullptr, 0, L, S, G) : ntt_two_ui(logn, P, &J, nullptr, 0, L, S, G);
 }
 
 // One phase over a device table of limbs (cross-shape launches). The caller
@@ -107,14 +145,13 @@ cudaError_t launch_ntt_phase_table(const Context &C, bool fwd, bool cols, const 
     count_kernel(C);
     ProfScope ps(C, fwd ? (cols ? KC_NTT_FWD_COLS : KC_NTT_FWD_BLOCKS) : (cols ? KC_NTT_INV_COLS : KC_NTT_INV_BLOCKS),
                  alg_bytes, st, ops);
-    if (C.q1()) {
-        bool found;
-        const cudaError_t e = fwd ? ntt_dispatch_q1_table_fwd(cols, logn, P, jobs, n_jobs, L, S, G, found)
-                                  : ntt_dispatch_q1_table_inv(cols, logn, P, jobs, n_jobs, L, S, G, found);
-        if (found) return e;
-    }
-    return fwd ? ntt_dispatch_table_fwd(cols, logn, P, jobs, n_jobs, L, S, G)
-               : ntt_dispatch_table_inv(cols, logn, P, jobs, n_jobs, L, S, G);
+    if (P.N1 == 1)
+        return fwd ? ntt_whole_tf(logn, P, nullptr, jobs, n_jobs, L, S, G)
+                   : ntt_whole_ti(logn, P, nullptr, jobs, n_jobs, L, S, G);
+    if (C.q1() && C.log_n >= 14)
+        return fwd ? ntt_two_tf1(logn, P, nullptr, jobs, n_jobs, L, S, G)
+                   : ntt_two_ti1(logn, P, nullptr, jobs, n_jobs, L, S, G);
+    return fwd ? ntt_two_tf(logn, P, nullptr, jobs, n_jobs, L, S, G) : ntt_two_ti(logn, P, nullptr, jobs, n_jobs, L, S, G);
 }
 
 // Full transform src -> dst with fused first load / last store. The first

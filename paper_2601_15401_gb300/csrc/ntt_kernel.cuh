@@ -1,6 +1,6 @@
 // Negacyclic NTT / INTT phase kernels over 64-bit NTT-friendly primes
-// (device code; instantiated by ntt_uf.cu, ntt_ui.cu, ntt_tf.cu, ntt_ti.cu,
-// the host logic is in ntt.cu).
+// (device code; instantiated by ntt_[ut][fi][1].cu and ntt_whole_[ut].cu, the
+// host logic is in ntt.cu).
 //
 // The transform is the evaluation map A[i] = sum_j a_j psi^((2 brv(i)+1) j)
 // (bit-reversed order), computed with Cooley-Tukey butterflies forward and
@@ -11,18 +11,28 @@
 // e = c + k N2. The forward transform's first log2 N1 stages only pair
 // elements of the same column c; its last log2 N2 stages only pair elements
 // of the same row block [b N2, (b+1) N2). So the transform runs as two
-// launches (column phase, block phase), each CTA loading a tile of whole
-// columns or whole blocks into shared memory, running its stages there and
-// writing back. The inverse runs the block phase first. N <= 256 runs one
-// block phase over the whole limb.
+// launches (column phase, block phase), each thread group loading whole
+// columns or whole blocks, running their stages in registers and shared
+// memory and writing back. The inverse runs the block phase first. N <= 2^12
+// runs all stages in one launch, the whole limb in one CTA.
 //
 // Inside a phase the sub-transform of n = 2^LOGN points is done in passes of
 // up to 4 stages: a thread holds 2^r points of one sub-problem in registers
 // (radix-2^r), runs r butterfly stages on them and writes them back; passes
-// are separated by __syncthreads. Butterflies are lazy (Harvey): forward
-// values stay in [0, 4q), inverse values in [0, 2q).
+// are separated by a barrier. Butterflies are lazy on signed values
+// (arith.cuh), with the corrections the prime's size asks for; a CTA works on
+// one limb, so the choice is one uniform branch per CTA:
+//   small primes (q < 2^53): forward values grow by 2.25 q a stage, at most
+//     101 q over 16 stages (64 q of that from an Eq. 17 load), no correction
+//     at all; inverse sums double every stage, so the one output of a pass
+//     that is a sum at all its stages is brought to [0, 2q) after the pass
+//     (the others end below 18 q, the next pass's sums below 288 q);
+//   big primes: forward values grow by q a stage, and the intermediate between
+//     the two phases is stored canonical (at most 8 stages, below 8 q; from
+//     2^60 on the sums are folded every second stage); inverse sums are
+//     folded to |x| <= q at every stage.
 //
-// Twiddles: tw[prime][k] = (psi^brv(k), Shoup companion) for the forward,
+// Twiddles: tw[prime][k] = (psi^brv(k), companion) for the forward,
 // psi^-brv(k) for the inverse. The stage with m groups uses tw[m + i] for
 // group i; in the block phase the global group index is b m_loc + i_loc and
 // m = N1 m_loc, so the index is m_loc (N1 + b) + i_loc.
@@ -46,28 +56,6 @@
 namespace ckks {
 
 // ---------------------------------------------------------------------------
-// butterflies
-// ---------------------------------------------------------------------------
-template <bool Q1>
-__device__ __forceinline__ void ct_bfly(u64 &X, u64 &Y, ulonglong2 w, u64 q) {
-    u64 q2 = q << 1;
-    u64 x = X >= q2 ? X - q2 : X;
-    u64 t = shoup_lazy_t<Q1>(Y, w.x, w.y, q);
-    X = x + t;
-    Y = x - t + q2;
-}
-
-template <bool Q1>
-__device__ __forceinline__ void gs_bfly(u64 &X, u64 &Y, ulonglong2 w, u64 q) {
-    u64 q2 = q << 1;
-    u64 s = X + Y;
-    s = s >= q2 ? s - q2 : s;
-    u64 d = X - Y + q2;
-    Y = shoup_lazy_t<Q1>(d, w.x, w.y, q);
-    X = s;
-}
-
-// ---------------------------------------------------------------------------
 // pass plan: LOGN stages in ceil(LOGN/4) passes of near-equal length
 // ---------------------------------------------------------------------------
 #ifndef CKKS_NTT_RMAX
@@ -82,24 +70,16 @@ struct Pass {
     static constexpr int start = P * base + (P < extra ? P : extra);
 };
 
-// Shared-memory layouts of a tile (n_sub = 2^lsub sub-problems of n points).
-//   columns: [n][n_sub] row-major (sub-problems side by side); threads run
-//            over sub-problems fastest, so every pass reads whole 128-byte
-//            row segments of global memory.
-//   blocks:  [n_sub][n + n/16] with one pad word per 16; threads run over
-//            point sets fastest.
-template <bool COLS, int LOGN>
-struct Layout {
-    int lsub;
-    __device__ __forceinline__ int off(int sp, int k) const {
-        if (COLS) return (k << lsub) + sp;
-        return sp * ((1 << LOGN) + (1 << LOGN >> 4)) + k + (k >> 4);
-    }
-    __device__ __forceinline__ void split(int s, int lsets, int &sp, int &set) const {
-        if (COLS) { sp = s & ((1 << lsub) - 1); set = s >> lsub; }
-        else { set = s & ((1 << lsets) - 1); sp = s >> lsets; }
-    }
-};
+// Position of the twiddle of stage e of a pass (E0, R), its sub-problem group
+// g and j < 2^e, within the pass's region of the twiddle table: the 2^R - 1
+// twiddles a point set needs are 2^E0 entries apart, so one base pointer and
+// constant offsets address them, and the threads of neighbouring groups read
+// neighbouring entries (in stage order the same reads were 2^e entries
+// apart: 16 to 32 cache lines per warp load, the L1 data stage 59 % busy in
+// the forward block phase).
+//   columns: region [2^E0, 2^(E0 + R)), entry (2^e - 1 + j) 2^E0 + g
+//   block b: region [N1 2^E0, N1 2^(E0 + R)), entry (b (2^R - 1) + 2^e - 1 + j) 2^E0 + g
+// (twiddle_slot in ntt.cu fills the table.)
 
 // ---------------------------------------------------------------------------
 // fused element-wise load / store with per-CTA base pointers
@@ -198,7 +178,18 @@ __device__ __forceinline__ StoreCtx make_store(const StoreSpec &S, const NttJob 
     return c;
 }
 
-template <int LM, bool Q1>
+// a + b of an Eq. 17 sum: lazy signed for small primes (at most 64 terms
+// below q each), canonical for the others
+template <bool SMALL>
+__device__ __forceinline__ u64 eq17_add(u64 s, u64 r, u64 q) {
+    return SMALL ? s + r : add_mod(s, lift_sign(r, q), q);
+}
+template <bool SMALL>
+__device__ __forceinline__ u64 eq17_sub(u64 r, u64 s, u64 q) {
+    return SMALL ? r - s : sub_mod(lift_sign(r, q), s, q);
+}
+
+template <int LM, bool SMALL, bool Q1>
 __device__ __forceinline__ u64 load_elem(const LoadCtx &c, int e) {
     const u64 q = c.m.q;
     const int mode = LM >= 0 ? LM : c.mode;
@@ -209,8 +200,8 @@ __device__ __forceinline__ u64 load_elem(const LoadCtx &c, int e) {
         // sum_t g_t T_t (mod q); with the self term: g_self a - sum
         u64 s = 0;
         for (int t = 0; t < c.mu; ++t)
-            s = add_mod(s, shoup_t<Q1>(c.b[(i64)t * c.N + e], c.g[t].w, c.g[t].wp, q), q);
-        if (c.with_self) s = sub_mod(shoup_t<Q1>(c.a[e], c.g[c.mu].w, c.g[c.mu].wp, q), s, q);
+            s = eq17_add<SMALL>(s, shoup_signed<Q1>(c.b[(i64)t * c.N + e], c.g[t].w, c.g[t].wp, q), q);
+        if (c.with_self) s = eq17_sub<SMALL>(shoup_signed<Q1>(c.a[e], c.g[c.mu].w, c.g[c.mu].wp, q), s, q);
         return s;
     }
     case LD_BCONVK: {
@@ -224,13 +215,13 @@ __device__ __forceinline__ u64 load_elem(const LoadCtx &c, int e) {
     }
 }
 
-template <int SM, bool Q1>
+template <int SM, bool SMALL, bool Q1>
 __device__ __forceinline__ void store_elem(const StoreCtx &c, int e, u64 v, bool fwd) {
     const u64 q = c.m.q;
     const int mode = SM >= 0 ? SM : c.mode;
     switch (mode) {
     case ST_LAZY:
-        c.dst[e] = v;
+        c.dst[e] = !SMALL && fwd ? canonical<SMALL>(v, q, c.m.canon) : v;
         break;
     case ST_SCALE:
         c.dst[e] = shoup_t<Q1>(v, c.c.w, c.c.wp, q);
@@ -246,292 +237,369 @@ __device__ __forceinline__ void store_elem(const StoreCtx &c, int e, u64 v, bool
     }
     case ST_MRS:
         // Algorithm 1, last step: A' = g^{mu,L-1} A - B
-        c.dst[e] = sub_mod(shoup_t<Q1>(c.aux[e], c.c.w, c.c.wp, q), fwd ? reduce4(v, q) : reduce2(v, q), q);
+        c.dst[e] = sub_mod(shoup_t<Q1>(c.aux[e], c.c.w, c.c.wp, q), canonical<SMALL>(v, q, c.m.canon), q);
         break;
     case ST_ADDSUB:
-        c.dst[e] = sub_mod(add_mod(c.aux[e], c.aux2[e], q), fwd ? reduce4(v, q) : reduce2(v, q), q);
+        c.dst[e] = sub_mod(add_mod(c.aux[e], c.aux2[e], q), canonical<SMALL>(v, q, c.m.canon), q);
         break;
     default:  // ST_REDUCE
-        c.dst[e] = fwd ? reduce4(v, q) : reduce2(v, q);
+        c.dst[e] = canonical<SMALL>(v, q, c.m.canon);
         break;
     }
 }
 
-// Fused loads / stores that sum over several limbs (the Eq. 17 load, the
-// ModDown store) issue the loads of several elements together.
-#ifndef CKKS_NTT_EQ17_BY_TERM
-#define CKKS_NTT_EQ17_BY_TERM 1
-#endif
-#ifndef CKKS_NTT_MODDOWN_GROUPS
-#define CKKS_NTT_MODDOWN_GROUPS 1
-#endif
+// ---------------------------------------------------------------------------
+// one pass of a phase
+// ---------------------------------------------------------------------------
+// Threads. Every thread takes 16 points of a sub-problem (n >= 16):
+//   columns: groups of 16 columns x n / 16 point sets, 16 adjacent columns
+//            fastest, so every access to global memory is whole 128-byte row
+//            segments; the tile is [n][16] per group; passes are separated by
+//            __syncthreads;
+//   blocks:  n / 16 threads per block, all in one warp, so passes are
+//            separated by __syncwarp and warps never wait for each other; the
+//            tile is [n + n / 16] per block (one pad word per 16).
+// The geometry is fixed at compile time: every address within a thread's
+// point set is one base plus constant offsets.
+//   whole:   N <= 2^12 takes one launch for all stages: one CTA of n / 16
+//            threads holds a limb (N >= 2^9), or a warp holds one or more
+//            (a block phase with N1 = 1).
+enum Shape { COLS = 0, BLOCKS = 1, WHOLE = 2 };
+constexpr int kWholeMax = 12;  // log2 of the largest limb one CTA transforms
 
-// One pass of R stages starting at local stage E0 on every point set of the
-// tile. GIN / GOUT: the pass reads / writes global memory (fused load /
-// store) instead of shared memory.
-template <int LOGN, int R, int E0, bool FWD, bool COLS, bool GIN, bool GOUT, int LM, int SM, bool Q1>
-__device__ __forceinline__ void run_pass(u64 *sm, const Layout<COLS, LOGN> &lay, const ulonglong2 *tw, int tw_b0,
-                                         int tw_bmul, u64 q, const LoadCtx &lc, const StoreCtx &sc, int t0,
-                                         int log_n2) {
-    constexpr int n = 1 << LOGN;
-    constexpr int EL = 1 << R;
-    constexpr int t_min = n >> (E0 + R);
-    constexpr int t0s = n >> (E0 + 1);
-    constexpr int lsets = LOGN - R;
-    const int total = 1 << (lay.lsub + lsets);
-    for (int s = threadIdx.x; s < total; s += blockDim.x) {
-        int sp, set;
-        lay.split(s, lsets, sp, set);
-        const int o = set & (t_min - 1);
-        const int g = set / t_min;
-        const int base = g * 2 * t0s + o;
-        u64 x[EL];
-        if constexpr (CKKS_NTT_EQ17_BY_TERM && GIN && LM == LD_EQ17) {
-            // Eq. 17 combination term by term: the EL loads of one term are
-            // in flight together (the per-element loop over the terms had
-            // one load in flight per thread)
-            const u64 q = lc.m.q;
-#pragma unroll
-            for (int k = 0; k < EL; ++k) x[k] = 0;
-            for (int t = 0; t < lc.mu; ++t) {
-                const Shoup g = lc.g[t];
-                const u64 *bt = lc.b + (i64)t * lc.N;
-#pragma unroll
-                for (int k = 0; k < EL; ++k) {
-                    const int pt = base + k * t_min;
-                    const int e = COLS ? t0 + sp + (pt << log_n2) : ((t0 + sp) << LOGN) + pt;
-                    x[k] = add_mod(x[k], shoup_t<Q1>(bt[e], g.w, g.wp, q), q);
-                }
-            }
-            if (lc.with_self) {
-                const Shoup g = lc.g[lc.mu];
-#pragma unroll
-                for (int k = 0; k < EL; ++k) {
-                    const int pt = base + k * t_min;
-                    const int e = COLS ? t0 + sp + (pt << log_n2) : ((t0 + sp) << LOGN) + pt;
-                    x[k] = sub_mod(shoup_t<Q1>(lc.a[e], g.w, g.wp, q), x[k], q);
-                }
-            }
-        } else {
-#pragma unroll
-            for (int k = 0; k < EL; ++k) {
-                const int pt = base + k * t_min;
-                if (GIN) {
-                    const int e = COLS ? t0 + sp + (pt << log_n2) : ((t0 + sp) << LOGN) + pt;
-                    x[k] = load_elem<LM, Q1>(lc, e);
-                } else {
-                    x[k] = sm[lay.off(sp, pt)];
-                }
-            }
-        }
-        const int twb = tw_b0 + tw_bmul * sp;
-        if (FWD) {
-#pragma unroll
-            for (int ep = 0; ep < R; ++ep) {
-                const int h = EL >> (ep + 1);
-                const int m = 1 << (E0 + ep);
-#pragma unroll
-                for (int k = 0; k < EL; ++k) {
-                    if ((k & h) == 0) {
-                        const int i = (g << ep) + (k >> (R - ep));
-                        ct_bfly<Q1>(x[k], x[k + h], tw[m * twb + i], q);
-                    }
-                }
-            }
-        } else {
-#pragma unroll
-            for (int ep = R - 1; ep >= 0; --ep) {
-                const int h = EL >> (ep + 1);
-                const int m = 1 << (E0 + ep);
-#pragma unroll
-                for (int k = 0; k < EL; ++k) {
-                    if ((k & h) == 0) {
-                        const int i = (g << ep) + (k >> (R - ep));
-                        gs_bfly<Q1>(x[k], x[k + h], tw[m * twb + i], q);
-                    }
-                }
-            }
-        }
-        if constexpr (CKKS_NTT_MODDOWN_GROUPS && GOUT && SM == ST_MODDOWN) {
-            // ModDown store (Eq. 5 with Eq. 11 / 12) four elements at a time,
-            // their K z-limb loads in flight together
-            const u64 q = sc.m.q;
-            constexpr int G4 = EL >= 4 ? 4 : EL;
-#pragma unroll
-            for (int k0 = 0; k0 < EL; k0 += G4) {
-                int e[G4];
-                Acc128Lazy acc[G4];  // sum of the P primes < 2^64 (context check)
-#pragma unroll
-                for (int u = 0; u < G4; ++u) {
-                    const int pt = base + (k0 + u) * t_min;
-                    e[u] = COLS ? t0 + sp + (pt << log_n2) : ((t0 + sp) << LOGN) + pt;
-                    acc[u].zero();
-                }
-                for (int i = 0; i < sc.K; ++i) {
-                    const u64 c = sc.cK[i];
-                    const u64 *zi = sc.aux + (i64)i * sc.N;
-                    u64 z[G4];
-#pragma unroll
-                    for (int u = 0; u < G4; ++u) z[u] = zi[e[u]];
-#pragma unroll
-                    for (int u = 0; u < G4; ++u) acc[u].mac(z[u], c);
-                }
-#pragma unroll
-                for (int u = 0; u < G4; ++u)
-                    sc.dst[e[u]] = sub_mod(shoup_t<Q1>(x[k0 + u], sc.c.w, sc.c.wp, q),
-                                           redc_t<Q1>(acc[u].hi, acc[u].lo, sc.m), q);
-            }
-        } else {
-#pragma unroll
-            for (int k = 0; k < EL; ++k) {
-                const int pt = base + k * t_min;
-                if (GOUT) {
-                    const int e = COLS ? t0 + sp + (pt << log_n2) : ((t0 + sp) << LOGN) + pt;
-                    store_elem<SM, Q1>(sc, e, x[k], FWD);
-                } else {
-                    sm[lay.off(sp, pt)] = x[k];
-                }
-            }
-        }
-    }
-}
-
-// Direct global access is used on a side whose pass reads / writes at
-// least 8 consecutive words per sub-problem (always true for column tiles).
-// CKKS_NTT_DIRECT_IN = 0 stages every tile through shared memory on the
-// load side (batched loads), keeping direct global stores.
-#ifndef CKKS_NTT_DIRECT_IN
-#define CKKS_NTT_DIRECT_IN 1
-#endif
-template <int LOGN, bool COLS, int P>
-struct PassAccess {
-    static constexpr int t_min = (1 << LOGN) >> (Pass<LOGN, P>::start + Pass<LOGN, P>::len);
-    static constexpr bool direct = COLS || t_min >= 8;
-    static constexpr bool direct_in = direct && CKKS_NTT_DIRECT_IN;
+template <int LOGN, int LOGN2, int SH>
+struct Geo {
+    static constexpr int n = 1 << LOGN;
+    static constexpr int sets = n >= 16 ? n / 16 : 1;               // threads per sub-problem
+    static constexpr int group = SH == COLS ? 16 * sets : sets;     // threads per tile unit (16 columns / one block)
+    static constexpr int unit = SH == COLS ? 16 * n : n + n / 16;   // shared words per tile unit
+    static constexpr int stride = SH == COLS ? 1 << LOGN2 : 1;      // elements between neighbouring points in memory
+    static constexpr int warp_blocks = SH == BLOCKS ? 32 / sets : 1;  // blocks per warp (whole: the limb)
+    // bytes of a warp's part of a block-phase CTA: its blocks, then their n - 1 twiddles each
+    static constexpr int warp_data = warp_blocks * unit;    // words (even)
+    static constexpr int warp_bytes = warp_data * 8 + warp_blocks * (n - 1) * 16;
+    // shared offset of point pt relative to the thread's sub-problem; additive
+    // over disjoint bit ranges of pt
+    static __device__ __forceinline__ constexpr int off(int pt) { return SH == COLS ? pt * 16 : pt + (pt >> 4); }
 };
 
-template <int LOGN, bool FWD, bool COLS, int LM, int SM, bool Q1, int I>
-__device__ __forceinline__ void run_passes(u64 *sm, const Layout<COLS, LOGN> &lay, const ulonglong2 *tw, int tw_b0,
-                                           int tw_bmul, u64 q, const LoadCtx &lc, const StoreCtx &sc, int t0,
-                                           int log_n2) {
-    constexpr int NP = Pass<LOGN, 0>::NP;
-    if constexpr (I < NP) {
-        constexpr int PP = FWD ? I : NP - 1 - I;
-        constexpr bool first = I == 0, last = I == NP - 1;
-        constexpr bool gin = first && PassAccess<LOGN, COLS, PP>::direct_in;
-        constexpr bool gout = last && PassAccess<LOGN, COLS, PP>::direct;
-        run_pass<LOGN, Pass<LOGN, PP>::len, Pass<LOGN, PP>::start, FWD, COLS, gin, gout, LM, SM, Q1>(
-            sm, lay, tw, tw_b0, tw_bmul, q, lc, sc, t0, log_n2);
-        if (!last || !gout) __syncthreads();
-        run_passes<LOGN, FWD, COLS, LM, SM, Q1, I + 1>(sm, lay, tw, tw_b0, tw_bmul, q, lc, sc, t0, log_n2);
-    }
+// Asynchronous 16-byte copy into shared memory (no registers held while the
+// load is in flight); groups complete in the order they were committed.
+__device__ __forceinline__ void async_copy16(void *dst, const void *src) {
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"((u32)__cvta_generic_to_shared(dst)), "l"(src)
+                 : "memory");
+}
+__device__ __forceinline__ void async_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
+template <int PENDING>
+__device__ __forceinline__ void async_wait() {
+    asm volatile("cp.async.wait_group %0;" ::"n"(PENDING) : "memory");
 }
 
-// 1: the column phases read their twiddles (the same n - 1 for every
-// column) from a copy in shared memory, 4 KB behind the tile: forward column
-// phase 55.0 vs 60.1 ms per bench step with them read from L1 / L2
-#ifndef CKKS_NTT_COL_TW_SMEM
-#define CKKS_NTT_COL_TW_SMEM 1
-#endif
+template <int SH>
+__device__ __forceinline__ void pass_sync() {
+    if (SH == BLOCKS) __syncwarp();
+    else __syncthreads();
+}
 
-// Staged stores that read an aux limb gather eight elements at a time.
-#ifndef CKKS_NTT_STORE_BATCH
-#define CKKS_NTT_STORE_BATCH 1
-#endif
+// Whether a pass reads / writes global memory itself: always for columns, for
+// blocks where it touches at least 8 consecutive words per sub-problem (the
+// other side is staged through shared memory by the warp).
+template <int LOGN, int SH, int P>
+struct PassAccess {
+    static constexpr int t_min = (1 << LOGN) >> (Pass<LOGN, P>::start + Pass<LOGN, P>::len);
+    static constexpr bool direct = SH == COLS || t_min >= 8;
+};
 
-// One tile (CTA) of one limb: tile index `tile` of the phase.
-template <int LOGN, bool FWD, bool COLS, int LM, int SM, bool Q1>
-__device__ __forceinline__ void phase_tile(u64 *sm, const NttPhase &P, const ulonglong2 *tw, u64 q,
-                                           const LoadCtx &lc, const StoreCtx &sc, int tile) {
-    constexpr int n = 1 << LOGN;
-    constexpr int NP = Pass<LOGN, 0>::NP;
-    const int lsub = P.log_sub;
-    const int n_sub = 1 << lsub;
-    Layout<COLS, LOGN> lay{lsub};
-    const int t0 = tile << lsub;  // first column (COLS) or block (!COLS)
-    constexpr int PF = FWD ? 0 : NP - 1;
-    constexpr int PL = FWD ? NP - 1 : 0;
-    constexpr bool gin = PassAccess<LOGN, COLS, PF>::direct_in;
-    constexpr bool gout = PassAccess<LOGN, COLS, PL>::direct;
-    const int total = n_sub << LOGN;
-    // twiddle base: columns -> 1; blocks -> N1 + block
-    const int tw_b0 = COLS ? 1 : P.N1 + t0;
-    const int tw_bmul = COLS ? 0 : 1;
-    if constexpr (COLS && CKKS_NTT_COL_TW_SMEM) {
-        // the column phase's n - 1 twiddles (the same for every column) copied
-        // once per CTA into shared memory behind the tile
-        ulonglong2 *tws = reinterpret_cast<ulonglong2 *>(sm + total);
-        for (int i = threadIdx.x; i < n; i += blockDim.x) tws[i] = tw[i];
-        __syncthreads();
-        tw = tws;
+// R stages of butterflies on the 2^R points of one set; tw: the set's first
+// twiddle, entries 2^E0 apart.
+template <int R, int E0, bool FWD, bool SMALL, bool Q1, bool LONG>
+__device__ __forceinline__ void set_stages(u64 (&x)[1 << R], const ulonglong2 *tw, u64 q) {
+    constexpr int EL = 1 << R;
+    if (FWD && !SMALL && LONG && E0 > 0 && !(q >> 60)) {
+        // more than 8 stages in one phase: |x| < 8 q at every pass's end, so
+        // folded to 4 q here the next pass ends below 8 q again
+#pragma unroll
+        for (int k = 0; k < EL; ++k) x[k] = fold_sign(x[k], q << 2);
     }
-    if (!gin) {
-        // coalesced global -> shared with the fused load, eight loads in
-        // flight per thread before their shared-memory stores
-        constexpr int U = 8;
-        for (int base = threadIdx.x; base < total; base += U * blockDim.x) {
-            u64 v[U];
 #pragma unroll
-            for (int u = 0; u < U; ++u) {
-                const int idx = base + u * blockDim.x;
-                if (idx < total) {
-                    int sp, k, e;
-                    if (COLS) { k = idx >> lsub; sp = idx & (n_sub - 1); e = t0 + sp + (k << P.log_n2); }
-                    else { sp = idx >> LOGN; k = idx & (n - 1); e = ((t0 + sp) << LOGN) + k; }
-                    v[u] = load_elem<LM, Q1>(lc, e);
-                }
-            }
+    for (int st = 0; st < R; ++st) {
+        const int ep = FWD ? st : R - 1 - st;
+        const int h = EL >> (ep + 1);
+        if (FWD && !SMALL && ep % 2 == 0 && (q >> 60)) {
+            // |x| < 4 q: two more stages after the fold stay below 4 q < 2^63
 #pragma unroll
-            for (int u = 0; u < U; ++u) {
-                const int idx = base + u * blockDim.x;
-                if (idx < total) {
-                    int sp, k;
-                    if (COLS) { k = idx >> lsub; sp = idx & (n_sub - 1); }
-                    else { sp = idx >> LOGN; k = idx & (n - 1); }
-                    sm[lay.off(sp, k)] = v[u];
+            for (int k = 0; k < EL; ++k)
+                if ((k & h) == 0) x[k] = fold_sign(x[k], q << 1);
+        }
+#pragma unroll
+        for (int k = 0; k < EL; ++k) {
+            if ((k & h) == 0) {
+                const ulonglong2 w = tw[((1 << ep) - 1 + (k >> (R - ep))) << E0];
+                if (FWD) {
+                    ct_bfly<SMALL, Q1>(x[k], x[k + h], w.x, w.y, q);
+                } else {
+                    gs_bfly<SMALL, Q1>(x[k], x[k + h], w.x, w.y, q);
+                    if (!SMALL) x[k] = fold_sign(x[k], q);
                 }
             }
         }
-        __syncthreads();
     }
-    run_passes<LOGN, FWD, COLS, LM, SM, Q1, 0>(sm, lay, tw, tw_b0, tw_bmul, q, lc, sc, t0, P.log_n2);
-    if (!gout) {
-        // shared -> global with the fused store (coalesced)
-        if constexpr (CKKS_NTT_STORE_BATCH && (SM == ST_MRS || SM == ST_ADDSUB)) {
-            // the store reads an aux limb: gather eight elements and their
-            // aux words first, so that eight loads are in flight per thread
-            constexpr int U = 8;
-            for (int base = threadIdx.x; base < total; base += U * blockDim.x) {
-                u64 v[U], a[U], a2[U];
-                int e[U];
+}
+
+// Loads of one point set from global memory: elements e + k dist, fused. The
+// loads of all points are in flight together (for Eq. 17 term by term: a
+// loop over the terms inside each element's load had one load in flight).
+template <int EL, int DIST, int LM, bool SMALL, bool Q1>
+__device__ __forceinline__ void load_set(u64 (&x)[EL], const LoadCtx &lc, int e) {
+    if constexpr (LM == LD_EQ17) {
+        const u64 q = lc.m.q;
 #pragma unroll
-                for (int u = 0; u < U; ++u) {
-                    const int idx = base + u * blockDim.x;
-                    e[u] = -1;
-                    if (idx < total) {
-                        int sp, k;
-                        if (COLS) { k = idx >> lsub; sp = idx & (n_sub - 1); e[u] = t0 + sp + (k << P.log_n2); }
-                        else { sp = idx >> LOGN; k = idx & (n - 1); e[u] = ((t0 + sp) << LOGN) + k; }
-                        v[u] = sm[lay.off(sp, k)];
-                        a[u] = sc.aux[e[u]];
-                        if (SM == ST_ADDSUB) a2[u] = sc.aux2[e[u]];
-                    }
-                }
+        for (int k = 0; k < EL; ++k) x[k] = 0;
+        for (int t = 0; t < lc.mu; ++t) {
+            const Shoup g = lc.g[t];
+            const u64 *bt = lc.b + (i64)t * lc.N + e;
 #pragma unroll
-                for (int u = 0; u < U; ++u) {
-                    if (e[u] < 0) continue;
-                    const u64 q = sc.m.q;
-                    const u64 r = FWD ? reduce4(v[u], q) : reduce2(v[u], q);
-                    if (SM == ST_MRS) sc.dst[e[u]] = sub_mod(shoup_t<Q1>(a[u], sc.c.w, sc.c.wp, q), r, q);
-                    else sc.dst[e[u]] = sub_mod(add_mod(a[u], a2[u], q), r, q);
+            for (int k = 0; k < EL; ++k)
+                x[k] = eq17_add<SMALL>(x[k], shoup_signed<Q1>(bt[k * DIST], g.w, g.wp, q), q);
+        }
+        if (lc.with_self) {
+            const Shoup g = lc.g[lc.mu];
+#pragma unroll
+            for (int k = 0; k < EL; ++k)
+                x[k] = eq17_sub<SMALL>(shoup_signed<Q1>(lc.a[e + k * DIST], g.w, g.wp, q), x[k], q);
+        }
+    } else {
+#pragma unroll
+        for (int k = 0; k < EL; ++k) x[k] = load_elem<LM, SMALL, Q1>(lc, e + k * DIST);
+    }
+}
+
+// Stores of one point set; the ModDown store takes four elements at a time,
+// their K z-limb loads in flight together.
+template <int EL, int DIST, int SM, bool FWD, bool SMALL, bool Q1>
+__device__ __forceinline__ void store_set(const u64 (&x)[EL], const StoreCtx &sc, int e) {
+    if constexpr (SM == ST_MODDOWN) {
+        const u64 q = sc.m.q;
+        constexpr int G4 = EL >= 4 ? 4 : EL;
+#pragma unroll
+        for (int k0 = 0; k0 < EL; k0 += G4) {
+            Acc128Lazy acc[G4];  // sum of the P primes < 2^64 (context check)
+#pragma unroll
+            for (int u = 0; u < G4; ++u) acc[u].zero();
+            for (int i = 0; i < sc.K; ++i) {
+                const u64 c = sc.cK[i];
+                const u64 *zi = sc.aux + (i64)i * sc.N + e;
+                u64 z[G4];
+#pragma unroll
+                for (int u = 0; u < G4; ++u) z[u] = zi[(k0 + u) * DIST];
+#pragma unroll
+                for (int u = 0; u < G4; ++u) acc[u].mac(z[u], c);
+            }
+#pragma unroll
+            for (int u = 0; u < G4; ++u)
+                sc.dst[e + (k0 + u) * DIST] = sub_mod(shoup_t<Q1>(x[k0 + u], sc.c.w, sc.c.wp, q),
+                                                      redc_t<Q1>(acc[u].hi, acc[u].lo, sc.m), q);
+        }
+    } else {
+#pragma unroll
+        for (int k = 0; k < EL; ++k) store_elem<SM, SMALL, Q1>(sc, e + k * DIST, x[k], FWD);
+    }
+}
+
+// Per-thread position in a phase: sub-problem and point-set lane.
+struct Lane {
+    u64 *sm;                 // the sub-problem's shared words (column: its column's)
+    const ulonglong2 *tw;    // the sub-problem's twiddles (columns: the shared copy)
+    int e;                   // element index of point 0
+    int set;                 // point set of the first iteration
+    int blk;                 // block within the warp (blocks only, else 0)
+    bool active;
+};
+
+template <int LOGN, int LOGN2, bool FWD, int SH, int LM, int SM, bool SMALL, bool Q1, int I>
+__device__ __forceinline__ void run_passes(const Lane &ln, u64 q, const LoadCtx &lc, const StoreCtx &sc, int N1) {
+    constexpr int NP = Pass<LOGN, 0>::NP;
+    if constexpr (I < NP) {
+        typedef Geo<LOGN, LOGN2, SH> G;
+        constexpr int P = FWD ? I : NP - 1 - I;
+        constexpr int R = Pass<LOGN, P>::len, E0 = Pass<LOGN, P>::start, EL = 1 << R;
+        constexpr bool first = I == 0, last = I == NP - 1;
+        constexpr bool gin = first && PassAccess<LOGN, SH, P>::direct;
+        constexpr bool gout = last && PassAccess<LOGN, SH, P>::direct;
+        constexpr int t_min = G::n >> (E0 + R);
+        constexpr int iters = (G::n >> R) / G::sets;
+        u64 x[iters][EL];
+        if constexpr (gin) {
+            if (ln.active) {
+#pragma unroll
+                for (int it = 0; it < iters; ++it) {
+                    const int set = ln.set + it * G::sets;
+                    const int base = (set / t_min) * (G::n >> E0) + (set & (t_min - 1));
+                    load_set<EL, t_min * G::stride, LM, SMALL, Q1>(x[it], lc, ln.e + base * G::stride);
                 }
             }
-        } else {
-            for (int idx = threadIdx.x; idx < total; idx += blockDim.x) {
-                int sp, k, e;
-                if (COLS) { k = idx >> lsub; sp = idx & (n_sub - 1); e = t0 + sp + (k << P.log_n2); }
-                else { sp = idx >> LOGN; k = idx & (n - 1); e = ((t0 + sp) << LOGN) + k; }
-                store_elem<SM, Q1>(sc, e, sm[lay.off(sp, k)], FWD);
+        }
+        // The data the previous pass exchanged is in place, and so are the
+        // twiddles: of all columns (copied by the CTA; their copy was issued
+        // before the loads above), or of this pass for the warp's blocks (the
+        // I-th of NP groups).
+        if constexpr (SH != COLS) async_wait<NP - 1 - I>();
+        pass_sync<SH>();
+        if (ln.active) {
+#pragma unroll
+            for (int it = 0; it < iters; ++it) {
+                const int set = ln.set + it * G::sets;
+                const int o = set & (t_min - 1), g = set / t_min;
+                const int base = g * (G::n >> E0) + o;
+                // columns: entry 0 unused; blocks: the warp's copy, passes in order of their stages
+                const ulonglong2 *tw = ln.tw + (SH == COLS ? 1 << E0 : G::warp_blocks * ((1 << E0) - 1)) +
+                                       ((ln.blk * (EL - 1)) << E0) + g;
+                u64 *s = ln.sm + G::off(base);
+                if constexpr (!gin) {
+#pragma unroll
+                    for (int k = 0; k < EL; ++k) x[it][k] = s[G::off(k * t_min)];
+                }
+                set_stages<R, E0, FWD, SMALL, Q1, (LOGN > 8)>(x[it], tw, q);
+                // inverse: the output that is a sum at every stage (below
+                // 288 q) -> [0, 2q); a store that multiplies takes it as it is
+                if constexpr (!FWD && SMALL && !(gout && (SM == ST_SCALE || SM == ST_MODDOWN)))
+                    x[it][0] = reduce_far(x[it][0] + (q << 9), q, lc.m.canon);
+                if constexpr (gout) {
+                    store_set<EL, t_min * G::stride, SM, FWD, SMALL, Q1>(x[it], sc, ln.e + base * G::stride);
+                } else {
+#pragma unroll
+                    for (int k = 0; k < EL; ++k) s[G::off(k * t_min)] = x[it][k];
+                }
+            }
+        }
+        if constexpr (!gout && last) pass_sync<SH>();
+        run_passes<LOGN, LOGN2, FWD, SH, LM, SM, SMALL, Q1, I + 1>(ln, q, lc, sc, N1);
+    }
+}
+
+// The twiddles of a warp's blocks, one commit group per pass in execution
+// order: copied asynchronously while the data is loaded, so a warp waits for
+// memory once instead of at every stage. (Read from L2 where they are used, the
+// forward block phase had 6.4 of 12 stall cycles per issue on them.)
+// The lanes (a warp's, or the CTA's for a whole limb) share the copies.
+template <int LOGN, int LOGN2, bool FWD, int SH, int I>
+__device__ __forceinline__ void copy_twiddles(ulonglong2 *dst, const ulonglong2 *tw, int N1, int b0, int lane) {
+    constexpr int NP = Pass<LOGN, 0>::NP;
+    if constexpr (I < NP) {
+        typedef Geo<LOGN, LOGN2, SH> G;
+        constexpr int T = SH == WHOLE ? G::sets : 32;
+        constexpr int P = FWD ? I : NP - 1 - I;
+        constexpr int R = Pass<LOGN, P>::len, E0 = Pass<LOGN, P>::start;
+        constexpr int per = ((1 << R) - 1) << E0;  // entries per block
+        ulonglong2 *d = dst + G::warp_blocks * ((1 << E0) - 1);
+        const ulonglong2 *s = tw + ((i64)N1 << E0) + (i64)b0 * per;
+        const int count = (N1 - b0 < G::warp_blocks ? N1 - b0 : G::warp_blocks) * per;
+#pragma unroll
+        for (int i = 0; i < (G::warp_blocks * per + T - 1) / T; ++i) {
+            const int k = i * T + lane;
+            if (k < count) async_copy16(d + k, s + k);
+        }
+        async_commit();
+        copy_twiddles<LOGN, LOGN2, FWD, SH, I + 1>(dst, tw, N1, b0, lane);
+    }
+}
+
+// One tile (CTA) of one limb: tile index `tile` of the phase.
+template <int LOGN, int LOGN2, bool FWD, int SH, int LM, int SM, bool SMALL, bool Q1>
+__device__ __forceinline__ void phase_tile(u64 *sm, const NttPhase &P, const ulonglong2 *tw, u64 q,
+                                           const LoadCtx &lc, const StoreCtx &sc, int tile) {
+    typedef Geo<LOGN, LOGN2, SH> G;
+    constexpr int n = G::n, NP = Pass<LOGN, 0>::NP;
+    const int tid = threadIdx.x;
+    Lane ln;
+    if constexpr (SH == COLS) {
+        const int groups = blockDim.x / G::group;
+        const int grp = tid / G::group;
+        ulonglong2 *tws = reinterpret_cast<ulonglong2 *>(sm + groups * G::unit);
+        ln.sm = sm + grp * G::unit + (tid & 15);
+        ln.tw = tws;
+        ln.e = (tile * groups + grp) * 16 + (tid & 15);
+        ln.set = (tid / 16) % G::sets;
+        ln.blk = 0;
+        ln.active = true;
+        // the n - 1 twiddles every column shares, copied while the first
+        // pass's loads are in flight
+        for (int i = tid; i < n; i += blockDim.x) tws[i] = tw[i];
+        run_passes<LOGN, LOGN2, FWD, SH, LM, SM, SMALL, Q1, 0>(ln, q, lc, sc, P.N1);
+    } else {
+        // a warp and its blocks, or the CTA and its limb
+        constexpr int BW = G::warp_blocks;
+        constexpr int T = SH == WHOLE ? G::sets : 32;
+        constexpr int W = BW * n / T;                     // words per lane
+        constexpr int U = W < 8 ? W : 8;
+        constexpr int PF = FWD ? 0 : NP - 1, PL = FWD ? NP - 1 : 0;
+        // with LOGN2 = 0 the launch may have fewer blocks than a warp takes
+        constexpr bool FULL = LOGN2 != 0 || SH == WHOLE;
+        const int lane = SH == WHOLE ? tid : tid & 31;
+        const int b0 = SH == WHOLE ? 0 : tile * (blockDim.x / G::sets) + (tid / 32) * BW;  // first block in the limb
+        u64 *wsm = SH == WHOLE ? sm : reinterpret_cast<u64 *>(reinterpret_cast<char *>(sm) + (tid / 32) * G::warp_bytes);
+        ulonglong2 *wtw = reinterpret_cast<ulonglong2 *>(wsm + G::warp_data);
+        ln.blk = SH == WHOLE ? 0 : lane / G::sets;
+        ln.sm = wsm + ln.blk * G::unit;
+        ln.tw = wtw;
+        ln.set = SH == WHOLE ? lane : lane % G::sets;
+        ln.e = (b0 + ln.blk) << LOGN;
+        ln.active = FULL || b0 + ln.blk < P.N1;
+        copy_twiddles<LOGN, LOGN2, FWD, SH, 0>(wtw, tw, P.N1, b0, lane);
+        const int words = (P.N1 - b0) * n;                // words of the limb from the first block on
+        const int e0 = b0 << LOGN;
+        // shared offset of word idx of the warp's blocks
+        auto woff = [](int idx) { return (idx >> LOGN) * G::unit + G::off(idx & (n - 1)); };
+        if constexpr (!PassAccess<LOGN, SH, PF>::direct) {
+            // coalesced global -> shared with the fused load, U loads in flight
+#pragma unroll
+            for (int i0 = 0; i0 < W; i0 += U) {
+                u64 v[U];
+#pragma unroll
+                for (int u = 0; u < U; ++u) {
+                    const int idx = lane + T * (i0 + u);
+                    if (FULL || idx < words) v[u] = load_elem<LM, SMALL, Q1>(lc, e0 + idx);
+                }
+#pragma unroll
+                for (int u = 0; u < U; ++u) {
+                    const int idx = lane + T * (i0 + u);
+                    if (FULL || idx < words) wsm[woff(idx)] = v[u];
+                }
+            }
+        }
+        run_passes<LOGN, LOGN2, FWD, SH, LM, SM, SMALL, Q1, 0>(ln, q, lc, sc, P.N1);
+        if constexpr (!PassAccess<LOGN, SH, PL>::direct) {
+            // shared -> global with the fused store (coalesced); a store that
+            // reads an aux limb gathers U elements and their aux words first
+#pragma unroll
+            for (int i0 = 0; i0 < W; i0 += U) {
+                if constexpr (SM == ST_MRS || SM == ST_ADDSUB) {
+                    u64 a[U], a2[U];
+#pragma unroll
+                    for (int u = 0; u < U; ++u) {
+                        const int idx = lane + T * (i0 + u);
+                        if (FULL || idx < words) {
+                            a[u] = sc.aux[e0 + idx];
+                            if (SM == ST_ADDSUB) a2[u] = sc.aux2[e0 + idx];
+                        }
+                    }
+#pragma unroll
+                    for (int u = 0; u < U; ++u) {
+                        const int idx = lane + T * (i0 + u);
+                        if (FULL || idx < words) {
+                            const u64 r = canonical<SMALL>(wsm[woff(idx)], q, sc.m.canon);
+                            if (SM == ST_MRS)
+                                sc.dst[e0 + idx] = sub_mod(shoup_t<Q1>(a[u], sc.c.w, sc.c.wp, q), r, q);
+                            else sc.dst[e0 + idx] = sub_mod(add_mod(a[u], a2[u], q), r, q);
+                        }
+                    }
+                } else {
+#pragma unroll
+                    for (int u = 0; u < U; ++u) {
+                        const int idx = lane + T * (i0 + u);
+                        if (FULL || idx < words) store_elem<SM, SMALL, Q1>(sc, e0 + idx, wsm[woff(idx)], FWD);
+                    }
+                }
             }
         }
     }
@@ -541,9 +609,9 @@ __device__ __forceinline__ void phase_tile(u64 *sm, const NttPhase &P, const ulo
 // the phase kernels: grid (tiles, limbs) for uniform launches, one
 // flattened dimension (limb * tiles + tile) for table launches
 // ---------------------------------------------------------------------------
-template <int LOGN, bool FWD, bool COLS, int LM, int SM, int MINB, bool Q1>
+template <int LOGN, int LOGN2, bool FWD, int SH, int LM, int SM, int MINB, bool Q1>
 __global__ void __launch_bounds__(256, MINB) ntt_phase_kernel(NttPhase P, LimbJobs J, LoadSpec L, StoreSpec S) {
-    extern __shared__ u64 sm[];
+    extern __shared__ __align__(16) u64 sm[];
     int b, p, l;
     decode_job(J, blockIdx.y, b, p, l);
     const int prime = J.prime[l];
@@ -551,13 +619,14 @@ __global__ void __launch_bounds__(256, MINB) ntt_phase_kernel(NttPhase P, LimbJo
     const ulonglong2 *tw = (FWD ? P.tw_fwd : P.tw_inv) + (i64)prime * P.N;
     const LoadCtx lc = make_load(L, J, P.N, b, p, l, prime, m);
     const StoreCtx sc = make_store(S, J, P.N, b, p, l, prime, m);
-    phase_tile<LOGN, FWD, COLS, LM, SM, Q1>(sm, P, tw, m.q, lc, sc, blockIdx.x);
+    if (small_prime(m.q)) phase_tile<LOGN, LOGN2, FWD, SH, LM, SM, true, Q1>(sm, P, tw, m.q, lc, sc, blockIdx.x);
+    else phase_tile<LOGN, LOGN2, FWD, SH, LM, SM, false, Q1>(sm, P, tw, m.q, lc, sc, blockIdx.x);
 }
 
-template <int LOGN, bool FWD, bool COLS, int LM, int SM, int MINB, bool Q1>
+template <int LOGN, int LOGN2, bool FWD, int SH, int LM, int SM, int MINB, bool Q1>
 __global__ void __launch_bounds__(256, MINB) ntt_phase_table_kernel(NttPhase P, const NttJob *jobs, int tiles,
                                                                     LoadSpec L, StoreSpec S) {
-    extern __shared__ u64 sm[];
+    extern __shared__ __align__(16) u64 sm[];
     const int job = blockIdx.x / tiles;
     const int tile = blockIdx.x - job * tiles;
     const NttJob j = jobs[job];
@@ -565,27 +634,28 @@ __global__ void __launch_bounds__(256, MINB) ntt_phase_table_kernel(NttPhase P, 
     const ulonglong2 *tw = (FWD ? P.tw_fwd : P.tw_inv) + (i64)j.prime * P.N;
     const LoadCtx lc = make_load(L, j, P.N, m);
     const StoreCtx sc = make_store(S, j, P.N, m);
-    phase_tile<LOGN, FWD, COLS, LM, SM, Q1>(sm, P, tw, m.q, lc, sc, tile);
+    if (small_prime(m.q)) phase_tile<LOGN, LOGN2, FWD, SH, LM, SM, true, Q1>(sm, P, tw, m.q, lc, sc, tile);
+    else phase_tile<LOGN, LOGN2, FWD, SH, LM, SM, false, Q1>(sm, P, tw, m.q, lc, sc, tile);
 }
 
 // ---------------------------------------------------------------------------
 // host-side launch of one instantiation
 // ---------------------------------------------------------------------------
 struct PhaseLaunch {
-    int tiles, threads;
+    int tiles, threads, shape;
     size_t smem;
     cudaStream_t st;
 };
 
-#ifndef CKKS_NTT_MINB
-#define CKKS_NTT_MINB 2         // run-time modes: 128 registers, two CTAs per SM
+// Resident CTAs of 256 threads per SM the kernels are compiled for.
+#ifndef CKKS_NTT_COL_MINB
+#define CKKS_NTT_COL_MINB 4     // columns: 64 registers (871 vs 842 G butterflies/s with three CTAs, 736 with two)
 #endif
-#ifndef CKKS_NTT_FAST_MINB
-#define CKKS_NTT_FAST_MINB 3    // fixed modes: 80 registers, three CTAs per SM
+#ifndef CKKS_NTT_COL_WIDE_MINB
+#define CKKS_NTT_COL_WIDE_MINB 3  // columns whose load or store sums over several limbs: 80 registers
 #endif
-#ifndef CKKS_NTT_EQ17_MINB
-#define CKKS_NTT_EQ17_MINB 3    // the Eq. 17 load spills a little at 80 registers; three CTAs per SM
-                                // still run the phase 9 % faster than two at 128
+#ifndef CKKS_NTT_BLOCK_MINB
+#define CKKS_NTT_BLOCK_MINB 2   // blocks: shared memory holds the twiddles of 16 warps per SM
 #endif
 
 template <typename K>
@@ -594,10 +664,10 @@ static inline cudaError_t allow_smem(K kern, size_t smem) {
     return cudaSuccess;
 }
 
-template <int LOGN, bool FWD, bool COLS, int LM, int SM, int MINB, bool Q1>
+template <int LOGN, int LOGN2, bool FWD, int SH, int LM, int SM, int MINB, bool Q1>
 static inline cudaError_t launch_uniform(const NttPhase &P, const LimbJobs &J, const LoadSpec &L,
                                          const StoreSpec &S, const PhaseLaunch &G) {
-    auto kern = ntt_phase_kernel<LOGN, FWD, COLS, LM, SM, MINB, Q1>;
+    auto kern = ntt_phase_kernel<LOGN, LOGN2, FWD, SH, LM, SM, MINB, Q1>;
     cudaError_t e = allow_smem(kern, G.smem);
     if (e != cudaSuccess) return e;
     dim3 grid(G.tiles, J.n_batch * J.n_polys * J.n_limbs);
@@ -605,10 +675,10 @@ static inline cudaError_t launch_uniform(const NttPhase &P, const LimbJobs &J, c
     return cudaGetLastError();
 }
 
-template <int LOGN, bool FWD, bool COLS, int LM, int SM, int MINB, bool Q1>
+template <int LOGN, int LOGN2, bool FWD, int SH, int LM, int SM, int MINB, bool Q1>
 static inline cudaError_t launch_table(const NttPhase &P, const NttJob *jobs, int n_jobs, const LoadSpec &L,
                                        const StoreSpec &S, const PhaseLaunch &G) {
-    auto kern = ntt_phase_table_kernel<LOGN, FWD, COLS, LM, SM, MINB, Q1>;
+    auto kern = ntt_phase_table_kernel<LOGN, LOGN2, FWD, SH, LM, SM, MINB, Q1>;
     cudaError_t e = allow_smem(kern, G.smem);
     if (e != cudaSuccess) return e;
     const long long blocks = (long long)n_jobs * G.tiles;
@@ -618,107 +688,132 @@ static inline cudaError_t launch_table(const NttPhase &P, const NttJob *jobs, in
     return cudaGetLastError();
 }
 
-// Dispatch of one direction (FWD) and job source (TABLE) over the phase
-// geometry (cols, log2 n) and the modes. dispatch_fast launches the
-// specialised kernel for the mode combinations of the hot path at n = 128 /
-// 256 (N = 2^14 .. 2^16), with the modular products in the form Q1 selects,
-// and sets `found`; dispatch_generic launches the run-time-mode kernel (the
-// general products, valid for every prime).
-#define CKKS_LAUNCH(LG, CO, LMv, SMv, MB, Q)                                                         \
+// Dispatch of one direction (FWD) and job source (TABLE) over the shape, log2
+// n and the modes. Every pair of modes the library uses has its own kernel
+// (a kernel with run-time modes kept every mode's pointers alive and its code
+// did not fit the instruction cache: 12-18 us a launch at N = 2^10 against
+// 5-7): a phase that fuses a mode has the plain mode on its other side.
+//   two phases (N >= 2^13): dispatch_two, with the products in the form Q1
+//   selects (N >= 2^14);
+//   one phase (2^9 <= N <= 2^12): dispatch_whole;
+//   N <= 2^8: dispatch_tiny, run-time modes.
+#define CKKS_LAUNCH(LG, LG2, SHv, LMv, SMv, MB, Q)                                                   \
     do {                                                                                             \
-        if constexpr (TABLE) return launch_table<LG, FWD, CO, LMv, SMv, MB, Q>(P, jobs, n_jobs, L, S, G); \
-        else return launch_uniform<LG, FWD, CO, LMv, SMv, MB, Q>(P, *J, L, S, G);                    \
+        if constexpr (TABLE) return launch_table<LG, LG2, FWD, SHv, LMv, SMv, MB, Q>(P, jobs, n_jobs, L, S, G); \
+        else return launch_uniform<LG, LG2, FWD, SHv, LMv, SMv, MB, Q>(P, *J, L, S, G);              \
     } while (0)
+#define CKKS_MODES(LMv, SMv) if (L.mode == LMv && S.mode == SMv)
+
+template <bool FWD, bool TABLE, bool Q1, int LG, int LG2>
+static inline cudaError_t dispatch_cols(const NttPhase &P, const LimbJobs *J, const NttJob *jobs, int n_jobs,
+                                        const LoadSpec &L, const StoreSpec &S, const PhaseLaunch &G) {
+    if constexpr (FWD) {
+        CKKS_MODES(LD_PLAIN, ST_LAZY) CKKS_LAUNCH(LG, LG2, COLS, LD_PLAIN, ST_LAZY, CKKS_NTT_COL_MINB, Q1);
+        CKKS_MODES(LD_EQ17, ST_LAZY) CKKS_LAUNCH(LG, LG2, COLS, LD_EQ17, ST_LAZY, CKKS_NTT_COL_WIDE_MINB, Q1);
+        CKKS_MODES(LD_BCONVK, ST_LAZY) CKKS_LAUNCH(LG, LG2, COLS, LD_BCONVK, ST_LAZY, CKKS_NTT_COL_WIDE_MINB, Q1);
+    } else {
+        CKKS_MODES(LD_PLAIN, ST_SCALE) CKKS_LAUNCH(LG, LG2, COLS, LD_PLAIN, ST_SCALE, CKKS_NTT_COL_MINB, Q1);
+        CKKS_MODES(LD_PLAIN, ST_MODDOWN) CKKS_LAUNCH(LG, LG2, COLS, LD_PLAIN, ST_MODDOWN, CKKS_NTT_COL_WIDE_MINB, Q1);
+    }
+    return cudaErrorInvalidValue;
+}
+
+template <bool FWD, bool TABLE, bool Q1, int LG>
+static inline cudaError_t dispatch_blocks(const NttPhase &P, const LimbJobs *J, const NttJob *jobs, int n_jobs,
+                                          const LoadSpec &L, const StoreSpec &S, const PhaseLaunch &G) {
+    if constexpr (FWD) {
+        CKKS_MODES(LD_PLAIN, ST_REDUCE) CKKS_LAUNCH(LG, LG, BLOCKS, LD_PLAIN, ST_REDUCE, CKKS_NTT_BLOCK_MINB, Q1);
+        CKKS_MODES(LD_PLAIN, ST_MRS) CKKS_LAUNCH(LG, LG, BLOCKS, LD_PLAIN, ST_MRS, CKKS_NTT_BLOCK_MINB, Q1);
+        CKKS_MODES(LD_PLAIN, ST_ADDSUB) CKKS_LAUNCH(LG, LG, BLOCKS, LD_PLAIN, ST_ADDSUB, CKKS_NTT_BLOCK_MINB, Q1);
+    } else {
+        CKKS_MODES(LD_PLAIN, ST_LAZY) CKKS_LAUNCH(LG, LG, BLOCKS, LD_PLAIN, ST_LAZY, CKKS_NTT_BLOCK_MINB, Q1);
+        CKKS_MODES(LD_ADD, ST_LAZY) CKKS_LAUNCH(LG, LG, BLOCKS, LD_ADD, ST_LAZY, CKKS_NTT_BLOCK_MINB, Q1);
+    }
+    return cudaErrorInvalidValue;
+}
 
 template <bool FWD, bool TABLE, bool Q1>
-static inline cudaError_t dispatch_fast(bool cols, int logn, const NttPhase &P, const LimbJobs *J,
-                                        const NttJob *jobs, int n_jobs, const LoadSpec &L, const StoreSpec &S,
-                                        const PhaseLaunch &G, bool &found) {
-    found = true;
-    // specialised: the phase that fuses a mode has the plain mode on its other side
-#define CKKS_FAST(LG)                                                                              \
-    if (logn == LG) {                                                                              \
-        if constexpr (FWD) {                                                                       \
-            if (cols && S.mode == ST_LAZY) {                                                       \
-                if (L.mode == LD_PLAIN) CKKS_LAUNCH(LG, true, LD_PLAIN, ST_LAZY, CKKS_NTT_FAST_MINB, Q1); \
-                if (L.mode == LD_EQ17) CKKS_LAUNCH(LG, true, LD_EQ17, ST_LAZY, CKKS_NTT_EQ17_MINB, Q1);   \
-            }                                                                                      \
-            if (!cols && L.mode == LD_PLAIN) {                                                     \
-                if (S.mode == ST_REDUCE) CKKS_LAUNCH(LG, false, LD_PLAIN, ST_REDUCE, CKKS_NTT_FAST_MINB, Q1); \
-                if (S.mode == ST_MRS) CKKS_LAUNCH(LG, false, LD_PLAIN, ST_MRS, CKKS_NTT_FAST_MINB, Q1);   \
-            }                                                                                      \
-        } else {                                                                                   \
-            if (!cols && S.mode == ST_LAZY) {                                                      \
-                if (L.mode == LD_PLAIN) CKKS_LAUNCH(LG, false, LD_PLAIN, ST_LAZY, CKKS_NTT_FAST_MINB, Q1); \
-                if (L.mode == LD_ADD) CKKS_LAUNCH(LG, false, LD_ADD, ST_LAZY, CKKS_NTT_FAST_MINB, Q1);    \
-            }                                                                                      \
-            if (cols && L.mode == LD_PLAIN) {                                                      \
-                if (S.mode == ST_SCALE) CKKS_LAUNCH(LG, true, LD_PLAIN, ST_SCALE, CKKS_NTT_FAST_MINB, Q1); \
-                if (S.mode == ST_MODDOWN) CKKS_LAUNCH(LG, true, LD_PLAIN, ST_MODDOWN, CKKS_NTT_FAST_MINB, Q1); \
-            }                                                                                      \
-        }                                                                                          \
+static inline cudaError_t dispatch_two(int logn, const NttPhase &P, const LimbJobs *J, const NttJob *jobs,
+                                       int n_jobs, const LoadSpec &L, const StoreSpec &S, const PhaseLaunch &G) {
+#define CKKS_COLS(LG, LG2) \
+    if (logn == LG && P.log_n2 == LG2) return dispatch_cols<FWD, TABLE, Q1, LG, LG2>(P, J, jobs, n_jobs, L, S, G)
+    if (G.shape == COLS) {
+        if constexpr (!Q1) CKKS_COLS(6, 7);
+        CKKS_COLS(7, 7);
+        CKKS_COLS(7, 8);
+        CKKS_COLS(8, 8);
+    } else {
+        if (logn == 7) return dispatch_blocks<FWD, TABLE, Q1, 7>(P, J, jobs, n_jobs, L, S, G);
+        if (logn == 8) return dispatch_blocks<FWD, TABLE, Q1, 8>(P, J, jobs, n_jobs, L, S, G);
     }
-    CKKS_FAST(7)
-    CKKS_FAST(8)
-#undef CKKS_FAST
-    found = false;
-    return cudaSuccess;
+#undef CKKS_COLS
+    return cudaErrorInvalidValue;
+}
+
+template <bool FWD, bool TABLE, int LG>
+static inline cudaError_t dispatch_whole_n(const NttPhase &P, const LimbJobs *J, const NttJob *jobs, int n_jobs,
+                                           const LoadSpec &L, const StoreSpec &S, const PhaseLaunch &G) {
+    if constexpr (FWD) {
+        CKKS_MODES(LD_PLAIN, ST_REDUCE) CKKS_LAUNCH(LG, 0, WHOLE, LD_PLAIN, ST_REDUCE, 2, false);
+        CKKS_MODES(LD_EQ17, ST_REDUCE) CKKS_LAUNCH(LG, 0, WHOLE, LD_EQ17, ST_REDUCE, 2, false);
+        CKKS_MODES(LD_EQ17, ST_MRS) CKKS_LAUNCH(LG, 0, WHOLE, LD_EQ17, ST_MRS, 2, false);
+        CKKS_MODES(LD_BCONVK, ST_ADDSUB) CKKS_LAUNCH(LG, 0, WHOLE, LD_BCONVK, ST_ADDSUB, 2, false);
+    } else {
+        CKKS_MODES(LD_PLAIN, ST_SCALE) CKKS_LAUNCH(LG, 0, WHOLE, LD_PLAIN, ST_SCALE, 2, false);
+        CKKS_MODES(LD_ADD, ST_MODDOWN) CKKS_LAUNCH(LG, 0, WHOLE, LD_ADD, ST_MODDOWN, 2, false);
+        CKKS_MODES(LD_PLAIN, ST_MODDOWN) CKKS_LAUNCH(LG, 0, WHOLE, LD_PLAIN, ST_MODDOWN, 2, false);
+    }
+    return cudaErrorInvalidValue;
 }
 
 template <bool FWD, bool TABLE>
-static inline cudaError_t dispatch_generic(bool cols, int logn, const NttPhase &P, const LimbJobs *J,
-                                           const NttJob *jobs, int n_jobs, const LoadSpec &L, const StoreSpec &S,
-                                           const PhaseLaunch &G) {
-#define CKKS_GENERIC(LG)                                                          \
-    case LG:                                                                      \
-        if (cols) CKKS_LAUNCH(LG, true, -1, -1, CKKS_NTT_MINB, false);            \
-        CKKS_LAUNCH(LG, false, -1, -1, CKKS_NTT_MINB, false)
+static inline cudaError_t dispatch_whole(int logn, const NttPhase &P, const LimbJobs *J, const NttJob *jobs,
+                                         int n_jobs, const LoadSpec &L, const StoreSpec &S, const PhaseLaunch &G) {
     switch (logn) {
-        CKKS_GENERIC(1);
-        CKKS_GENERIC(2);
-        CKKS_GENERIC(3);
-        CKKS_GENERIC(4);
-        CKKS_GENERIC(5);
-        CKKS_GENERIC(6);
-        CKKS_GENERIC(7);
-        CKKS_GENERIC(8);
-    default:
-        return cudaErrorInvalidValue;
+    case 9: return dispatch_whole_n<FWD, TABLE, 9>(P, J, jobs, n_jobs, L, S, G);
+    case 10: return dispatch_whole_n<FWD, TABLE, 10>(P, J, jobs, n_jobs, L, S, G);
+    case 11: return dispatch_whole_n<FWD, TABLE, 11>(P, J, jobs, n_jobs, L, S, G);
+    case 12: return dispatch_whole_n<FWD, TABLE, 12>(P, J, jobs, n_jobs, L, S, G);
+    default: return cudaErrorInvalidValue;
     }
-#undef CKKS_GENERIC
+}
+
+template <bool FWD>
+static inline cudaError_t dispatch_tiny(int logn, const NttPhase &P, const LimbJobs *J, const LoadSpec &L,
+                                        const StoreSpec &S, const PhaseLaunch &G) {
+    constexpr bool TABLE = false;
+    const NttJob *jobs = nullptr;
+    const int n_jobs = 0;
+    switch (logn) {
+    case 4: CKKS_LAUNCH(4, 0, BLOCKS, -1, -1, 2, false);
+    case 5: CKKS_LAUNCH(5, 0, BLOCKS, -1, -1, 2, false);
+    case 6: CKKS_LAUNCH(6, 0, BLOCKS, -1, -1, 2, false);
+    case 7: CKKS_LAUNCH(7, 0, BLOCKS, -1, -1, 2, false);
+    case 8: CKKS_LAUNCH(8, 0, BLOCKS, -1, -1, 2, false);
+    default: return cudaErrorInvalidValue;
+    }
 }
 #undef CKKS_LAUNCH
+#undef CKKS_MODES
 
-// general products: the specialised kernel if one matches, else the generic one
-template <bool FWD, bool TABLE>
-static inline cudaError_t dispatch_phase(bool cols, int logn, const NttPhase &P, const LimbJobs *J,
-                                         const NttJob *jobs, int n_jobs, const LoadSpec &L, const StoreSpec &S,
-                                         const PhaseLaunch &G) {
-    bool found;
-    const cudaError_t e = dispatch_fast<FWD, TABLE, false>(cols, logn, P, J, jobs, n_jobs, L, S, G, found);
-    if (found) return e;
-    return dispatch_generic<FWD, TABLE>(cols, logn, P, J, jobs, n_jobs, L, S, G);
-}
-
-// ntt_uf.cu / ntt_ui.cu / ntt_tf.cu / ntt_ti.cu: general products;
-// ntt_uf1.cu / ntt_ui1.cu / ntt_tf1.cu / ntt_ti1.cu: the specialised kernels
-// with the products for primes = 1 (mod 2^32) (`found` false when none
-// matches: the caller then takes the general dispatch)
-cudaError_t ntt_dispatch_q1_uniform_fwd(bool cols, int logn, const NttPhase &P, const LimbJobs &J,
-                                        const LoadSpec &L, const StoreSpec &S, const PhaseLaunch &G, bool &found);
-cudaError_t ntt_dispatch_q1_uniform_inv(bool cols, int logn, const NttPhase &P, const LimbJobs &J,
-                                        const LoadSpec &L, const StoreSpec &S, const PhaseLaunch &G, bool &found);
-cudaError_t ntt_dispatch_q1_table_fwd(bool cols, int logn, const NttPhase &P, const NttJob *jobs, int n_jobs,
-                                      const LoadSpec &L, const StoreSpec &S, const PhaseLaunch &G, bool &found);
-cudaError_t ntt_dispatch_q1_table_inv(bool cols, int logn, const NttPhase &P, const NttJob *jobs, int n_jobs,
-                                      const LoadSpec &L, const StoreSpec &S, const PhaseLaunch &G, bool &found);
-cudaError_t ntt_dispatch_uniform_fwd(bool cols, int logn, const NttPhase &P, const LimbJobs &J, const LoadSpec &L,
-                                     const StoreSpec &S, const PhaseLaunch &G);
-cudaError_t ntt_dispatch_uniform_inv(bool cols, int logn, const NttPhase &P, const LimbJobs &J, const LoadSpec &L,
-                                     const StoreSpec &S, const PhaseLaunch &G);
-cudaError_t ntt_dispatch_table_fwd(bool cols, int logn, const NttPhase &P, const NttJob *jobs, int n_jobs,
-                                   const LoadSpec &L, const StoreSpec &S, const PhaseLaunch &G);
-cudaError_t ntt_dispatch_table_inv(bool cols, int logn, const NttPhase &P, const NttJob *jobs, int n_jobs,
-                                   const LoadSpec &L, const StoreSpec &S, const PhaseLaunch &G);
+// One translation unit per direction, job source (u: uniform, t: table) and
+// product form (ntt_*1.cu: primes = 1 (mod 2^32)) so that they compile in
+// parallel; ntt_whole.cu holds the one-phase kernels.
+#define CKKS_DECL(name)                                                                              \
+    cudaError_t name(int logn, const NttPhase &P, const LimbJobs *J, const NttJob *jobs, int n_jobs, \
+                     const LoadSpec &L, const StoreSpec &S, const PhaseLaunch &G)
+CKKS_DECL(ntt_two_uf);
+CKKS_DECL(ntt_two_ui);
+CKKS_DECL(ntt_two_tf);
+CKKS_DECL(ntt_two_ti);
+CKKS_DECL(ntt_two_uf1);
+CKKS_DECL(ntt_two_ui1);
+CKKS_DECL(ntt_two_tf1);
+CKKS_DECL(ntt_two_ti1);
+CKKS_DECL(ntt_whole_uf);
+CKKS_DECL(ntt_whole_ui);
+CKKS_DECL(ntt_whole_tf);
+CKKS_DECL(ntt_whole_ti);
+#undef CKKS_DECL
 
 }  // namespace ckks

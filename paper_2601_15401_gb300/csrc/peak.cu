@@ -1,9 +1,8 @@
 // Integer-arithmetic peaks of this GPU for the operations the hot path is
 // built from, measured with register-only kernels (no memory traffic):
-//   kind 0  lazy Shoup product  x w - floor(x w'/2^64) q      (NTT twiddles,
-//           fused scalings)
-//   kind 1  Harvey's lazy Cooley-Tukey butterfly (one Shoup product plus its
-//           additions and correction; the forward NTT's unit of work)
+//   kind 0  lazy Shoup product with the balanced companion (fused scalings)
+//   kind 1  lazy Cooley-Tukey butterfly in the form the NTT runs for this q
+//           (arith.cuh; the forward NTT's unit of work)
 //   kind 2  64 x 64 -> 128-bit multiply-accumulate (BConv, key MAC, tensor
 //           product dot products)
 //   kind 3  Montgomery product with R = 2^64 (tensor product, key preparation)
@@ -13,7 +12,7 @@
 //           shuffles: four XOR stages of 8 swaps, no barrier
 //   kind 5  the same exchange through shared memory (store, __syncwarp,
 //           load), the way the NTT kernels pass data between passes
-//   kind 6  kind 1 for a modulus q = 1 (mod 2^32) (shoup_lazy_q1)
+//   kind 6  kind 1 for a modulus q = 1 (mod 2^32)
 //   kind 7  kind 0 for a modulus q = 1 (mod 2^32)
 // Kinds 4 and 5 count one operation per value moved.
 // Each thread runs kChains independent dependency chains so that issue, not
@@ -30,22 +29,6 @@ struct PeakConsts {
     u64 q, qinv;
     u64 w[kChains], wp[kChains];
 };
-
-__device__ __forceinline__ void ct_bfly_peak(u64 &X, u64 &Y, u64 w, u64 wp, u64 q) {
-    const u64 q2 = q << 1;
-    const u64 x = X >= q2 ? X - q2 : X;
-    const u64 t = shoup_lazy(Y, w, wp, q);
-    X = x + t;
-    Y = x - t + q2;
-}
-
-__device__ __forceinline__ void ct_bfly_peak_q1(u64 &X, u64 &Y, u64 w, u64 wp, u64 q) {
-    const u64 q2 = q << 1;
-    const u64 x = X >= q2 ? X - q2 : X;
-    const u64 t = shoup_lazy_q1(Y, w, wp, (uint32_t)(q >> 32));
-    X = x + t;
-    Y = x - t + q2;
-}
 
 // 16 x 16 transpose within each half-warp: lane i holds row i in v[0..15];
 // afterwards it holds column i. Stage s swaps the elements whose index bit
@@ -70,7 +53,8 @@ __device__ __forceinline__ void transpose16_shfl(u64 (&v)[16]) {
     }
 }
 
-template <int KIND>
+// SMALL: the butterfly form of primes below 2^kSmallBits
+template <int KIND, bool SMALL = false>
 __global__ void __launch_bounds__(256) peak_kernel(PeakConsts P, int iters, u64 *out) {
     const u64 tid = (u64)blockIdx.x * blockDim.x + threadIdx.x;
     const u64 q = P.q;
@@ -83,18 +67,18 @@ __global__ void __launch_bounds__(256) peak_kernel(PeakConsts P, int iters, u64 
     Acc128Lazy acc[kChains];
 #pragma unroll
     for (int i = 0; i < kChains; ++i) acc[i].zero();
-    const ModQ m{q, P.qinv};
+    const ModQ m{q, P.qinv, {0, 0}, 0};
     for (int it = 0; it < iters; ++it) {
 #pragma unroll
         for (int i = 0; i < kChains; ++i) {
             if (KIND == 0) {
-                x[i] = shoup_lazy(x[i], P.w[i], P.wp[i], q);
+                x[i] = shoup_signed<false>(x[i], P.w[i], P.wp[i], q);
             } else if (KIND == 1) {
-                ct_bfly_peak(x[i], y[i], P.w[i], P.wp[i], q);
+                ct_bfly<SMALL, false>(x[i], y[i], P.w[i], P.wp[i], q);
             } else if (KIND == 6) {
-                ct_bfly_peak_q1(x[i], y[i], P.w[i], P.wp[i], q);
+                ct_bfly<SMALL, true>(x[i], y[i], P.w[i], P.wp[i], q);
             } else if (KIND == 7) {
-                x[i] = shoup_lazy_q1(x[i], P.w[i], P.wp[i], (uint32_t)(q >> 32));
+                x[i] = shoup_signed<true>(x[i], P.w[i], P.wp[i], q);
             } else if (KIND == 2) {
                 acc[i].mac(x[i], P.w[i]);
                 x[i] += y[i];
@@ -154,16 +138,23 @@ extern "C" int ckks_peak_int(int kind, uint64_t q, const uint64_t *w, const uint
     P.qinv = inv;
     for (int i = 0; i < kChains; ++i) {
         if (w[i] >= q) return CKKS_EINVAL;
-        P.w[i] = w[i];
-        P.wp[i] = wp[i];
+        const Shoup c = kind == 1 || kind == 6 ? make_twiddle(w[i], q) : make_shoup(w[i], q);
+        P.w[i] = c.w;
+        P.wp[i] = c.wp;
     }
     cudaStream_t st = (cudaStream_t)stream;
     switch (kind) {
     case 0: peak_kernel<0><<<blocks, threads, 0, st>>>(P, iters, (u64 *)out); break;
-    case 1: peak_kernel<1><<<blocks, threads, 0, st>>>(P, iters, (u64 *)out); break;
+    case 1:
+        if (small_prime(q)) peak_kernel<1, true><<<blocks, threads, 0, st>>>(P, iters, (u64 *)out);
+        else peak_kernel<1><<<blocks, threads, 0, st>>>(P, iters, (u64 *)out);
+        break;
     case 2: peak_kernel<2><<<blocks, threads, 0, st>>>(P, iters, (u64 *)out); break;
     case 3: peak_kernel<3><<<blocks, threads, 0, st>>>(P, iters, (u64 *)out); break;
-    case 6: peak_kernel<6><<<blocks, threads, 0, st>>>(P, iters, (u64 *)out); break;
+    case 6:
+        if (small_prime(q)) peak_kernel<6, true><<<blocks, threads, 0, st>>>(P, iters, (u64 *)out);
+        else peak_kernel<6><<<blocks, threads, 0, st>>>(P, iters, (u64 *)out);
+        break;
     case 7: peak_kernel<7><<<blocks, threads, 0, st>>>(P, iters, (u64 *)out); break;
     case 4: exchange_kernel<4><<<blocks, threads, 0, st>>>(iters, (u64 *)out); break;
     default: exchange_kernel<5><<<blocks, threads, 0, st>>>(iters, (u64 *)out); break;

@@ -130,6 +130,7 @@ struct Builder {
     const Context &C;
     const u64 *keys;
     int H;
+    bool one_phase;  // N <= 2^12: a transform is one launch
     std::map<std::pair<int, int>, Stage> st;
 
     Stage &at(int round, int step, int kind) {
@@ -139,11 +140,28 @@ struct Builder {
     }
     int prime_of_slot(int x, int level) const { return x < level ? x : C.L + (x - level); }
 
-    // both phases of one transform: phase-1 entry, phase-2 entry
+    // both phases of one transform: phase-1 entry, phase-2 entry (one entry
+    // with the first's load and the second's store where one launch does all)
     void ntt_pair(int round, int step, bool fwd, const NttJob &p1, const NttJob &p2, const LoadSpec &L1,
                   const StoreSpec &S1, const LoadSpec &L2, const StoreSpec &S2, double bytes1, double bytes2,
                   double ops1, double ops2) {
         Stage &a = at(round, step, SK_NTT);
+        if (one_phase) {
+            NttJob j = p1;
+            j.dst = p2.dst;
+            j.aux = p2.aux;
+            j.aux2 = p2.aux2;
+            j.c = p2.c;
+            a.fwd = fwd;
+            a.cols = false;
+            a.L = L1;
+            a.S = S2;
+            a.ntt.push_back(j);
+            a.bytes += bytes1 + bytes2 - 2.0 * C.N * sizeof(u64);  // the intermediate stays on chip
+            a.ops += ops1 + ops2;
+            a.limb_transforms += 1;
+            return;
+        }
         a.fwd = fwd;
         a.cols = fwd;  // forward starts with the column phase, inverse with the block phase
         a.L = L1;
@@ -162,6 +180,12 @@ struct Builder {
         b.ops += ops2;
     }
 };
+
+bool one_phase(const Context &C) {
+    int log_n1, log_n2;
+    ntt_geometry(C.log_n, log_n1, log_n2);
+    return log_n1 == 0;
+}
 
 int node_heights(const Plan &P, std::vector<int> &h) {
     h.assign(P.nodes.size(), 0);
@@ -452,7 +476,7 @@ int build(ckks_wave &W, char *scratch, std::vector<char> &tables) {
         std::vector<int> h;
         H = std::max(H, node_heights(*w.plan, h));
     }
-    Builder B{C, W.evk->keys, H, {}};
+    Builder B{C, W.evk->keys, H, one_phase(C), {}};
     Bump bump{scratch, 0};
     for (const WaveProduct &w : W.items) build_product(B, w, bump);
     W.stages.clear();
@@ -536,7 +560,7 @@ cudaError_t enqueue(ckks_wave &W, char *ws /* the job tables */, cudaStream_t st
         const int n = s.count();
         switch (s.kind) {
         case SK_NTT:
-            if (s.fwd == s.cols) count_op(C, s.fwd ? OP_LIMB_NTT : OP_LIMB_INTT, s.limb_transforms);
+            if (s.limb_transforms) count_op(C, s.fwd ? OP_LIMB_NTT : OP_LIMB_INTT, s.limb_transforms);
             e = launch_ntt_phase_table(C, s.fwd, s.cols, (const NttJob *)(ws + s.off), n, s.L, s.S, s.bytes, s.ops,
                                        st);
             break;
@@ -577,9 +601,7 @@ int ckks_wave_create(ckks_context *ctx, const ckks_wave_item *items, uint32_t n,
     *out = nullptr;
     if (!ctx || !items || n < 1 || !evk || evk->ctx != ctx) return CKKS_EINVAL;
     const Context &C = ctx->c;
-    int log_n1, log_n2;
-    ntt_geometry(C.log_n, log_n1, log_n2);
-    if (log_n1 == 0) return CKKS_EINVAL;  // ring degrees of one-phase transforms (N <= 256) are not supported
+    if (C.log_n <= 8) return CKKS_EINVAL;  // N <= 256 is not supported
     ckks_wave *W = new (std::nothrow) ckks_wave();
     if (!W) return CKKS_ENOMEM;
     W->ctx = ctx;
@@ -636,7 +658,7 @@ int ckks_wave_create(ckks_context *ctx, const ckks_wave_item *items, uint32_t n,
             std::vector<int> h;
             H = std::max(H, node_heights(*w.plan, h));
         }
-        Builder B{C, evk->keys, H, {}};
+        Builder B{C, evk->keys, H, one_phase(C), {}};
         for (const WaveProduct &w : W->items) build_product(B, w, sizing);
     }
     W->scratch_bytes = sizing.off;
