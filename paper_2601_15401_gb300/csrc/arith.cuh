@@ -229,6 +229,76 @@ CKKS_HD u64 canonical(u64 v, u64 q, Canon c) {
 }
 
 // ---------------------------------------------------------------------------
+// dot products by limbs
+// ---------------------------------------------------------------------------
+// Operands v = v0 + v1 2^SB with both limbs below 2^30; a product is three
+// wide multiply-adds, one per sum (Karatsuba's middle term), with no carry
+// between them:
+//   s0 = sum a0 b0,  s1 = sum a1 b1,  sx = sum (a0 + a1)(b0 + b1),
+//   a . b = s0 + (sx - s0 - s1) 2^SB + s1 2^(2 SB),
+// exact while s0, s1 and the middle sum a0 b1 + a1 b0 stay below 2^64 (sx may
+// wrap: only the difference counts). SB = 30 (operands below 2^60): at most 8
+// terms. SB = 27 (small primes: limbs below 2^27 and 2^26): at most 512
+// terms. Measured as a register-only stream on a GB300: 15.8 warp cycles per
+// product and scheduler, against 33-40 for a 64 x 64 -> 128-bit product (high
+// and low words separately) added with carry.
+constexpr int kLimbTerms30 = 8;
+constexpr int kLimbTerms27 = 512;
+
+struct Limbs {
+    u32 lo, hi, sum;
+};
+
+template <int SB>
+CKKS_HD Limbs split_limbs(u64 v) {
+    Limbs l;
+    l.lo = (u32)v & ((1u << SB) - 1);
+    l.hi = (u32)(v >> SB);
+    l.sum = l.lo + l.hi;
+    return l;
+}
+
+// a word holding its own limbs (low limb in the low half)
+template <int SB>
+CKKS_HD u64 pack_limbs(u64 v) {
+    return ((v >> SB) << 32) | (v & ((1u << SB) - 1));
+}
+CKKS_HD Limbs packed_limbs(u64 w) { return Limbs{lo32(w), hi32(w), lo32(w) + hi32(w)}; }
+
+struct DotLimbs {
+    u64 s0, s1, sx;
+    CKKS_HD void zero() { s0 = s1 = sx = 0; }
+    CKKS_HD void mac(const Limbs &a, const Limbs &b) {
+        s0 = mad_wide(a.lo, b.lo, s0);
+        s1 = mad_wide(a.hi, b.hi, s1);
+        sx = mad_wide(a.sum, b.sum, sx);
+    }
+    // SB = 30: brings the sums of up to 7 terms (or of a folded value, worth
+    // one, and 6 terms) back to a value below 2 q 2^60 + 2^60: the middle sum's
+    // high part and the high sum, reduced mod q, and two low limbs.
+    CKKS_HD void fold(u64 q, Canon c) {
+        u64 x = sx - s0 - s1;
+        x += s0 >> 30;
+        s0 &= (1u << 30) - 1;
+        // s1 + (x >> 30) < 7 2^60 + 2^35: below 256 q for q >= 2^53
+        s1 = reduce_near(s1 + (x >> 30), q, c);
+        x &= (1u << 30) - 1;
+        sx = x + s0 + s1;
+    }
+    // the sum as hi 2^64 + lo
+    template <int SB>
+    CKKS_HD void value(u64 &hi, u64 &lo) const {
+        const u64 x = sx - s0 - s1;
+        u64 l = s0 + (x << SB);
+        u64 h = (x >> (64 - SB)) + (s1 >> (64 - 2 * SB)) + (l < s0 ? 1ull : 0ull);
+        const u64 m = l + (s1 << (2 * SB));
+        h += m < l ? 1ull : 0ull;
+        lo = m;
+        hi = h;
+    }
+};
+
+// ---------------------------------------------------------------------------
 // host: companions
 // ---------------------------------------------------------------------------
 // (w, balanced companion) for 0 <= w < q: w (mod 2^64, possibly negative) and

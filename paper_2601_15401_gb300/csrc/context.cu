@@ -108,6 +108,8 @@ int context_build(Context &C, const uint32_t log_n, const uint32_t L, const uint
     }
     C.primes_q1 = true;
     for (int i = 0; i < NP; ++i) C.primes_q1 = C.primes_q1 && (C.primes[i] & 0xffffffffull) == 1;
+    C.limbs30 = true;
+    for (int i = 0; i < NP; ++i) C.limbs30 = C.limbs30 && (C.primes[i] >> 60) == 0;
     // BConv sums of products stay below hi < q only if sum of source primes < 2^64
     // (see Acc128); check every digit and the P basis.
     {

@@ -163,6 +163,8 @@ struct Context {
     // cheaper forms of the Shoup product and of REDC (shoup_lazy_q1,
     // redc_q1); set at creation. tune_q1 = 0 keeps the general forms.
     bool primes_q1 = false;
+    // every prime is below 2^60: dot products run on 30-bit limbs (DotLimbs)
+    bool limbs30 = false;
     int tune_q1 = 1;
     bool q1() const { return primes_q1 && tune_q1 != 0; }
 };

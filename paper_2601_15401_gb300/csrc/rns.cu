@@ -374,36 +374,52 @@ cudaError_t launch_tensor_table(const Context &C, const TensorJob *jobs, int n_j
 // y'_j = [y_j (Q_beta/q_j)^-1]_{q_j} was produced by the INTT's epilogue.
 // blockIdx.y = (t, beta) job, blockIdx.z = batch.
 // ---------------------------------------------------------------------------
-// Coefficients per thread of the key MAC: four adjacent coefficients read
-// with two 16-byte loads per stream (more bytes in flight per thread; the
-// kernel is bound by load latency, not by its multiplies). Measured on the
-// bench step: 17.5 ms at four, 18.1 at two, 19.4 at one.
+// Coefficients per thread of the key MAC of single products / of pairs of
+// products (CKKS_MAC_PAIR, rns.h: two products of the same shape share each
+// term's key loads), its largest block (the "mac_threads" tunable is cut to
+// it) and the CTAs of that size per SM it is compiled for.
 #ifndef CKKS_MAC_VEC
-#define CKKS_MAC_VEC 4
+#define CKKS_MAC_VEC 2
 #endif
-// Two products of the same shape per thread share each term's key loads
-// (CKKS_MAC_PAIR, rns.h), two coefficients each.
 #ifndef CKKS_MAC_VEC_PAIR
-#define CKKS_MAC_VEC_PAIR 2
+#define CKKS_MAC_VEC_PAIR 1
 #endif
-// Largest key-MAC block (the "mac_threads" tunable's upper bound). At 1024
-// the four-coefficient form gets 64 registers and spills 96-196 bytes a
-// thread to L1; bounding the block at 512 removed the spills (106
-// registers) but cut the resident warps, and the MAC took 20.3 instead of
-// 17.5 ms per bench step.
-#define CKKS_MAC_MAX_THREADS 1024
+#define CKKS_MAC_MAX_THREADS 256
+#ifndef CKKS_MAC_MINB
+#define CKKS_MAC_MINB 4
+#endif
 
-// Coefficients per thread of BConv (1: measured fastest; 2 was 3 % slower)
+// Limb width of a prime's keys and accumulators: 27 bits for small primes
+// when the terms of the largest product (11 keys, every digit) fit one sum.
+__device__ __forceinline__ int key_limb_bits(u64 q, int key_digits) {
+    return small_prime(q) && 11 * key_digits <= kLimbTerms27 ? 27 : 30;
+}
+// Coefficients per thread of BConv, its largest block (the "bconv_threads"
+// tunable is cut to it) and the CTAs of that size per SM it is compiled for.
 #ifndef CKKS_BCONV_VEC
-#define CKKS_BCONV_VEC 1
+#define CKKS_BCONV_VEC 2
+#endif
+#define CKKS_BCONV_MAX_THREADS 256
+#ifndef CKKS_BCONV_MINB
+#define CKKS_BCONV_MINB 3
 #endif
 
-// One CTA: the constants of (level, digit) staged in shared memory, then one
-// coefficient per thread. y: limb 0 of the prescaled d_t; dst: slot 0 of the
-// (t, digit) ModUp output.
-template <int AMAX, bool Q1>
+// One CTA: the constants of (level, digit) staged in shared memory, then
+// CKKS_BCONV_VEC adjacent coefficients per thread (16-byte loads and stores
+// for two). y: limb 0 of the prescaled d_t; dst: slot 0 of the (t, digit)
+// ModUp output. Bound by the integer multiply pipe: |digit| products per
+// target and coefficient.
+// LIMB: the sources' limbs stay in registers, the constants hold their own
+// limbs in shared memory, a product is three multiply-adds; sums of more than
+// kLimbTerms30 sources are added as 128-bit words. Every lane reads the same
+// constant, but shared memory still returns 32 lanes' worth of bytes, so a
+// constant is one 8-byte word (its limbs' sum is added up again) and serves
+// CKKS_BCONV_VEC coefficients. Otherwise (a prime of 2^60 or more)
+// 64 x 64 -> 128-bit products.
+template <int AMAX, bool Q1, bool LIMB>
 __device__ __forceinline__ void bconv_block(const u64 *ctab, const u64 *y0, u64 *dst0, int level, int beta,
-                                            int alpha, int L, int K, int n_primes, int N, const ModQ *mods, u64 *cs) {
+                                            int alpha, int L, int K, int n_primes, int N, const ModQ *mods,
+                                            u64 *cs) {
     const int d0 = beta * alpha;
     int d1 = d0 + alpha;
     if (d1 > level) d1 = level;
@@ -414,11 +430,10 @@ __device__ __forceinline__ void bconv_block(const u64 *ctab, const u64 *y0, u64 
     for (int i = threadIdx.x; i < na * n_t; i += blockDim.x) {
         int jj = i / n_t, ti = i % n_t;
         int x = ti < nq_t ? (ti < d0 ? ti : ti + na) : L + (ti - nq_t);
-        cs[i] = ctab[(i64)jj * n_primes + x];
+        const u64 c = ctab[(i64)jj * n_primes + x];
+        cs[ti * na + jj] = LIMB ? pack_limbs<30>(c) : c;
     }
     __syncthreads();
-    // CKKS_BCONV_VEC adjacent coefficients per thread (16-byte loads and
-    // stores for two)
     constexpr int V = CKKS_BCONV_VEC;
     const int e = (blockIdx.x * blockDim.x + threadIdx.x) * V;
     if (e >= N) return;
@@ -431,72 +446,111 @@ __device__ __forceinline__ void bconv_block(const u64 *ctab, const u64 *y0, u64 
 #pragma unroll
             for (int v = 0; v < V; ++v) y[jj][v] = 0ull;
     }
+    Limbs yl[LIMB ? AMAX : 1][V];
+    if constexpr (LIMB) {
+#pragma unroll
+        for (int jj = 0; jj < AMAX; ++jj)
+#pragma unroll
+            for (int v = 0; v < V; ++v) yl[jj][v] = split_limbs<30>(y[jj][v]);
+    }
     u64 *dst = dst0 + e;
     for (int ti = 0; ti < n_t; ++ti) {
         const int slot = ti < nq_t ? (ti < d0 ? ti : ti + na) : level + (ti - nq_t);
         const int x = ti < nq_t ? slot : L + (ti - nq_t);
         const ModQ m = mods[x];
         // sum over the digit: hi stays below q because the digit's primes sum to < 2^64
-        Acc128Lazy acc[V];
-#pragma unroll
-        for (int v = 0; v < V; ++v) acc[v].zero();
-#pragma unroll
-        for (int jj = 0; jj < AMAX; ++jj)
-            if (jj < na) {
-                const u64 c = cs[jj * n_t + ti];
-#pragma unroll
-                for (int v = 0; v < V; ++v) acc[v].mac(y[jj][v], c);
-            }
         u64 r[V];
+        if constexpr (LIMB) {
+            const u64 *ct = cs + ti * na;
+            u64 hi[V], lo[V];
 #pragma unroll
-        for (int v = 0; v < V; ++v) r[v] = redc_t<Q1>(acc[v].hi, acc[v].lo, m);
+            for (int j0 = 0; j0 < AMAX; j0 += kLimbTerms30) {
+                DotLimbs acc[V];
+#pragma unroll
+                for (int v = 0; v < V; ++v) acc[v].zero();
+#pragma unroll
+                for (int k = 0; k < kLimbTerms30; ++k)
+                    if (j0 + k < AMAX && j0 + k < na) {
+                        const Limbs c = packed_limbs(ct[j0 + k]);
+#pragma unroll
+                        for (int v = 0; v < V; ++v) acc[v].mac(yl[j0 + k < AMAX ? j0 + k : 0][v], c);
+                    }
+#pragma unroll
+                for (int v = 0; v < V; ++v) {
+                    u64 h, l;
+                    acc[v].template value<30>(h, l);
+                    if (j0 == 0) {
+                        hi[v] = h;
+                        lo[v] = l;
+                    } else {
+                        lo[v] += l;
+                        hi[v] += h + (lo[v] < l ? 1ull : 0ull);
+                    }
+                }
+            }
+#pragma unroll
+            for (int v = 0; v < V; ++v) r[v] = redc_t<Q1>(hi[v], lo[v], m);
+        } else {
+            const u64 *ct = cs + ti * na;
+            Acc128Lazy acc[V];
+#pragma unroll
+            for (int v = 0; v < V; ++v) acc[v].zero();
+#pragma unroll
+            for (int jj = 0; jj < AMAX; ++jj)
+                if (jj < na) {
+                    const u64 c = ct[jj];
+#pragma unroll
+                    for (int v = 0; v < V; ++v) acc[v].mac(y[jj][v], c);
+                }
+#pragma unroll
+            for (int v = 0; v < V; ++v) r[v] = redc_t<Q1>(acc[v].hi, acc[v].lo, m);
+        }
         store_span<V>(dst + (i64)slot * N, r);
     }
 }
 
-template <int AMAX, bool Q1>
-__global__ void __launch_bounds__(1024) bconv_kernel(BconvArgs A) {
-    extern __shared__ u64 cs[];  // [alpha][n_targets] Montgomery constants
+template <int AMAX, bool Q1, bool LIMB>
+__global__ void __launch_bounds__(CKKS_BCONV_MAX_THREADS, CKKS_BCONV_MINB) bconv_kernel(BconvArgs A) {
+    extern __shared__ u64 cs[];  // [n_targets][|digit|] Montgomery constants
     const int job = blockIdx.y;
     const int b = blockIdx.z;
     const int t = job / A.n_digits;
     const int beta = job % A.n_digits;
-    bconv_block<AMAX, Q1>(A.consts + (i64)beta * A.alpha * A.n_primes,
+    bconv_block<AMAX, Q1, LIMB>(A.consts + (i64)beta * A.alpha * A.n_primes,
                       A.y.ptr + (i64)b * A.y.bstride + (i64)t * A.y.pstride,
                       A.ext.ptr + (i64)b * A.ext.bstride + (i64)(t * A.n_digits + beta) * A.ext.pstride, A.level, beta,
                       A.alpha, A.L, A.K, A.n_primes, A.N, A.mods, cs);
 }
 
 // Table launch: blockIdx.y = (product, d_t, digit) entry.
-template <int AMAX, bool Q1>
-__global__ void __launch_bounds__(1024) bconv_table_kernel(const BconvJob *jobs, int alpha, int L, int K,
+template <int AMAX, bool Q1, bool LIMB>
+__global__ void __launch_bounds__(CKKS_BCONV_MAX_THREADS, CKKS_BCONV_MINB) bconv_table_kernel(const BconvJob *jobs, int alpha, int L, int K,
                                                            int n_primes, int N, const ModQ *mods) {
     extern __shared__ u64 cs[];
     const BconvJob J = jobs[blockIdx.y];
-    bconv_block<AMAX, Q1>(J.consts, J.y, J.ext, J.level, J.beta, alpha, L, K, n_primes, N, mods, cs);
+    bconv_block<AMAX, Q1, LIMB>(J.consts, J.y, J.ext, J.level, J.beta, alpha, L, K, n_primes, N, mods, cs);
 }
 
-template <bool Q1>
+template <bool Q1, bool LIMB>
 static void launch_bconv_sized(int alpha, dim3 grid, int thr, size_t smem, const BconvArgs &A, cudaStream_t st) {
-    if (alpha <= 4) bconv_kernel<4, Q1><<<grid, thr, smem, st>>>(A);
-    else if (alpha <= 8) bconv_kernel<8, Q1><<<grid, thr, smem, st>>>(A);
-    else if (alpha <= 12) bconv_kernel<12, Q1><<<grid, thr, smem, st>>>(A);
-    else bconv_kernel<16, Q1><<<grid, thr, smem, st>>>(A);
+    if (alpha <= 4) bconv_kernel<4, Q1, LIMB><<<grid, thr, smem, st>>>(A);
+    else if (alpha <= 8) bconv_kernel<8, Q1, LIMB><<<grid, thr, smem, st>>>(A);
+    else if (alpha <= 12) bconv_kernel<12, Q1, LIMB><<<grid, thr, smem, st>>>(A);
+    else bconv_kernel<16, Q1, LIMB><<<grid, thr, smem, st>>>(A);
 }
 
-template <bool Q1>
+template <bool Q1, bool LIMB>
 static void launch_bconv_table_sized(const Context &C, dim3 grid, int thr, size_t smem, const BconvJob *jobs,
                                      cudaStream_t st) {
-    const int np = C.L + C.K;
-    if (C.alpha <= 4) bconv_table_kernel<4, Q1><<<grid, thr, smem, st>>>(jobs, C.alpha, C.L, C.K, np, C.N, C.d_mods);
-    else if (C.alpha <= 8) bconv_table_kernel<8, Q1><<<grid, thr, smem, st>>>(jobs, C.alpha, C.L, C.K, np, C.N, C.d_mods);
-    else if (C.alpha <= 12)
-        bconv_table_kernel<12, Q1><<<grid, thr, smem, st>>>(jobs, C.alpha, C.L, C.K, np, C.N, C.d_mods);
-    else bconv_table_kernel<16, Q1><<<grid, thr, smem, st>>>(jobs, C.alpha, C.L, C.K, np, C.N, C.d_mods);
+    const int np = C.L + C.K, a = C.alpha;
+    if (a <= 4) bconv_table_kernel<4, Q1, LIMB><<<grid, thr, smem, st>>>(jobs, a, C.L, C.K, np, C.N, C.d_mods);
+    else if (a <= 8) bconv_table_kernel<8, Q1, LIMB><<<grid, thr, smem, st>>>(jobs, a, C.L, C.K, np, C.N, C.d_mods);
+    else if (a <= 12) bconv_table_kernel<12, Q1, LIMB><<<grid, thr, smem, st>>>(jobs, a, C.L, C.K, np, C.N, C.d_mods);
+    else bconv_table_kernel<16, Q1, LIMB><<<grid, thr, smem, st>>>(jobs, a, C.L, C.K, np, C.N, C.d_mods);
 }
 
 cudaError_t launch_bconv(const Context &C, const BconvArgs &A, cudaStream_t st) {
-    const int thr = C.tune_bconv_threads;
+    const int thr = std::min(C.tune_bconv_threads, CKKS_BCONV_MAX_THREADS);
     dim3 grid((A.N + thr * CKKS_BCONV_VEC - 1) / (thr * CKKS_BCONV_VEC), A.n_t * A.n_digits, A.n_batch);
     size_t smem = (size_t)A.alpha * (A.level + A.K) * sizeof(u64);
     count_kernel(C);
@@ -511,8 +565,12 @@ cudaError_t launch_bconv(const Context &C, const BconvArgs &A, cudaStream_t st) 
     }
     macs *= (double)A.n_t * A.n_batch * A.N;
     ProfScope ps(C, KC_BCONV, ((double)A.n_t * A.level + limbs_out) * A.n_batch * A.N * sizeof(u64), st, macs);
-    if (C.q1()) launch_bconv_sized<true>(A.alpha, grid, thr, smem, A, st);
-    else launch_bconv_sized<false>(A.alpha, grid, thr, smem, A, st);
+    if (C.limbs30) {
+        if (C.q1()) launch_bconv_sized<true, true>(A.alpha, grid, thr, smem, A, st);
+        else launch_bconv_sized<false, true>(A.alpha, grid, thr, smem, A, st);
+    } else {
+        launch_bconv_sized<false, false>(A.alpha, grid, thr, smem, A, st);
+    }
     return cudaGetLastError();
 }
 
@@ -520,14 +578,18 @@ cudaError_t launch_bconv_table(const Context &C, const BconvJob *jobs, int n_job
                                cudaStream_t st) {
     if (n_jobs <= 0) return cudaSuccess;
     if (n_jobs > 65535) return cudaErrorInvalidValue;
-    const int thr = C.tune_bconv_threads;
+    const int thr = std::min(C.tune_bconv_threads, CKKS_BCONV_MAX_THREADS);
     dim3 grid((C.N + thr * CKKS_BCONV_VEC - 1) / (thr * CKKS_BCONV_VEC), (unsigned)n_jobs);
     size_t smem = (size_t)C.alpha * (C.L + C.K) * sizeof(u64);
     count_kernel(C);
     count_op(C, OP_BCONV, (unsigned long long)n_jobs);
     ProfScope ps(C, KC_BCONV, bytes, st, macs);
-    if (C.q1()) launch_bconv_table_sized<true>(C, grid, thr, smem, jobs, st);
-    else launch_bconv_table_sized<false>(C, grid, thr, smem, jobs, st);
+    if (C.limbs30) {
+        if (C.q1()) launch_bconv_table_sized<true, true>(C, grid, thr, smem, jobs, st);
+        else launch_bconv_table_sized<false, true>(C, grid, thr, smem, jobs, st);
+    } else {
+        launch_bconv_table_sized<false, false>(C, grid, thr, smem, jobs, st);
+    }
     return cudaGetLastError();
 }
 
@@ -540,21 +602,26 @@ cudaError_t launch_bconv_table(const Context &C, const BconvJob *jobs, int n_job
 // Grid: x = coefficient chunk, y = target limb, z = batch (fastest-varying
 // batch would reuse key tiles in L2; see launch order below).
 // ---------------------------------------------------------------------------
-// V coefficients of accumulator limb x of one product: dsrc / esrc point at
-// limb x, coefficient e of the D tuple / the first ModUp output; krow at the
-// prime's row, coefficient e, of the first key.
 // V coefficients of accumulator limb x of P products of the same shape
 // (level, n, digits) at once: the key words of each term are loaded once
 // for all P. dsrc / esrc point at limb x, coefficient e of each product's D
 // tuple / first ModUp output; krow at the prime's row, coefficient e, of the
 // first key.
-template <int V, int P, bool Q1>
+// FORM 0: 64 x 64 -> 128-bit products (a context with a prime of 2^60 or
+// more). FORM 1 / 2: products on limbs (DotLimbs, three multiply-adds each),
+// the prepared keys holding their own limbs (keyprep_kernel): 1 = big prime,
+// 30-bit limbs, the sums brought below 2 q 2^60 every 7 terms; 2 = small
+// prime, 27-bit limbs, no carry over all terms (at most 11 keys x 46 digits:
+// kLimbTerms27, else FORM 1's base is used; see key_limb_bits).
+template <int V, int P, bool Q1, int FORM>
 __device__ __forceinline__ void mac_span(const u64 *const *dsrc, const i64 *dstride, const u64 *const *esrc,
                                          const i64 *estride, int n, int nd, int my_digit, const u64 *krow,
                                          i64 key_pstride, int key_digits, const ModQ m, u64 *const *dst,
                                          const i64 *astride) {
     const u64 q = m.q;
-    Acc128 a0[P][V], a1[P][V];
+    constexpr int SB = FORM == 2 ? 27 : 30;
+    typedef typename std::conditional<FORM == 0, Acc128, DotLimbs>::type Acc;
+    Acc a0[P][V], a1[P][V];
 #pragma unroll
     for (int p = 0; p < P; ++p)
 #pragma unroll
@@ -562,6 +629,7 @@ __device__ __forceinline__ void mac_span(const u64 *const *dsrc, const i64 *dstr
             a0[p][v].zero();
             a1[p][v].zero();
         }
+    int left = kLimbTerms30 - 1;
     for (int t = 2; t <= n; ++t) {
         for (int beta = 0; beta < nd; ++beta) {
             const u64 *key = krow + ((i64)((t - 2) * key_digits + beta) * 2) * key_pstride;
@@ -574,13 +642,38 @@ __device__ __forceinline__ void mac_span(const u64 *const *dsrc, const i64 *dstr
             }
             load_span<V>(key, k0);
             load_span<V>(key + key_pstride, k1);
+            if constexpr (FORM == 0) {
 #pragma unroll
-            for (int p = 0; p < P; ++p)
+                for (int p = 0; p < P; ++p)
+#pragma unroll
+                    for (int v = 0; v < V; ++v) {
+                        a0[p][v].mac(tv[p][v], k0[v], q);
+                        a1[p][v].mac(tv[p][v], k1[v], q);
+                    }
+            } else {
 #pragma unroll
                 for (int v = 0; v < V; ++v) {
-                    a0[p][v].mac(tv[p][v], k0[v], q);
-                    a1[p][v].mac(tv[p][v], k1[v], q);
+                    const Limbs c0 = packed_limbs(k0[v]), c1 = packed_limbs(k1[v]);
+#pragma unroll
+                    for (int p = 0; p < P; ++p) {
+                        const Limbs x = split_limbs<SB>(tv[p][v]);
+                        a0[p][v].mac(x, c0);
+                        a1[p][v].mac(x, c1);
+                    }
                 }
+                if constexpr (FORM == 1) {
+                    if (--left == 0) {
+#pragma unroll
+                        for (int p = 0; p < P; ++p)
+#pragma unroll
+                            for (int v = 0; v < V; ++v) {
+                                a0[p][v].fold(q, m.canon);
+                                a1[p][v].fold(q, m.canon);
+                            }
+                        left = kLimbTerms30 - 2;
+                    }
+                }
+            }
         }
     }
 #pragma unroll
@@ -588,19 +681,40 @@ __device__ __forceinline__ void mac_span(const u64 *const *dsrc, const i64 *dstr
         u64 r0[V], r1[V];
 #pragma unroll
         for (int v = 0; v < V; ++v) {
-            r0[v] = redc_t<Q1>(a0[p][v].hi, a0[p][v].lo, m);
-            r1[v] = redc_t<Q1>(a1[p][v].hi, a1[p][v].lo, m);
+            u64 h0, l0, h1, l1;
+            if constexpr (FORM == 0) {
+                h0 = a0[p][v].hi, l0 = a0[p][v].lo, h1 = a1[p][v].hi, l1 = a1[p][v].lo;
+            } else {
+                a0[p][v].template value<SB>(h0, l0);
+                a1[p][v].template value<SB>(h1, l1);
+            }
+            r0[v] = redc_t<Q1>(h0, l0, m);
+            r1[v] = redc_t<Q1>(h1, l1, m);
         }
         store_span<V>(dst[p], r0);
         store_span<V>(dst[p] + astride[p], r1);
     }
 }
 
+// the FORM of a prime's accumulators
+template <int V, int P, bool Q1, bool LIMB>
+__device__ __forceinline__ void mac_limb(const u64 *const *dsrc, const i64 *dstride, const u64 *const *esrc,
+                                         const i64 *estride, int n, int nd, int my_digit, const u64 *krow,
+                                         i64 key_pstride, int key_digits, const ModQ m, u64 *const *dst,
+                                         const i64 *astride) {
+    if constexpr (!LIMB)
+        mac_span<V, P, Q1, 0>(dsrc, dstride, esrc, estride, n, nd, my_digit, krow, key_pstride, key_digits, m, dst, astride);
+    else if (key_limb_bits(m.q, key_digits) == 27)
+        mac_span<V, P, Q1, 2>(dsrc, dstride, esrc, estride, n, nd, my_digit, krow, key_pstride, key_digits, m, dst, astride);
+    else
+        mac_span<V, P, Q1, 1>(dsrc, dstride, esrc, estride, n, nd, my_digit, krow, key_pstride, key_digits, m, dst, astride);
+}
+
 // Batch elements b_first + g P + p (p < P) of group g; blockIdx.x runs over
 // groups fastest, then coefficient chunks, then accumulator limbs, so that
 // blocks that share key rows run next to each other.
-template <bool Q1, int P, int V>
-__global__ void __launch_bounds__(CKKS_MAC_MAX_THREADS) mac_kernel(MacArgs A, int b_first, int n_groups) {
+template <bool Q1, int P, int V, bool LIMB>
+__global__ void __launch_bounds__(CKKS_MAC_MAX_THREADS, CKKS_MAC_MINB) mac_kernel(MacArgs A, int b_first, int n_groups) {
     const int chunks = (A.N + blockDim.x * V - 1) / (blockDim.x * V);
     int bid = blockIdx.x;
     const int g = bid % n_groups;
@@ -625,18 +739,19 @@ __global__ void __launch_bounds__(CKKS_MAC_MAX_THREADS) mac_kernel(MacArgs A, in
         estr[p] = A.ext.pstride;
         astr[p] = A.acc.pstride;
     }
-    mac_span<V, P, Q1>(ds, dstr, es, estr, A.n, A.n_digits, isq ? x / A.alpha : -1, A.keys + (i64)prime * A.N + e,
+    mac_limb<V, P, Q1, LIMB>(ds, dstr, es, estr, A.n, A.n_digits, isq ? x / A.alpha : -1, A.keys + (i64)prime * A.N + e,
                        A.key_pstride, A.key_digits, A.mods[prime], os, astr);
 }
 
 template <int P, int V>
 static void launch_mac_part(const Context &C, const MacArgs &A, int b_first, int n_groups, cudaStream_t st) {
-    const int thr = C.tune_mac_threads;
+    const int thr = std::min(C.tune_mac_threads, CKKS_MAC_MAX_THREADS);
     const int chunks = (A.N + thr * V - 1) / (thr * V);
     const long long blocks = (long long)chunks * (A.level + A.K) * n_groups;
     count_kernel(C);
-    if (C.q1()) mac_kernel<true, P, V><<<(unsigned)blocks, thr, 0, st>>>(A, b_first, n_groups);
-    else mac_kernel<false, P, V><<<(unsigned)blocks, thr, 0, st>>>(A, b_first, n_groups);
+    if (!C.limbs30) mac_kernel<false, P, V, false><<<(unsigned)blocks, thr, 0, st>>>(A, b_first, n_groups);
+    else if (C.q1()) mac_kernel<true, P, V, true><<<(unsigned)blocks, thr, 0, st>>>(A, b_first, n_groups);
+    else mac_kernel<false, P, V, true><<<(unsigned)blocks, thr, 0, st>>>(A, b_first, n_groups);
 }
 
 cudaError_t launch_mac(const Context &C, const MacArgs &A, cudaStream_t st) {
@@ -658,8 +773,8 @@ cudaError_t launch_mac(const Context &C, const MacArgs &A, cudaStream_t st) {
 // job [, job2], x), ordered by prime so that neighbouring blocks read the
 // same key rows; blockIdx.y = coefficient chunk. P = 2: the target pairs
 // two products of the same shape (job2), which share the key loads.
-template <bool Q1, int P, int V>
-__global__ void __launch_bounds__(CKKS_MAC_MAX_THREADS) mac_table_kernel(const MacJob *jobs, const MacTarget *targets,
+template <bool Q1, int P, int V, bool LIMB>
+__global__ void __launch_bounds__(CKKS_MAC_MAX_THREADS, CKKS_MAC_MINB) mac_table_kernel(const MacJob *jobs, const MacTarget *targets,
                                                                          const u64 *keys, i64 key_pstride,
                                                                          int key_digits, int alpha, int L, int N,
                                                                          const ModQ *mods) {
@@ -684,7 +799,7 @@ __global__ void __launch_bounds__(CKKS_MAC_MAX_THREADS) mac_table_kernel(const M
         estr[p] = J.estride;
         astr[p] = J.astride;
     }
-    mac_span<V, P, Q1>(ds, dstr, es, estr, J0.n, J0.nd, isq ? x / alpha : -1, keys + (i64)prime * N + e, key_pstride,
+    mac_limb<V, P, Q1, LIMB>(ds, dstr, es, estr, J0.n, J0.nd, isq ? x / alpha : -1, keys + (i64)prime * N + e, key_pstride,
                        key_digits, mods[prime], os, astr);
 }
 
@@ -692,18 +807,18 @@ template <int P, int V>
 static cudaError_t launch_mac_table_part(const Context &C, const MacJob *jobs, const MacTarget *targets, int n,
                                          const u64 *keys, cudaStream_t st) {
     if (n <= 0) return cudaSuccess;
-    const int thr = C.tune_mac_threads;
+    const int thr = std::min(C.tune_mac_threads, CKKS_MAC_MAX_THREADS);
     const int chunks = (C.N + thr * V - 1) / (thr * V);
     if (chunks > 65535) return cudaErrorInvalidValue;
     count_kernel(C);
     dim3 grid((unsigned)n, (unsigned)chunks);
     const i64 kps = (i64)(C.L + C.K) * C.N;
-    if (C.q1())
-        mac_table_kernel<true, P, V><<<grid, thr, 0, st>>>(jobs, targets, keys, kps, C.dnum, C.alpha, C.L, C.N,
-                                                           C.d_mods);
-    else
-        mac_table_kernel<false, P, V><<<grid, thr, 0, st>>>(jobs, targets, keys, kps, C.dnum, C.alpha, C.L, C.N,
-                                                            C.d_mods);
+#define CKKS_MACT(Q, LB) \
+    mac_table_kernel<Q, P, V, LB><<<grid, thr, 0, st>>>(jobs, targets, keys, kps, C.dnum, C.alpha, C.L, C.N, C.d_mods)
+    if (!C.limbs30) CKKS_MACT(false, false);
+    else if (C.q1()) CKKS_MACT(true, true);
+    else CKKS_MACT(false, true);
+#undef CKKS_MACT
     return cudaGetLastError();
 }
 
@@ -788,20 +903,25 @@ cudaError_t launch_rschain_table(const Context &C, const RsJob *jobs, int n_jobs
 // keys
 // ---------------------------------------------------------------------------
 // In place: v <- v * fold[x] R^-1, fold = P^-1 R^2 on Q limbs, R^2 on P
-// limbs, giving the Montgomery form of P^-1 ek (Q limbs) or ek (P limbs).
+// limbs, giving the Montgomery form of P^-1 ek (Q limbs) or ek (P limbs);
+// with `limbs`, each word then holds its own two limbs (the key MAC's FORM 1
+// and 2).
 __global__ void __launch_bounds__(kThreads) keyprep_kernel(u64 *keys, i64 n_rows, int n_primes, int N,
-                                                           const ModQ *mods, const u64 *fold) {
+                                                           const ModQ *mods, const u64 *fold, int key_digits,
+                                                           bool limbs) {
     const i64 gid = (i64)blockIdx.x * blockDim.x + threadIdx.x;
     if (gid >= n_rows * N) return;
     const int x = (int)((gid / N) % n_primes);
-    keys[gid] = mont_mul(keys[gid], fold[x], mods[x]);
+    const u64 v = mont_mul(keys[gid], fold[x], mods[x]);
+    if (limbs) keys[gid] = key_limb_bits(mods[x].q, key_digits) == 27 ? pack_limbs<27>(v) : pack_limbs<30>(v);
+    else keys[gid] = v;
 }
 
 cudaError_t launch_keyprep(const Context &C, u64 *keys, long long n_rows, cudaStream_t st) {
     i64 total = n_rows * C.N;
     count_kernel(C);
     keyprep_kernel<<<(unsigned)((total + kThreads - 1) / kThreads), kThreads, 0, st>>>(
-        keys, n_rows, C.L + C.K, C.N, C.d_mods, C.d_keyfold);
+        keys, n_rows, C.L + C.K, C.N, C.d_mods, C.d_keyfold, C.dnum, C.limbs30);
     return cudaGetLastError();
 }
 

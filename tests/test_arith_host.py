@@ -1,8 +1,8 @@
 """The kernels' modular arithmetic (csrc/arith.cuh) compiled as plain C++ and
 compared with 128-bit integers at the edges of its ranges: products by a
 constant with both companions (operands up to the stated bounds, constants
-next to 0, q/2 and q, primes of every size and of the form h 2^32 + 1) and
-the reductions of small multiples of q."""
+next to 0, q/2 and q, primes of every size and of the form h 2^32 + 1), the
+reductions of small multiples of q, and the dot products by limbs."""
 import os
 import shutil
 import subprocess
@@ -31,6 +31,19 @@ template <bool Q1> static void products(u64 q, u64 w, i64 x, int m) {
     const Shoup h = make_shoup_halved(w, q);
     const i64 t = (i64)remainder_mad<Q1, 2>((u64)y, h.w, quot_halved((u64)y, h.wp), 0ull - 2 * q, 0);
     check((double)(t < 0 ? -t : t) < 2.25 * (double)q && smod(t, q) == smod((i128)smod(y, q) * w, q), "halved", q, w, y);
+}
+template <int SB> static void dots(u64 q, u64 qb, int terms, std::mt19937_64 &g) {
+    DotLimbs d;
+    d.zero();
+    u128 sum = 0;
+    for (int i = 0; i < terms; ++i) {
+        const u64 a = g() % 3 ? q - 1 - g() % 5 % q : g() % q, b = g() % 3 ? qb - 1 - g() % 5 % qb : g() % qb;
+        d.mac(split_limbs<SB>(a), packed_limbs(pack_limbs<SB>(b)));
+        sum += (u128)a * b;
+    }
+    u64 hi, lo;
+    d.value<SB>(hi, lo);
+    check(hi == (u64)(sum >> 64) && lo == (u64)sum, "dot", q, qb, terms);
 }
 int main() {
     std::mt19937_64 g(20);
@@ -65,6 +78,24 @@ int main() {
             const i128 v = (i128)((((u128)g() << 64) | g()) % ((u128)span * 2 * q - 1)) - ((i128)span * q - 1);
             const u64 r = small_prime(q) ? canonical<true>((u64)(i64)v, q, c) : canonical<false>((u64)(i64)v, q, c);
             check(r == smod(v, q), "canonical", q, w, (i64)v);
+        }
+        for (int it = 0; it < 2000 && q < (1ull << 60); ++it) {
+            const u64 qb = it % 2 ? q : (1ull << 60) - 131071;
+            dots<30>(q, qb, 1 + it % kLimbTerms30, g);
+            if (small_prime(q)) dots<27>(q, q, 1 + it % kLimbTerms27, g);
+            // fold: 7 terms, then 6 at a time
+            DotLimbs d;
+            d.zero();
+            u128 sum = 0;
+            for (int i = 0; i < 7 + 6 * (it % 5); ++i) {
+                const u64 a = q - 1 - g() % 7 % q, b = it % 3 ? q - 1 : g() % q;
+                d.mac(split_limbs<30>(a), split_limbs<30>(b));
+                sum = (sum + (u128)a * b) % q;
+                if (i >= 6 && (i - 6) % 6 == 0) d.fold(q, c);
+            }
+            u64 hi, lo;
+            d.value<30>(hi, lo);
+            check(hi < q && (u64)((((u128)hi << 64) | lo) % q) == (u64)sum, "fold", q, it, 0);
         }
     }
     printf("bad %ld\n", bad);
