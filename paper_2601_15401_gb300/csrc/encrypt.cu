@@ -64,24 +64,8 @@ __global__ void crt2_kernel(const u64 *P, double *out, int limbs, int N, u64 q0,
     }
 }
 
-struct Src4 {
-    const i64 *p[4];
-};
-
-// signed [4][batch][N] (v, e0, e1, m) -> W[b][p][x][N] residues, x < level;
-// blockIdx.y = b * 4 + p
-__global__ void signed4_kernel(Src4 src, u64 *W, int level, int N, const ModQ *mods) {
-    const i64 gid = (i64)blockIdx.x * blockDim.x + threadIdx.x;
-    if (gid >= (i64)level * N) return;
-    const int b = blockIdx.y / 4, p = blockIdx.y % 4;
-    const int x = (int)(gid / N), i = (int)(gid % N);
-    const i64 v = src.p[p][(i64)b * N + i];
-    const u64 q = mods[x].q;
-    const u64 r = v >= 0 ? ((u64)v) % q : ((u64)(-v)) % q;
-    W[((i64)blockIdx.y * level) * N + gid] = (v >= 0 || r == 0) ? r : q - r;
-}
-
-// c0 = V pk0 + E0 + M, c1 = V pk1 + E1 for every batch element (blockIdx.y)
+// c0 = V pk0 + T, c1 = V pk1 + E1 for every batch element (blockIdx.y), with
+// T the transform of e0 + m
 __global__ void enc_batch_kernel(const u64 *W, const u64 *pk, i64 pk_pstride, u64 *out, i64 out_bstride,
                                  i64 out_pstride, int level, int N, const ModQ *mods, const u64 *r2) {
     const i64 gid = (i64)blockIdx.x * blockDim.x + threadIdx.x;
@@ -91,10 +75,11 @@ __global__ void enc_batch_kernel(const u64 *W, const u64 *pk, i64 pk_pstride, u6
     const ModQ m = mods[x];
     const u64 q = m.q;
     const i64 plane = (i64)level * N;
-    const u64 *w = W + (i64)b * 4 * plane + gid;  // V, E0, E1, M
+    const u64 *w = W + (i64)b * 3 * plane + gid;  // V, T, E1
     u64 *c0 = out + (i64)b * out_bstride + gid, *c1 = c0 + out_pstride;
-    *c0 = add_mod(add_mod(mulmod_full(w[0], pk[gid], m, r2[x]), w[plane], q), w[3 * plane], q);
-    *c1 = add_mod(mulmod_full(w[0], pk[pk_pstride + gid], m, r2[x]), w[2 * plane], q);
+    const u64 v = mont_mul(w[0], r2[x], m);  // V R, so that one REDC per product is left
+    *c0 = add_mod(mont_mul(v, pk[gid], m), w[plane], q);
+    *c1 = add_mod(mont_mul(v, pk[pk_pstride + gid], m), w[2 * plane], q);
 }
 
 // P[b][x] = C0 + C1 S over the lowest `limbs` limbs of every batch element
@@ -111,12 +96,6 @@ __global__ void dec_batch_kernel(const u64 *ct, i64 bstride, i64 pstride, const 
 
 unsigned blocks(i64 n) { return (unsigned)((n + kThr - 1) / kThr); }
 
-// NTT of `limbs` limbs in place (prime index = limb index)
-cudaError_t ntt_limbs(const Context &C, u64 *buf, int limbs, cudaStream_t st) {
-    LimbView v{buf, 0, (i64)limbs * C.N};
-    return transform_plain(C, true, 1, 1, limbs, v, v, st);
-}
-
 u64 host_inv(u64 a, u64 q) {
     unsigned __int128 r = 1, b = a % q;
     u64 e = q - 2;
@@ -130,7 +109,7 @@ u64 host_inv(u64 a, u64 q) {
 
 size_t enc_batch_ws(const Context &C, uint32_t level, uint32_t batch) {
     const uint32_t chunk = std::min<uint32_t>(16383u, 65535u / (4u * level));
-    return (size_t)std::min(batch, chunk) * 4 * level * C.N * sizeof(u64);
+    return (size_t)std::min(batch, chunk) * 4 * level * C.N * sizeof(u64);  // three planes are used
 }
 
 size_t dec_batch_ws(const Context &C, uint32_t batch) {
@@ -166,10 +145,8 @@ int ckks_public_key(ckks_context *ctx, const int64_t *s, const uint64_t *a, cons
     cudaStream_t st = (cudaStream_t)stream;
     const size_t plane = (size_t)(C.L + C.K) * C.N;
     u64 *S = (u64 *)workspace, *E = S + plane;
-    cudaError_t err = launch_signed_to_res(C, (const long long *)s, S, st);
-    if (err == cudaSuccess) err = launch_signed_to_res(C, (const long long *)e, E, st);
-    if (err == cudaSuccess) err = ntt_limbs(C, S, C.L, st);
-    if (err == cudaSuccess) err = ntt_limbs(C, E, C.L, st);
+    const u64 *sa[2] = {(const u64 *)s, (const u64 *)e}, *sb[2] = {nullptr, nullptr};
+    cudaError_t err = transform_signed(C, 1, 2, C.L, sa, sb, LimbView{S, 0, (i64)plane}, st);
     if (err == cudaSuccess) {
         count_kernel(C);
         pk_kernel<<<blocks((i64)C.L * C.N), kThr, 0, st>>>(S, E, (const u64 *)a, (u64 *)pk, C.L, C.N, C.d_mods, C.d_r2);
@@ -211,15 +188,13 @@ int ckks_encrypt_batch(ckks_context *ctx, const int64_t *m, const int64_t *v, co
     cudaError_t err = cudaSuccess;
     for (uint32_t b0 = 0; b0 < batch && err == cudaSuccess; b0 += chunk) {
         const uint32_t cb = std::min(chunk, batch - b0);
-        Src4 src{{(const i64 *)v + b0 * N, (const i64 *)e0 + b0 * N, (const i64 *)e1 + b0 * N,
-                  (const i64 *)m + b0 * N}};
-        count_kernel(C);
-        signed4_kernel<<<dim3(blocks((i64)level * N), cb * 4), kThr, 0, st>>>(src, W, (int)level, C.N, C.d_mods);
-        err = cudaGetLastError();
-        if (err == cudaSuccess) {
-            LimbView w{W, 4 * (i64)level * N, (i64)level * N};
-            err = transform_plain(C, true, (int)cb, 4, (int)level, w, w, st);
-        }
+        // V = NTT(v), T = NTT(e0 + m), E1 = NTT(e1): the signed inputs are
+        // reduced into every limb as the transform loads them, and e0 and m
+        // take one transform together
+        const u64 *sa[3] = {(const u64 *)v + b0 * N, (const u64 *)e0 + b0 * N, (const u64 *)e1 + b0 * N};
+        const u64 *sb[3] = {nullptr, (const u64 *)m + b0 * N, nullptr};
+        LimbView w{W, 3 * (i64)level * N, (i64)level * N};
+        err = transform_signed(C, (int)cb, 3, (int)level, sa, sb, w, st);
         if (err == cudaSuccess) {
             count_kernel(C);
             enc_batch_kernel<<<dim3(blocks((i64)level * N), cb), kThr, 0, st>>>(
@@ -269,8 +244,8 @@ int ckks_decrypt_batch(ckks_context *ctx, const ckks_tuple *ct, uint32_t batch, 
     const int limbs = ct[0].level >= 2 ? 2 : 1;
     const i64 N = C.N;
     u64 *S = (u64 *)workspace, *P = S + (size_t)(C.L + C.K) * N;
-    cudaError_t err = launch_signed_to_res(C, (const long long *)s, S, st);
-    if (err == cudaSuccess) err = ntt_limbs(C, S, limbs, st);
+    const u64 *sa[1] = {(const u64 *)s}, *sb[1] = {nullptr};
+    cudaError_t err = transform_signed(C, 1, 1, limbs, sa, sb, LimbView{S, 0, (i64)limbs * N}, st);
     if (err == cudaSuccess) {
         count_kernel(C);
         dec_batch_kernel<<<dim3(blocks((i64)limbs * N), batch), kThr, 0, st>>>(

@@ -107,6 +107,24 @@ cudaError_t transform_plain(const Context &C, bool fwd, int B, int polys, int le
     return ntt_transform(C, fwd, J, L, S, nullptr, st);
 }
 
+// Forward transform of signed integer polynomials into limbs [0, level):
+// polynomial p of batch element b is sa[p][b N ..] (+ sb[p][b N ..]).
+cudaError_t transform_signed(const Context &C, int B, int polys, int level, const u64 *const *sa,
+                             const u64 *const *sb, LimbView out, cudaStream_t st) {
+    LimbJobs J = jobs(B, polys, level);
+    LoadSpec L{};
+    L.mode = LD_SIGNED;
+    L.one = C.d_one;
+    for (int p = 0; p < polys; ++p) {
+        L.sa[p] = sa[p];
+        L.sb[p] = sb[p];
+    }
+    StoreSpec S{};
+    S.mode = ST_REDUCE;
+    S.dst = out;
+    return ntt_transform(C, true, J, L, S, nullptr, st);
+}
+
 // Algorithm 1 on `polys` polynomials: in (level limbs, NTT) -> out (level - mu).
 static cudaError_t multi_rs_alg1(const Context &C, Ws &ws, int B, int polys, int level, int mu, LimbView in,
                                  LimbView out, cudaStream_t st) {

@@ -29,6 +29,9 @@ cudaError_t run_tensor(const Context &C, int B, int level, int m, const LimbView
 cudaError_t transform_plain(const Context &C, bool fwd, int B, int polys, int level, LimbView in, LimbView out,
                             cudaStream_t st);
 
+cudaError_t transform_signed(const Context &C, int B, int polys, int level, const u64 *const *sa,
+                             const u64 *const *sb, LimbView out, cudaStream_t st);
+
 // scale of a plan's output from the inputs' scales (Section V: each
 // rescale divides by the prime it removes)
 double plan_scale(const Context &C, const Plan &P, int level, const double *scales);

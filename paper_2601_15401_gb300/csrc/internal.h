@@ -13,7 +13,8 @@ namespace ckks {
 // LD_ADD     a + b
 // LD_EQ17    sum_t g_t T_t, or g_self a - sum_t g_t T_t (Eq. 17)
 // LD_BCONVK  sum_i z_i [p_i^-1]_q (scaled BConv of Eq. 12; z = b)
-enum LoadMode { LD_PLAIN = 0, LD_ADD = 1, LD_EQ17 = 2, LD_BCONVK = 3 };
+// LD_SIGNED  a (+ b): signed 64-bit integers, the same for every limb
+enum LoadMode { LD_PLAIN = 0, LD_ADD = 1, LD_EQ17 = 2, LD_BCONVK = 3, LD_SIGNED = 4 };
 // ST_REDUCE  canonical value
 // ST_LAZY    lazy value (between the two phases)
 // ST_SCALE   v * c (Shoup constant per launch limb)
@@ -49,6 +50,10 @@ struct LoadSpec {
     const ModQ *mods;   // LD_BCONVK
     const u64 *cK;      // LD_BCONVK: [prime][64] Montgomery constants
     int K;
+    // LD_SIGNED: polynomial p of batch element b is sa[p][b N ..] (+ sb[p][b N ..]
+    // where set); `one` [prime] reduces
+    const u64 *sa[3], *sb[3];
+    const Shoup *one;
 };
 
 struct StoreSpec {

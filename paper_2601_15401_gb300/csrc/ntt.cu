@@ -119,6 +119,7 @@ cudaError_t launch_ntt_phase(const Context &C, bool fwd, bool cols, const LimbJo
     // integer work: one Shoup product per butterfly (log2 n stages of N / 2
     // per limb) plus the Shoup products of the fused load / store
     double ops = jobs_d * (double)C.N * 0.5 * logn;
+    if (L.mode == LD_SIGNED) ops += jobs_d * (double)C.N;
     if (L.mode == LD_EQ17) ops += jobs_d * (double)C.N * (L.mu + L.with_self);
     if (S.mode == ST_SCALE || S.mode == ST_MODDOWN || S.mode == ST_MRS) ops += jobs_d * (double)C.N;
     ProfScope ps(C, fwd ? (cols ? KC_NTT_FWD_COLS : KC_NTT_FWD_BLOCKS) : (cols ? KC_NTT_INV_COLS : KC_NTT_INV_BLOCKS),

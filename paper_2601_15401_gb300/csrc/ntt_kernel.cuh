@@ -122,6 +122,11 @@ __device__ __forceinline__ LoadCtx make_load(const LoadSpec &L, const LimbJobs &
     if (L.mode == LD_EQ17 || L.mode == LD_BCONVK) c.b = L.b.ptr + (i64)b * L.b.bstride + (i64)p * L.b.pstride;
     if (L.mode == LD_EQ17) c.g = L.g + (i64)l * (L.mu + 1);
     if (L.mode == LD_BCONVK) c.cK = L.cK + (i64)prime * CKKS_MAX_PRIMES;
+    if (L.mode == LD_SIGNED) {
+        c.a = L.sa[p] + (i64)b * N;
+        c.b = L.sb[p] ? L.sb[p] + (i64)b * N : nullptr;
+        c.g = L.one + prime;
+    }
     return c;
 }
 
@@ -189,6 +194,20 @@ __device__ __forceinline__ u64 eq17_sub(u64 r, u64 s, u64 q) {
     return SMALL ? r - s : sub_mod(lift_sign(r, q), s, q);
 }
 
+// any signed 64-bit integer mod q (canonical); `one`: the constant 1
+template <bool Q1>
+__device__ __forceinline__ u64 signed_mod(u64 v, Shoup one, u64 q) {
+    // beyond the product's range (|v| < 2^63 - 2^33) v = 4 (v >> 2) + (v & 3)
+    const bool far = (i64)(v ^ (v << 1)) < 0;  // |v| >= 2^62
+    u64 r = shoup_t<Q1>(far ? (u64)((i64)v >> 2) : v, one.w, one.wp, q);
+    if (far) {
+        r = add_mod(r, r, q);
+        r = add_mod(r, r, q);
+        r = add_mod(r, shoup_t<Q1>(v & 3, one.w, one.wp, q), q);
+    }
+    return r;
+}
+
 template <int LM, bool SMALL, bool Q1>
 __device__ __forceinline__ u64 load_elem(const LoadCtx &c, int e) {
     const u64 q = c.m.q;
@@ -209,6 +228,11 @@ __device__ __forceinline__ u64 load_elem(const LoadCtx &c, int e) {
         acc.zero();
         for (int i = 0; i < c.K; ++i) acc.mac(c.b[(i64)i * c.N + e], c.cK[i]);
         return redc_t<Q1>(acc.hi, acc.lo, c.m);
+    }
+    case LD_SIGNED: {
+        const Shoup one = *c.g;
+        const u64 v = signed_mod<Q1>(c.a[e], one, q);
+        return c.b ? add_mod(v, signed_mod<Q1>(c.b[e], one, q), q) : v;
     }
     default:
         return c.a[e];
@@ -711,6 +735,8 @@ static inline cudaError_t dispatch_cols(const NttPhase &P, const LimbJobs *J, co
         CKKS_MODES(LD_PLAIN, ST_LAZY) CKKS_LAUNCH(LG, LG2, COLS, LD_PLAIN, ST_LAZY, CKKS_NTT_COL_MINB, Q1);
         CKKS_MODES(LD_EQ17, ST_LAZY) CKKS_LAUNCH(LG, LG2, COLS, LD_EQ17, ST_LAZY, CKKS_NTT_COL_WIDE_MINB, Q1);
         CKKS_MODES(LD_BCONVK, ST_LAZY) CKKS_LAUNCH(LG, LG2, COLS, LD_BCONVK, ST_LAZY, CKKS_NTT_COL_WIDE_MINB, Q1);
+        if constexpr (!TABLE)
+            CKKS_MODES(LD_SIGNED, ST_LAZY) CKKS_LAUNCH(LG, LG2, COLS, LD_SIGNED, ST_LAZY, CKKS_NTT_COL_WIDE_MINB, Q1);
     } else {
         CKKS_MODES(LD_PLAIN, ST_SCALE) CKKS_LAUNCH(LG, LG2, COLS, LD_PLAIN, ST_SCALE, CKKS_NTT_COL_MINB, Q1);
         CKKS_MODES(LD_PLAIN, ST_MODDOWN) CKKS_LAUNCH(LG, LG2, COLS, LD_PLAIN, ST_MODDOWN, CKKS_NTT_COL_WIDE_MINB, Q1);
@@ -755,6 +781,8 @@ static inline cudaError_t dispatch_whole_n(const NttPhase &P, const LimbJobs *J,
                                            const LoadSpec &L, const StoreSpec &S, const PhaseLaunch &G) {
     if constexpr (FWD) {
         CKKS_MODES(LD_PLAIN, ST_REDUCE) CKKS_LAUNCH(LG, 0, WHOLE, LD_PLAIN, ST_REDUCE, 2, false);
+        if constexpr (!TABLE)
+            CKKS_MODES(LD_SIGNED, ST_REDUCE) CKKS_LAUNCH(LG, 0, WHOLE, LD_SIGNED, ST_REDUCE, 2, false);
         CKKS_MODES(LD_EQ17, ST_REDUCE) CKKS_LAUNCH(LG, 0, WHOLE, LD_EQ17, ST_REDUCE, 2, false);
         CKKS_MODES(LD_EQ17, ST_MRS) CKKS_LAUNCH(LG, 0, WHOLE, LD_EQ17, ST_MRS, 2, false);
         CKKS_MODES(LD_BCONVK, ST_ADDSUB) CKKS_LAUNCH(LG, 0, WHOLE, LD_BCONVK, ST_ADDSUB, 2, false);
