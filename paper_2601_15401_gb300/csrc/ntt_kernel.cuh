@@ -208,6 +208,26 @@ __device__ __forceinline__ u64 signed_mod(u64 v, Shoup one, u64 q) {
     return r;
 }
 
+// out[u] = sum_i z_i[u DIST] c_i R^-1 mod q over the K limbs z_i (N apart) of the
+// P basis, for G elements whose loads are in flight together. The sum of the
+// P primes is below 2^64 (context check), so the high word stays below q.
+template <int G, int DIST, bool Q1>
+__device__ __forceinline__ void scaled_bconv(u64 (&out)[G], const u64 *z, int N, const u64 *cK, int K, ModQ m) {
+    Acc128Lazy acc[G];
+#pragma unroll
+    for (int u = 0; u < G; ++u) acc[u].zero();
+    for (int i = 0; i < K; ++i) {
+        const u64 c = cK[i];
+        u64 v[G];
+#pragma unroll
+        for (int u = 0; u < G; ++u) v[u] = z[(i64)i * N + u * DIST];
+#pragma unroll
+        for (int u = 0; u < G; ++u) acc[u].mac(v[u], c);
+    }
+#pragma unroll
+    for (int u = 0; u < G; ++u) out[u] = redc_t<Q1>(acc[u].hi, acc[u].lo, m);
+}
+
 template <int LM, bool SMALL, bool Q1>
 __device__ __forceinline__ u64 load_elem(const LoadCtx &c, int e) {
     const u64 q = c.m.q;
@@ -224,10 +244,9 @@ __device__ __forceinline__ u64 load_elem(const LoadCtx &c, int e) {
         return s;
     }
     case LD_BCONVK: {
-        Acc128Lazy acc;  // sum of the P primes < 2^64 (context check)
-        acc.zero();
-        for (int i = 0; i < c.K; ++i) acc.mac(c.b[(i64)i * c.N + e], c.cK[i]);
-        return redc_t<Q1>(acc.hi, acc.lo, c.m);
+        u64 r[1];
+        scaled_bconv<1, 1, Q1>(r, c.b + e, c.N, c.cK, c.K, c.m);
+        return r[0];
     }
     case LD_SIGNED: {
         const Shoup one = *c.g;
@@ -252,11 +271,9 @@ __device__ __forceinline__ void store_elem(const StoreCtx &c, int e, u64 v, bool
         break;
     case ST_MODDOWN: {
         // c* = v N^-1 - sum_i z_i [p_i^-1 R]_q  (Eq. 5 with Eq. 11 / 12)
-        u64 x = shoup_t<Q1>(v, c.c.w, c.c.wp, q);
-        Acc128Lazy acc;  // sum of the P primes < 2^64 (context check)
-        acc.zero();
-        for (int i = 0; i < c.K; ++i) acc.mac(c.aux[(i64)i * c.N + e], c.cK[i]);
-        c.dst[e] = sub_mod(x, redc_t<Q1>(acc.hi, acc.lo, c.m), q);
+        u64 r[1];
+        scaled_bconv<1, 1, Q1>(r, c.aux + e, c.N, c.cK, c.K, c.m);
+        c.dst[e] = sub_mod(shoup_t<Q1>(v, c.c.w, c.c.wp, q), r[0], q);
         break;
     }
     case ST_MRS:
@@ -290,6 +307,11 @@ __device__ __forceinline__ void store_elem(const StoreCtx &c, int e, u64 v, bool
 //            (a block phase with N1 = 1).
 enum Shape { COLS = 0, BLOCKS = 1, WHOLE = 2 };
 constexpr int kWholeMax = 12;  // log2 of the largest limb one CTA transforms
+
+// elements whose sums over the K z-limbs run together
+#ifndef CKKS_NTT_MODDOWN_GROUP
+#define CKKS_NTT_MODDOWN_GROUP 4
+#endif
 
 template <int LOGN, int LOGN2, int SH>
 struct Geo {
@@ -392,6 +414,15 @@ __device__ __forceinline__ void load_set(u64 (&x)[EL], const LoadCtx &lc, int e)
             for (int k = 0; k < EL; ++k)
                 x[k] = eq17_sub<SMALL>(shoup_signed<Q1>(lc.a[e + k * DIST], g.w, g.wp, q), x[k], q);
         }
+    } else if constexpr (LM == LD_BCONVK) {
+        constexpr int G = EL >= CKKS_NTT_MODDOWN_GROUP ? CKKS_NTT_MODDOWN_GROUP : EL;
+#pragma unroll
+        for (int k0 = 0; k0 < EL; k0 += G) {
+            u64 r[G];
+            scaled_bconv<G, DIST, Q1>(r, lc.b + e + k0 * DIST, lc.N, lc.cK, lc.K, lc.m);
+#pragma unroll
+            for (int u = 0; u < G; ++u) x[k0 + u] = r[u];
+        }
     } else {
 #pragma unroll
         for (int k = 0; k < EL; ++k) x[k] = load_elem<LM, SMALL, Q1>(lc, e + k * DIST);
@@ -404,25 +435,14 @@ template <int EL, int DIST, int SM, bool FWD, bool SMALL, bool Q1>
 __device__ __forceinline__ void store_set(const u64 (&x)[EL], const StoreCtx &sc, int e) {
     if constexpr (SM == ST_MODDOWN) {
         const u64 q = sc.m.q;
-        constexpr int G4 = EL >= 4 ? 4 : EL;
+        constexpr int G = EL >= CKKS_NTT_MODDOWN_GROUP ? CKKS_NTT_MODDOWN_GROUP : EL;
 #pragma unroll
-        for (int k0 = 0; k0 < EL; k0 += G4) {
-            Acc128Lazy acc[G4];  // sum of the P primes < 2^64 (context check)
+        for (int k0 = 0; k0 < EL; k0 += G) {
+            u64 r[G];
+            scaled_bconv<G, DIST, Q1>(r, sc.aux + e + k0 * DIST, sc.N, sc.cK, sc.K, sc.m);
 #pragma unroll
-            for (int u = 0; u < G4; ++u) acc[u].zero();
-            for (int i = 0; i < sc.K; ++i) {
-                const u64 c = sc.cK[i];
-                const u64 *zi = sc.aux + (i64)i * sc.N + e;
-                u64 z[G4];
-#pragma unroll
-                for (int u = 0; u < G4; ++u) z[u] = zi[(k0 + u) * DIST];
-#pragma unroll
-                for (int u = 0; u < G4; ++u) acc[u].mac(z[u], c);
-            }
-#pragma unroll
-            for (int u = 0; u < G4; ++u)
-                sc.dst[e + (k0 + u) * DIST] = sub_mod(shoup_t<Q1>(x[k0 + u], sc.c.w, sc.c.wp, q),
-                                                      redc_t<Q1>(acc[u].hi, acc[u].lo, sc.m), q);
+            for (int u = 0; u < G; ++u)
+                sc.dst[e + (k0 + u) * DIST] = sub_mod(shoup_t<Q1>(x[k0 + u], sc.c.w, sc.c.wp, q), r[u], q);
         }
     } else {
 #pragma unroll
@@ -448,8 +468,8 @@ __device__ __forceinline__ void run_passes(const Lane &ln, u64 q, const LoadCtx 
         constexpr int P = FWD ? I : NP - 1 - I;
         constexpr int R = Pass<LOGN, P>::len, E0 = Pass<LOGN, P>::start, EL = 1 << R;
         constexpr bool first = I == 0, last = I == NP - 1;
-        constexpr bool gin = first && PassAccess<LOGN, SH, P>::direct;
-        constexpr bool gout = last && PassAccess<LOGN, SH, P>::direct;
+        constexpr bool gin = first && LM >= 0 && PassAccess<LOGN, SH, P>::direct;
+        constexpr bool gout = last && SM >= 0 && PassAccess<LOGN, SH, P>::direct;
         constexpr int t_min = G::n >> (E0 + R);
         constexpr int iters = (G::n >> R) / G::sets;
         u64 x[iters][EL];
@@ -574,7 +594,13 @@ __device__ __forceinline__ void phase_tile(u64 *sm, const NttPhase &P, const ulo
         const int e0 = b0 << LOGN;
         // shared offset of word idx of the warp's blocks
         auto woff = [](int idx) { return (idx >> LOGN) * G::unit + G::off(idx & (n - 1)); };
-        if constexpr (!PassAccess<LOGN, SH, PF>::direct) {
+        // run-time modes (N <= 2^8): both sides staged, one element at a time
+        constexpr bool RT = LM < 0;
+        if constexpr (RT) {
+#pragma unroll 1
+            for (int idx = lane; idx < W * T; idx += T)
+                if (idx < words) wsm[woff(idx)] = load_elem<LM, SMALL, Q1>(lc, e0 + idx);
+        } else if constexpr (!PassAccess<LOGN, SH, PF>::direct) {
             // coalesced global -> shared with the fused load, U loads in flight
 #pragma unroll
             for (int i0 = 0; i0 < W; i0 += U) {
@@ -592,7 +618,11 @@ __device__ __forceinline__ void phase_tile(u64 *sm, const NttPhase &P, const ulo
             }
         }
         run_passes<LOGN, LOGN2, FWD, SH, LM, SM, SMALL, Q1, 0>(ln, q, lc, sc, P.N1);
-        if constexpr (!PassAccess<LOGN, SH, PL>::direct) {
+        if constexpr (RT) {
+#pragma unroll 1
+            for (int idx = lane; idx < W * T; idx += T)
+                if (idx < words) store_elem<SM, SMALL, Q1>(sc, e0 + idx, wsm[woff(idx)], FWD);
+        } else if constexpr (!PassAccess<LOGN, SH, PL>::direct) {
             // shared -> global with the fused store (coalesced); a store that
             // reads an aux limb gathers U elements and their aux words first
 #pragma unroll
@@ -676,7 +706,14 @@ struct PhaseLaunch {
 #define CKKS_NTT_COL_MINB 4     // columns: 64 registers (871 vs 842 G butterflies/s with three CTAs, 736 with two)
 #endif
 #ifndef CKKS_NTT_COL_WIDE_MINB
-#define CKKS_NTT_COL_WIDE_MINB 3  // columns whose load or store sums over several limbs: 80 registers
+#define CKKS_NTT_COL_WIDE_MINB 4  // columns with an Eq. 17 or signed load (411 -> 393 us per k = 12, batch 8 launch
+                                  // against three CTAs)
+#endif
+#ifndef CKKS_NTT_COL_MODDOWN_MINB
+#define CKKS_NTT_COL_MODDOWN_MINB 3  // columns whose store sums over the K z-limbs: 80 registers
+#endif
+#ifndef CKKS_NTT_COL_BCONVK_MINB
+#define CKKS_NTT_COL_BCONVK_MINB 2  // columns whose load sums over the K z-limbs: 128 registers
 #endif
 #ifndef CKKS_NTT_BLOCK_MINB
 #define CKKS_NTT_BLOCK_MINB 2   // blocks: shared memory holds the twiddles of 16 warps per SM
@@ -734,12 +771,12 @@ static inline cudaError_t dispatch_cols(const NttPhase &P, const LimbJobs *J, co
     if constexpr (FWD) {
         CKKS_MODES(LD_PLAIN, ST_LAZY) CKKS_LAUNCH(LG, LG2, COLS, LD_PLAIN, ST_LAZY, CKKS_NTT_COL_MINB, Q1);
         CKKS_MODES(LD_EQ17, ST_LAZY) CKKS_LAUNCH(LG, LG2, COLS, LD_EQ17, ST_LAZY, CKKS_NTT_COL_WIDE_MINB, Q1);
-        CKKS_MODES(LD_BCONVK, ST_LAZY) CKKS_LAUNCH(LG, LG2, COLS, LD_BCONVK, ST_LAZY, CKKS_NTT_COL_WIDE_MINB, Q1);
+        CKKS_MODES(LD_BCONVK, ST_LAZY) CKKS_LAUNCH(LG, LG2, COLS, LD_BCONVK, ST_LAZY, CKKS_NTT_COL_BCONVK_MINB, Q1);
         if constexpr (!TABLE)
             CKKS_MODES(LD_SIGNED, ST_LAZY) CKKS_LAUNCH(LG, LG2, COLS, LD_SIGNED, ST_LAZY, CKKS_NTT_COL_WIDE_MINB, Q1);
     } else {
         CKKS_MODES(LD_PLAIN, ST_SCALE) CKKS_LAUNCH(LG, LG2, COLS, LD_PLAIN, ST_SCALE, CKKS_NTT_COL_MINB, Q1);
-        CKKS_MODES(LD_PLAIN, ST_MODDOWN) CKKS_LAUNCH(LG, LG2, COLS, LD_PLAIN, ST_MODDOWN, CKKS_NTT_COL_WIDE_MINB, Q1);
+        CKKS_MODES(LD_PLAIN, ST_MODDOWN) CKKS_LAUNCH(LG, LG2, COLS, LD_PLAIN, ST_MODDOWN, CKKS_NTT_COL_MODDOWN_MINB, Q1);
     }
     return cudaErrorInvalidValue;
 }

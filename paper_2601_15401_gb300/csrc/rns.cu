@@ -837,14 +837,21 @@ cudaError_t launch_mac_table(const Context &C, const MacJob *jobs, const MacTarg
 // u = 1..mu-1 and t < l-u (Eq. 6 applied inside Algorithm 1, step 2).
 // After it, limb t holds a^{(t),{l-1-t}}.
 // ---------------------------------------------------------------------------
-__device__ __forceinline__ void rschain_coeff(u64 *base, int N, int level, int mu, const ModQ *mods, const Shoup *one,
+// MU: mu at compile time (the limbs stay in registers), 0 = at run time (the
+// limbs live in a local-memory array).
+template <int MU>
+__device__ __forceinline__ void rschain_coeff(u64 *base, int N, int level, int mu_, const ModQ *mods, const Shoup *one,
                                               const Shoup *invq) {
+    const int mu = MU ? MU : mu_;
     const int l0 = level - mu;
-    u64 a[CKKS_MAX_PRIMES];
+    u64 a[MU ? MU : CKKS_MAX_PRIMES];
+#pragma unroll
     for (int t = 0; t < mu; ++t) a[t] = base[(i64)t * N];
+#pragma unroll
     for (int u = 1; u < mu; ++u) {
         const int top = mu - u;  // index of limb level-u
         const int ptop = l0 + top;
+#pragma unroll
         for (int t = 0; t < top; ++t) {
             const int pt = l0 + t;
             const u64 qt = mods[pt].q;
@@ -854,7 +861,19 @@ __device__ __forceinline__ void rschain_coeff(u64 *base, int N, int level, int m
             a[t] = shoup(sub_mod(a[t], tr, qt), inv.w, inv.wp, qt);
         }
     }
+#pragma unroll
     for (int t = 0; t < mu - 1; ++t) base[(i64)t * N] = a[t];
+}
+
+__device__ __forceinline__ void rschain_any(u64 *base, int N, int level, int mu, const ModQ *mods, const Shoup *one,
+                                            const Shoup *invq) {
+    switch (mu) {
+    case 2: return rschain_coeff<2>(base, N, level, mu, mods, one, invq);
+    case 3: return rschain_coeff<3>(base, N, level, mu, mods, one, invq);
+    case 4: return rschain_coeff<4>(base, N, level, mu, mods, one, invq);
+    case 5: return rschain_coeff<5>(base, N, level, mu, mods, one, invq);
+    default: return rschain_coeff<0>(base, N, level, mu, mods, one, invq);
+    }
 }
 
 __global__ void __launch_bounds__(kThreads) rschain_kernel(RsChainArgs A) {
@@ -865,7 +884,7 @@ __global__ void __launch_bounds__(kThreads) rschain_kernel(RsChainArgs A) {
     const int p = (int)((gid % per) / A.N);
     const int e = (int)(gid % A.N);
     u64 *base = A.v.ptr + (i64)b * A.v.bstride + (i64)p * A.v.pstride + e;  // slot 0 = limb level - mu
-    rschain_coeff(base, A.N, A.level, A.mu, A.mods, A.one, A.invq);
+    rschain_any(base, A.N, A.level, A.mu, A.mods, A.one, A.invq);
 }
 
 // Table launch: blockIdx.y = tuple entry, x over its polynomials x coefficients.
@@ -876,7 +895,7 @@ __global__ void __launch_bounds__(kThreads) rschain_table_kernel(const RsJob *jo
     if (gid >= (i64)J.n_polys * N) return;
     const int p = (int)(gid / N);
     const int e = (int)(gid % N);
-    rschain_coeff(J.v + (i64)p * J.pstride + e, N, J.level, J.mu, mods, one, invq);
+    rschain_any(J.v + (i64)p * J.pstride + e, N, J.level, J.mu, mods, one, invq);
 }
 
 cudaError_t launch_rschain(const Context &C, const RsChainArgs &A, cudaStream_t st) {

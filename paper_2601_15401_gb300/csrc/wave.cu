@@ -484,7 +484,13 @@ int build(ckks_wave &W, char *scratch, std::vector<char> &tables) {
     for (auto &kv : B.st) {
         Stage &s = kv.second;
         if (s.count() == 0) continue;
-        if (s.kind == SK_NTT) s.off = put(tables, s.ntt);
+        if (s.kind == SK_NTT) {
+            // limbs of one prime next to each other: neighbouring CTAs read
+            // the same twiddles
+            std::stable_sort(s.ntt.begin(), s.ntt.end(),
+                             [](const NttJob &a, const NttJob &b) { return a.prime < b.prime; });
+            s.off = put(tables, s.ntt);
+        }
         if (s.kind == SK_TENSOR && s.fixed) {
             // one launch per shape: entries grouped by shape code
             // (the entries' children were sorted when they were built)
