@@ -76,6 +76,7 @@ __device__ void smem_fft(double2 *s, int lg, int sign, double2 *tw, const double
 // Y[k1][n2] = exp(sign 2 pi i n2 k1 / N) sum_n1 x[N2 n1 + n2] exp(sign 2 pi i n1 k1 / N1)
 __global__ void __launch_bounds__(kThr) fft_cols_kernel(const double2 *x, double2 *y, int lg1, int lg2, int sign,
                                                         const double2 *T) {
+    grid_dependency_wait();
     extern __shared__ double2 sm[];
     const int N1 = 1 << lg1, N2 = 1 << lg2, N = N1 * N2;
     const int tc = N2 < kTC ? N2 : kTC;
@@ -100,6 +101,7 @@ __global__ void __launch_bounds__(kThr) fft_cols_kernel(const double2 *x, double
 // Step 2 (rows): X[k1 + N1 k2] = sum_n2 Y[k1][n2] exp(sign 2 pi i n2 k2 / N2)
 __global__ void __launch_bounds__(kThr) fft_rows_kernel(const double2 *y, double2 *X, int lg1, int lg2, int sign,
                                                         const double2 *T) {
+    grid_dependency_wait();
     extern __shared__ double2 sm[];
     const int N1 = 1 << lg1, N2 = 1 << lg2, N = N1 * N2;
     const int tr = N1 < kTC ? N1 : kTC;
@@ -121,6 +123,7 @@ __global__ void __launch_bounds__(kThr) fft_rows_kernel(const double2 *y, double
 
 // decode, before the DFT: x_i = m_i omega^i
 __global__ void twist_kernel(const double *m, double2 *x, int N, const double2 *T) {
+    grid_dependency_wait();
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= N) return;
     const size_t o = (size_t)blockIdx.y * N + i;
@@ -130,6 +133,7 @@ __global__ void twist_kernel(const double *m, double2 *x, int N, const double2 *
 
 // decode, after: z_j = Z[(5^j mod 2N - 1) / 2] / scale
 __global__ void slots_kernel(const double2 *Z, double *z, int N, double inv_scale) {
+    grid_dependency_wait();
     const int j = blockIdx.x * blockDim.x + threadIdx.x;
     if (j >= N / 2) return;
     const double2 v = Z[(size_t)blockIdx.y * N + (pow5(j, 2u * N) - 1) / 2];
@@ -140,6 +144,7 @@ __global__ void slots_kernel(const double2 *Z, double *z, int N, double inv_scal
 
 // encode, before: V[(5^j - 1)/2] = scale z_j, V[(2N - 5^j - 1)/2] = conj
 __global__ void scatter_kernel(const double *z, double2 *V, int N, double scale) {
+    grid_dependency_wait();
     const int j = blockIdx.x * blockDim.x + threadIdx.x;
     if (j >= N / 2) return;
     const double *zi = z + ((size_t)blockIdx.y * (N / 2) + j) * 2;
@@ -152,6 +157,7 @@ __global__ void scatter_kernel(const double *z, double2 *V, int N, double scale)
 
 // encode, after: m_i = round(Re(omega^-i w_i) / N)
 __global__ void untwist_round_kernel(const double2 *w, long long *m, int N, const double2 *T) {
+    grid_dependency_wait();
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= N) return;
     const size_t o = (size_t)blockIdx.y * N + i;
@@ -162,6 +168,7 @@ __global__ void untwist_round_kernel(const double2 *w, long long *m, int N, cons
 
 // T[j] = exp(i pi j / N) for j < 2N
 __global__ void roots_kernel(double2 *T, int N) {
+    grid_dependency_wait();
     const int j = blockIdx.x * blockDim.x + threadIdx.x;
     if (j < 2 * N) T[j] = cis_pi((double)j / N);
 }
@@ -181,11 +188,11 @@ cudaError_t dft(const Context &C, const double2 *in, double2 *tmp, double2 *out,
     const size_t sm2 = (size_t)(kTC * N2 + N2 / 2 + 1) * sizeof(double2);
     const int tc = N2 < kTC ? N2 : kTC, tr = N1 < kTC ? N1 : kTC;
     count_kernel(C);
-    fft_cols_kernel<<<dim3(N2 / tc, batch), kThr, sm1, st>>>(in, tmp, lg1, lg2, sign, T);
+    launch_dependent(fft_cols_kernel, dim3(N2 / tc, batch), dim3(kThr), sm1, st, in, tmp, lg1, lg2, sign, T);
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
     count_kernel(C);
-    fft_rows_kernel<<<dim3(N1 / tr, batch), kThr, sm2, st>>>(tmp, out, lg1, lg2, sign, T);
+    launch_dependent(fft_rows_kernel, dim3(N1 / tr, batch), dim3(kThr), sm2, st, tmp, out, lg1, lg2, sign, T);
     return cudaGetLastError();
 }
 
@@ -194,7 +201,7 @@ size_t embed_ws(const Context &C, uint32_t batch) { return (2 * (size_t)batch + 
 // the roots table at the end of the workspace, filled on `st`
 cudaError_t roots(const Context &C, double2 *T, cudaStream_t st) {
     count_kernel(C);
-    roots_kernel<<<(2 * C.N + kThr - 1) / kThr, kThr, 0, st>>>(T, C.N);
+    launch_dependent(roots_kernel, dim3((2 * C.N + kThr - 1) / kThr), dim3(kThr), 0, st, T, C.N);
     return cudaGetLastError();
 }
 
@@ -222,13 +229,13 @@ int ckks_encode(ckks_context *ctx, const double *z, uint32_t batch, double scale
     cudaError_t err = roots(C, T, st);
     if (err == cudaSuccess) {
         count_kernel(C);
-        scatter_kernel<<<dim3((C.N / 2 + kThr - 1) / kThr, batch), kThr, 0, st>>>(z, A, C.N, scale);
+        launch_dependent(scatter_kernel, dim3((C.N / 2 + kThr - 1) / kThr, batch), dim3(kThr), 0, st, z, A, C.N, scale);
         err = cudaGetLastError();
     }
     if (err == cudaSuccess) err = dft(C, A, Bf, A, (int)batch, -1, T, st);
     if (err == cudaSuccess) {
         count_kernel(C);
-        untwist_round_kernel<<<dim3((C.N + kThr - 1) / kThr, batch), kThr, 0, st>>>(A, (long long *)m, C.N, T);
+        launch_dependent(untwist_round_kernel, dim3((C.N + kThr - 1) / kThr, batch), dim3(kThr), 0, st, A, (long long *)m, C.N, T);
         err = cudaGetLastError();
     }
     if (err != cudaSuccess) {
@@ -252,13 +259,13 @@ int ckks_decode(ckks_context *ctx, const double *m, uint32_t batch, double scale
     cudaError_t err = roots(C, T, st);
     if (err == cudaSuccess) {
         count_kernel(C);
-        twist_kernel<<<dim3((C.N + kThr - 1) / kThr, batch), kThr, 0, st>>>(m, A, C.N, T);
+        launch_dependent(twist_kernel, dim3((C.N + kThr - 1) / kThr, batch), dim3(kThr), 0, st, m, A, C.N, T);
         err = cudaGetLastError();
     }
     if (err == cudaSuccess) err = dft(C, A, Bf, A, (int)batch, +1, T, st);
     if (err == cudaSuccess) {
         count_kernel(C);
-        slots_kernel<<<dim3((C.N / 2 + kThr - 1) / kThr, batch), kThr, 0, st>>>(A, z, C.N, 1.0 / scale);
+        launch_dependent(slots_kernel, dim3((C.N / 2 + kThr - 1) / kThr, batch), dim3(kThr), 0, st, A, z, C.N, 1.0 / scale);
         err = cudaGetLastError();
     }
     if (err != cudaSuccess) {

@@ -41,6 +41,7 @@ __global__ void pk_kernel(const u64 *S, const u64 *E, const u64 *a, u64 *pk, int
 // Garner lift of (x0 mod q0, x1 mod q1) to [0, q0 q1), centred, as double.
 __global__ void crt2_kernel(const u64 *P, double *out, int limbs, int N, u64 q0, u64 q1, Shoup q0inv_mod_q1,
                             Shoup one_q1) {
+    grid_dependency_wait();
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= N) return;
     P += (i64)blockIdx.y * limbs * N;  // batch element
@@ -68,6 +69,7 @@ __global__ void crt2_kernel(const u64 *P, double *out, int limbs, int N, u64 q0,
 // T the transform of e0 + m
 __global__ void enc_batch_kernel(const u64 *W, const u64 *pk, i64 pk_pstride, u64 *out, i64 out_bstride,
                                  i64 out_pstride, int level, int N, const ModQ *mods, const u64 *r2) {
+    grid_dependency_wait();
     const i64 gid = (i64)blockIdx.x * blockDim.x + threadIdx.x;
     if (gid >= (i64)level * N) return;
     const int b = blockIdx.y;
@@ -85,6 +87,7 @@ __global__ void enc_batch_kernel(const u64 *W, const u64 *pk, i64 pk_pstride, u6
 // P[b][x] = C0 + C1 S over the lowest `limbs` limbs of every batch element
 __global__ void dec_batch_kernel(const u64 *ct, i64 bstride, i64 pstride, const u64 *S, u64 *P, int limbs, int N,
                                  const ModQ *mods, const u64 *r2) {
+    grid_dependency_wait();
     const i64 gid = (i64)blockIdx.x * blockDim.x + threadIdx.x;
     if (gid >= (i64)limbs * N) return;
     const int b = blockIdx.y;
@@ -197,8 +200,7 @@ int ckks_encrypt_batch(ckks_context *ctx, const int64_t *m, const int64_t *v, co
         err = transform_signed(C, (int)cb, 3, (int)level, sa, sb, w, st);
         if (err == cudaSuccess) {
             count_kernel(C);
-            enc_batch_kernel<<<dim3(blocks((i64)level * N), cb), kThr, 0, st>>>(
-                W, (const u64 *)pk, (i64)C.L * N, (u64 *)out[b0].data, os, ps, (int)level, C.N, C.d_mods, C.d_r2);
+            launch_dependent(enc_batch_kernel, dim3(blocks((i64)level * N), cb), dim3(kThr), 0, st, W, (const u64 *)pk, (i64)C.L * N, (u64 *)out[b0].data, os, ps, (int)level, C.N, C.d_mods, C.d_r2);
             err = cudaGetLastError();
         }
     }
@@ -248,8 +250,7 @@ int ckks_decrypt_batch(ckks_context *ctx, const ckks_tuple *ct, uint32_t batch, 
     cudaError_t err = transform_signed(C, 1, 1, limbs, sa, sb, LimbView{S, 0, (i64)limbs * N}, st);
     if (err == cudaSuccess) {
         count_kernel(C);
-        dec_batch_kernel<<<dim3(blocks((i64)limbs * N), batch), kThr, 0, st>>>(
-            (const u64 *)ct[0].data, cs, (i64)ct[0].poly_stride * N, S, P, limbs, C.N, C.d_mods, C.d_r2);
+        launch_dependent(dec_batch_kernel, dim3(blocks((i64)limbs * N), batch), dim3(kThr), 0, st, (const u64 *)ct[0].data, cs, (i64)ct[0].poly_stride * N, S, P, limbs, C.N, C.d_mods, C.d_r2);
         err = cudaGetLastError();
     }
     if (err == cudaSuccess) {
@@ -264,7 +265,7 @@ int ckks_decrypt_batch(ckks_context *ctx, const ckks_tuple *ct, uint32_t batch, 
             one_q1 = make_shoup(1, q1);
         }
         count_kernel(C);
-        crt2_kernel<<<dim3(blocks(N), batch), kThr, 0, st>>>(P, out, limbs, C.N, q0, q1, inv, one_q1);
+        launch_dependent(crt2_kernel, dim3(blocks(N), batch), dim3(kThr), 0, st, P, out, limbs, C.N, q0, q1, inv, one_q1);
         err = cudaGetLastError();
     }
     if (err != cudaSuccess) {

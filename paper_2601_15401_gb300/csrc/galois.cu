@@ -33,6 +33,7 @@ __device__ __forceinline__ uint32_t perm(uint32_t i, uint32_t g, int log_n) {
 // blockIdx.x = (output poly, limb, chunk), blockIdx.y = batch element.
 __global__ void __launch_bounds__(kThr) automorphism_kernel(LimbView in, LimbView out, AutoMap map, int level,
                                                             int log_n, uint32_t g) {
+    grid_dependency_wait();
     extern __shared__ u64 stage[];
     const int log_c = log_n < kLogChunk ? log_n : kLogChunk;
     const int chunk = 1 << log_c;
@@ -71,8 +72,8 @@ cudaError_t launch_automorphism(const Context &C, LimbView in, LimbView out, con
     ProfScope ps(C, KC_AUTOMORPHISM, (double)batch * (reads + map.n_out) * level * C.N * sizeof(u64), st);
     const int log_c = C.log_n < kLogChunk ? C.log_n : kLogChunk;
     dim3 grid((unsigned)((i64)map.n_out * level << (C.log_n - log_c)), (unsigned)batch);
-    automorphism_kernel<<<grid, kThr, (size_t)sizeof(u64) << log_c, st>>>(in, out, map, level, C.log_n, g);
-    return cudaGetLastError();
+    return launch_dependent(automorphism_kernel, grid, dim3(kThr), (size_t)sizeof(u64) << log_c, st, in, out, map, level,
+                            C.log_n, g);
 }
 
 }  // namespace ckks

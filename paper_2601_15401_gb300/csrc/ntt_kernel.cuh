@@ -569,6 +569,7 @@ __device__ __forceinline__ void phase_tile(u64 *sm, const NttPhase &P, const ulo
         // the n - 1 twiddles every column shares, copied while the first
         // pass's loads are in flight
         for (int i = tid; i < n; i += blockDim.x) tws[i] = tw[i];
+        grid_dependency_wait();
         run_passes<LOGN, LOGN2, FWD, SH, LM, SM, SMALL, Q1, 0>(ln, q, lc, sc, P.N1);
     } else {
         // a warp and its blocks, or the CTA and its limb
@@ -590,6 +591,7 @@ __device__ __forceinline__ void phase_tile(u64 *sm, const NttPhase &P, const ulo
         ln.e = (b0 + ln.blk) << LOGN;
         ln.active = FULL || b0 + ln.blk < P.N1;
         copy_twiddles<LOGN, LOGN2, FWD, SH, 0>(wtw, tw, P.N1, b0, lane);
+        grid_dependency_wait();
         const int words = (P.N1 - b0) * n;                // words of the limb from the first block on
         const int e0 = b0 << LOGN;
         // shared offset of word idx of the warp's blocks
@@ -681,6 +683,7 @@ template <int LOGN, int LOGN2, bool FWD, int SH, int LM, int SM, int MINB, bool 
 __global__ void __launch_bounds__(256, MINB) ntt_phase_table_kernel(NttPhase P, const NttJob *jobs, int tiles,
                                                                     LoadSpec L, StoreSpec S) {
     extern __shared__ __align__(16) u64 sm[];
+    grid_dependency_wait();  // the job table may have been written just before
     const int job = blockIdx.x / tiles;
     const int tile = blockIdx.x - job * tiles;
     const NttJob j = jobs[job];
@@ -732,8 +735,7 @@ static inline cudaError_t launch_uniform(const NttPhase &P, const LimbJobs &J, c
     cudaError_t e = allow_smem(kern, G.smem);
     if (e != cudaSuccess) return e;
     dim3 grid(G.tiles, J.n_batch * J.n_polys * J.n_limbs);
-    kern<<<grid, G.threads, G.smem, G.st>>>(P, J, L, S);
-    return cudaGetLastError();
+    return launch_dependent(kern, grid, dim3(G.threads), G.smem, G.st, P, J, L, S);
 }
 
 template <int LOGN, int LOGN2, bool FWD, int SH, int LM, int SM, int MINB, bool Q1>
@@ -745,8 +747,7 @@ static inline cudaError_t launch_table(const NttPhase &P, const NttJob *jobs, in
     const long long blocks = (long long)n_jobs * G.tiles;
     if (blocks <= 0) return cudaSuccess;
     if (blocks > 0x7FFFFFFFll) return cudaErrorInvalidValue;
-    kern<<<(unsigned)blocks, G.threads, G.smem, G.st>>>(P, jobs, G.tiles, L, S);
-    return cudaGetLastError();
+    return launch_dependent(kern, dim3((unsigned)blocks), dim3(G.threads), G.smem, G.st, P, jobs, G.tiles, L, S);
 }
 
 // Dispatch of one direction (FWD) and job source (TABLE) over the shape, log2

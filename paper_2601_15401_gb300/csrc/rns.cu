@@ -222,6 +222,7 @@ struct TensorOcc {
 
 template <int MAXT, bool Q1, int V>
 __global__ void __launch_bounds__(kThreads, TensorOcc<MAXT>::minb) tensor_kernel(TensorArgs A) {
+    grid_dependency_wait();
     const i64 r = ((i64)blockIdx.x * blockDim.x + threadIdx.x) * V;  // limb * N + coefficient
     if (r >= (i64)A.level * A.N) return;
     const int j = (int)(r >> A.log_n);
@@ -233,6 +234,7 @@ __global__ void __launch_bounds__(kThreads, TensorOcc<MAXT>::minb) tensor_kernel
 template <int MAXT, bool Q1, int V>
 __global__ void __launch_bounds__(kThreads, TensorOcc<MAXT>::minb) tensor_table_kernel(const TensorJob *jobs, int N, int log_n,
                                                                 const ModQ *mods, const Shoup *rfix) {
+    grid_dependency_wait();
     __shared__ TensorJob J;
     {
         // the entry is copied by many threads, one word each
@@ -280,20 +282,20 @@ constexpr int kTensorVecMaxT = CKKS_TENSOR_VEC_MAXT;
 
 template <bool Q1, int V>
 static void launch_tensor_sized(int maxt, dim3 blocks, const TensorArgs &A, cudaStream_t st) {
-    if (maxt <= 3) tensor_kernel<3, Q1, V><<<blocks, kThreads, 0, st>>>(A);
-    else if (maxt <= 4) tensor_kernel<4, Q1, V><<<blocks, kThreads, 0, st>>>(A);
-    else if (maxt <= 5 && (V == 1 || kTensorVecMaxT >= 5)) tensor_kernel<5, Q1, V><<<blocks, kThreads, 0, st>>>(A);
+    if (maxt <= 3) launch_dependent(tensor_kernel<3, Q1, V>, blocks, dim3(kThreads), 0, st, A);
+    else if (maxt <= 4) launch_dependent(tensor_kernel<4, Q1, V>, blocks, dim3(kThreads), 0, st, A);
+    else if (maxt <= 5 && (V == 1 || kTensorVecMaxT >= 5)) launch_dependent(tensor_kernel<5, Q1, V>, blocks, dim3(kThreads), 0, st, A);
     else if constexpr (V == 1) {
-        if (maxt <= 7) tensor_kernel<7, Q1, 1><<<blocks, kThreads, 0, st>>>(A);
-        else if (maxt <= 9) tensor_kernel<9, Q1, 1><<<blocks, kThreads, 0, st>>>(A);
-        else tensor_kernel<CKKS_MAX_TUPLE, Q1, 1><<<blocks, kThreads, 0, st>>>(A);
+        if (maxt <= 7) launch_dependent(tensor_kernel<7, Q1, 1>, blocks, dim3(kThreads), 0, st, A);
+        else if (maxt <= 9) launch_dependent(tensor_kernel<9, Q1, 1>, blocks, dim3(kThreads), 0, st, A);
+        else launch_dependent(tensor_kernel<CKKS_MAX_TUPLE, Q1, 1>, blocks, dim3(kThreads), 0, st, A);
     }
 }
 
 template <bool Q1, int V>
 static void launch_tensor_table_sized(const Context &C, int maxt, dim3 blocks, const TensorJob *jobs,
                                       cudaStream_t st) {
-#define CKKS_TT(MT, VV) tensor_table_kernel<MT, Q1, VV><<<blocks, kThreads, 0, st>>>(jobs, C.N, C.log_n, C.d_mods, C.d_rfix)
+#define CKKS_TT(MT, VV) launch_dependent(tensor_table_kernel<MT, Q1, VV>, blocks, dim3(kThreads), 0, st, jobs, C.N, C.log_n, C.d_mods, C.d_rfix)
     if (maxt <= 3) CKKS_TT(3, V);
     else if (maxt <= 4) CKKS_TT(4, V);
     else if (maxt <= 5 && (V == 1 || kTensorVecMaxT >= 5)) CKKS_TT(5, V);
@@ -434,6 +436,7 @@ __device__ __forceinline__ void bconv_block(const u64 *ctab, const u64 *y0, u64 
         cs[ti * na + jj] = LIMB ? pack_limbs<30>(c) : c;
     }
     __syncthreads();
+    grid_dependency_wait();
     constexpr int V = CKKS_BCONV_VEC;
     const int e = (blockIdx.x * blockDim.x + threadIdx.x) * V;
     if (e >= N) return;
@@ -526,6 +529,7 @@ __global__ void __launch_bounds__(CKKS_BCONV_MAX_THREADS, CKKS_BCONV_MINB) bconv
 template <int AMAX, bool Q1, bool LIMB>
 __global__ void __launch_bounds__(CKKS_BCONV_MAX_THREADS, CKKS_BCONV_MINB) bconv_table_kernel(const BconvJob *jobs, int alpha, int L, int K,
                                                            int n_primes, int N, const ModQ *mods) {
+    grid_dependency_wait();
     extern __shared__ u64 cs[];
     const BconvJob J = jobs[blockIdx.y];
     bconv_block<AMAX, Q1, LIMB>(J.consts, J.y, J.ext, J.level, J.beta, alpha, L, K, n_primes, N, mods, cs);
@@ -533,20 +537,20 @@ __global__ void __launch_bounds__(CKKS_BCONV_MAX_THREADS, CKKS_BCONV_MINB) bconv
 
 template <bool Q1, bool LIMB>
 static void launch_bconv_sized(int alpha, dim3 grid, int thr, size_t smem, const BconvArgs &A, cudaStream_t st) {
-    if (alpha <= 4) bconv_kernel<4, Q1, LIMB><<<grid, thr, smem, st>>>(A);
-    else if (alpha <= 8) bconv_kernel<8, Q1, LIMB><<<grid, thr, smem, st>>>(A);
-    else if (alpha <= 12) bconv_kernel<12, Q1, LIMB><<<grid, thr, smem, st>>>(A);
-    else bconv_kernel<16, Q1, LIMB><<<grid, thr, smem, st>>>(A);
+    if (alpha <= 4) launch_dependent(bconv_kernel<4, Q1, LIMB>, grid, dim3(thr), smem, st, A);
+    else if (alpha <= 8) launch_dependent(bconv_kernel<8, Q1, LIMB>, grid, dim3(thr), smem, st, A);
+    else if (alpha <= 12) launch_dependent(bconv_kernel<12, Q1, LIMB>, grid, dim3(thr), smem, st, A);
+    else launch_dependent(bconv_kernel<16, Q1, LIMB>, grid, dim3(thr), smem, st, A);
 }
 
 template <bool Q1, bool LIMB>
 static void launch_bconv_table_sized(const Context &C, dim3 grid, int thr, size_t smem, const BconvJob *jobs,
                                      cudaStream_t st) {
     const int np = C.L + C.K, a = C.alpha;
-    if (a <= 4) bconv_table_kernel<4, Q1, LIMB><<<grid, thr, smem, st>>>(jobs, a, C.L, C.K, np, C.N, C.d_mods);
-    else if (a <= 8) bconv_table_kernel<8, Q1, LIMB><<<grid, thr, smem, st>>>(jobs, a, C.L, C.K, np, C.N, C.d_mods);
-    else if (a <= 12) bconv_table_kernel<12, Q1, LIMB><<<grid, thr, smem, st>>>(jobs, a, C.L, C.K, np, C.N, C.d_mods);
-    else bconv_table_kernel<16, Q1, LIMB><<<grid, thr, smem, st>>>(jobs, a, C.L, C.K, np, C.N, C.d_mods);
+    if (a <= 4) launch_dependent(bconv_table_kernel<4, Q1, LIMB>, grid, dim3(thr), smem, st, jobs, a, C.L, C.K, np, C.N, C.d_mods);
+    else if (a <= 8) launch_dependent(bconv_table_kernel<8, Q1, LIMB>, grid, dim3(thr), smem, st, jobs, a, C.L, C.K, np, C.N, C.d_mods);
+    else if (a <= 12) launch_dependent(bconv_table_kernel<12, Q1, LIMB>, grid, dim3(thr), smem, st, jobs, a, C.L, C.K, np, C.N, C.d_mods);
+    else launch_dependent(bconv_table_kernel<16, Q1, LIMB>, grid, dim3(thr), smem, st, jobs, a, C.L, C.K, np, C.N, C.d_mods);
 }
 
 cudaError_t launch_bconv(const Context &C, const BconvArgs &A, cudaStream_t st) {
@@ -715,6 +719,7 @@ __device__ __forceinline__ void mac_limb(const u64 *const *dsrc, const i64 *dstr
 // blocks that share key rows run next to each other.
 template <bool Q1, int P, int V, bool LIMB>
 __global__ void __launch_bounds__(CKKS_MAC_MAX_THREADS, CKKS_MAC_MINB) mac_kernel(MacArgs A, int b_first, int n_groups) {
+    grid_dependency_wait();
     const int chunks = (A.N + blockDim.x * V - 1) / (blockDim.x * V);
     int bid = blockIdx.x;
     const int g = bid % n_groups;
@@ -749,9 +754,9 @@ static void launch_mac_part(const Context &C, const MacArgs &A, int b_first, int
     const int chunks = (A.N + thr * V - 1) / (thr * V);
     const long long blocks = (long long)chunks * (A.level + A.K) * n_groups;
     count_kernel(C);
-    if (!C.limbs30) mac_kernel<false, P, V, false><<<(unsigned)blocks, thr, 0, st>>>(A, b_first, n_groups);
-    else if (C.q1()) mac_kernel<true, P, V, true><<<(unsigned)blocks, thr, 0, st>>>(A, b_first, n_groups);
-    else mac_kernel<false, P, V, true><<<(unsigned)blocks, thr, 0, st>>>(A, b_first, n_groups);
+    if (!C.limbs30) launch_dependent(mac_kernel<false, P, V, false>, dim3((unsigned)blocks), dim3(thr), 0, st, A, b_first, n_groups);
+    else if (C.q1()) launch_dependent(mac_kernel<true, P, V, true>, dim3((unsigned)blocks), dim3(thr), 0, st, A, b_first, n_groups);
+    else launch_dependent(mac_kernel<false, P, V, true>, dim3((unsigned)blocks), dim3(thr), 0, st, A, b_first, n_groups);
 }
 
 cudaError_t launch_mac(const Context &C, const MacArgs &A, cudaStream_t st) {
@@ -778,6 +783,7 @@ __global__ void __launch_bounds__(CKKS_MAC_MAX_THREADS, CKKS_MAC_MINB) mac_table
                                                                          const u64 *keys, i64 key_pstride,
                                                                          int key_digits, int alpha, int L, int N,
                                                                          const ModQ *mods) {
+    grid_dependency_wait();
     const MacTarget T = targets[blockIdx.x];
     const int e = (blockIdx.y * blockDim.x + threadIdx.x) * V;
     if (e >= N) return;
@@ -814,7 +820,7 @@ static cudaError_t launch_mac_table_part(const Context &C, const MacJob *jobs, c
     dim3 grid((unsigned)n, (unsigned)chunks);
     const i64 kps = (i64)(C.L + C.K) * C.N;
 #define CKKS_MACT(Q, LB) \
-    mac_table_kernel<Q, P, V, LB><<<grid, thr, 0, st>>>(jobs, targets, keys, kps, C.dnum, C.alpha, C.L, C.N, C.d_mods)
+    launch_dependent(mac_table_kernel<Q, P, V, LB>, grid, dim3(thr), 0, st, jobs, targets, keys, kps, C.dnum, C.alpha, C.L, C.N, C.d_mods)
     if (!C.limbs30) CKKS_MACT(false, false);
     else if (C.q1()) CKKS_MACT(true, true);
     else CKKS_MACT(false, true);
@@ -877,6 +883,7 @@ __device__ __forceinline__ void rschain_any(u64 *base, int N, int level, int mu,
 }
 
 __global__ void __launch_bounds__(kThreads) rschain_kernel(RsChainArgs A) {
+    grid_dependency_wait();
     const i64 gid = (i64)blockIdx.x * blockDim.x + threadIdx.x;
     const i64 per = (i64)A.n_polys * A.N;
     if (gid >= per * A.n_batch) return;
@@ -890,6 +897,7 @@ __global__ void __launch_bounds__(kThreads) rschain_kernel(RsChainArgs A) {
 // Table launch: blockIdx.y = tuple entry, x over its polynomials x coefficients.
 __global__ void __launch_bounds__(kThreads) rschain_table_kernel(const RsJob *jobs, int N, const ModQ *mods,
                                                                  const Shoup *one, const Shoup *invq) {
+    grid_dependency_wait();
     const RsJob J = jobs[blockIdx.y];
     const i64 gid = (i64)blockIdx.x * blockDim.x + threadIdx.x;
     if (gid >= (i64)J.n_polys * N) return;
@@ -903,7 +911,7 @@ cudaError_t launch_rschain(const Context &C, const RsChainArgs &A, cudaStream_t 
     i64 total = (i64)A.n_batch * A.n_polys * A.N;
     count_kernel(C);
     ProfScope ps(C, KC_RSCHAIN, 2.0 * A.n_batch * A.n_polys * A.mu * A.N * sizeof(u64), st);
-    rschain_kernel<<<(unsigned)((total + kThreads - 1) / kThreads), kThreads, 0, st>>>(A);
+    launch_dependent(rschain_kernel, dim3((unsigned)((total + kThreads - 1) / kThreads)), dim3(kThreads), 0, st, A);
     return cudaGetLastError();
 }
 
@@ -914,7 +922,7 @@ cudaError_t launch_rschain_table(const Context &C, const RsJob *jobs, int n_jobs
     count_kernel(C);
     ProfScope ps(C, KC_RSCHAIN, bytes, st);
     dim3 grid((unsigned)(((i64)max_polys * C.N + kThreads - 1) / kThreads), (unsigned)n_jobs);
-    rschain_table_kernel<<<grid, kThreads, 0, st>>>(jobs, C.N, C.d_mods, C.d_one, C.d_invq);
+    launch_dependent(rschain_table_kernel, grid, dim3(kThreads), 0, st, jobs, C.N, C.d_mods, C.d_one, C.d_invq);
     return cudaGetLastError();
 }
 
@@ -989,6 +997,7 @@ cudaError_t launch_pointwise_mul(const Context &C, u64 *St, const u64 *S, cudaSt
 // dst <- dst + src over [batch][polys][level][N] limb views (limb x mod q_x)
 __global__ void __launch_bounds__(kThreads) add_limbs_kernel(LimbView dst, LimbView src, int polys, int level, int N,
                                                              const ModQ *mods) {
+    grid_dependency_wait();
     const i64 gid = (i64)blockIdx.x * blockDim.x + threadIdx.x;
     const i64 per_poly = (i64)level * N;
     if (gid >= per_poly * polys) return;
@@ -1007,7 +1016,7 @@ cudaError_t launch_add_limbs(const Context &C, LimbView dst, LimbView src, int b
     if (total == 0 || batch == 0) return cudaSuccess;
     count_kernel(C);
     dim3 grid((unsigned)((total + kThreads - 1) / kThreads), (unsigned)batch);
-    add_limbs_kernel<<<grid, kThreads, 0, st>>>(dst, src, polys, level, C.N, C.d_mods);
+    launch_dependent(add_limbs_kernel, grid, dim3(kThreads), 0, st, dst, src, polys, level, C.N, C.d_mods);
     return cudaGetLastError();
 }
 

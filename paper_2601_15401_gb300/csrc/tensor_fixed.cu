@@ -105,6 +105,7 @@ __device__ __forceinline__ void tensor_fixed_coeff(const View &v, i64 r, int j, 
 
 template <int A, int B, int C, bool Q1>
 __global__ void __launch_bounds__(kThreads, 3) tensor_fixed_kernel(TensorArgs T) {
+    grid_dependency_wait();
     const i64 r = (i64)blockIdx.x * blockDim.x + threadIdx.x;  // limb * N + coefficient
     if (r >= (i64)T.level * T.N) return;
     const int j = (int)(r >> T.log_n);
@@ -116,6 +117,7 @@ __global__ void __launch_bounds__(kThreads, 3) tensor_fixed_kernel(TensorArgs T)
 template <int A, int B, int C, bool Q1>
 __global__ void __launch_bounds__(kThreads, 3) tensor_fixed_table_kernel(const TensorJob *jobs, int N, int log_n,
                                                                         const ModQ *mods, const Shoup *rfix) {
+    grid_dependency_wait();
     __shared__ TensorJob J;
     {
         static_assert(sizeof(TensorJob) % sizeof(u64) == 0, "TensorJob is a whole number of words");
@@ -156,9 +158,8 @@ template <bool Q1>
 cudaError_t launch_uniform(const TensorArgs &T, int code, cudaStream_t st) {
     dim3 blocks((unsigned)(((i64)T.level * T.N + kThreads - 1) / kThreads), T.n_batch);
     return with_shape(code, [&](auto a, auto b, auto c) {
-        tensor_fixed_kernel<decltype(a)::value, decltype(b)::value, decltype(c)::value, Q1>
-            <<<blocks, kThreads, 0, st>>>(T);
-        return cudaGetLastError();
+        return launch_dependent(tensor_fixed_kernel<decltype(a)::value, decltype(b)::value, decltype(c)::value, Q1>,
+                                blocks, dim3(kThreads), 0, st, T);
     });
 }
 
@@ -167,9 +168,9 @@ cudaError_t launch_table(const Context &C, const TensorJob *jobs, int n_jobs, in
                          cudaStream_t st) {
     dim3 blocks((unsigned)(((i64)max_level * C.N + kThreads - 1) / kThreads), (unsigned)n_jobs);
     return with_shape(code, [&](auto a, auto b, auto c) {
-        tensor_fixed_table_kernel<decltype(a)::value, decltype(b)::value, decltype(c)::value, Q1>
-            <<<blocks, kThreads, 0, st>>>(jobs, C.N, C.log_n, C.d_mods, C.d_rfix);
-        return cudaGetLastError();
+        return launch_dependent(
+            tensor_fixed_table_kernel<decltype(a)::value, decltype(b)::value, decltype(c)::value, Q1>, blocks,
+            dim3(kThreads), 0, st, jobs, C.N, C.log_n, C.d_mods, C.d_rfix);
     });
 }
 
