@@ -291,23 +291,26 @@ static cudaError_t relin_core(const Context &C, Ws &ws, int B, int n, int level,
         Bc.mods = C.d_mods;
         TRY(launch_bconv(C, Bc, st));
     }
-    // 3. NTT of the converted limbs, one launch pair per digit
-    for (int beta = 0; beta < nd; ++beta) {
-        const int d0 = beta * A, d1 = std::min(level, d0 + A);
-        const int nt = level - (d1 - d0) + K;
-        LimbJobs J = jobs(B, n - 1, nt);
-        int l = 0;
-        for (int x = 0; x < level; ++x) {
-            if (x >= d0 && x < d1) continue;
-            J.slot[l] = J.dslot[l] = (uint8_t)x;
-            J.prime[l] = (uint8_t)x;
-            ++l;
+    // 3. NTT of the converted limbs: the limbs of as many digits as a launch's
+    // limb list holds go together (three digits of a full-size chain ran as
+    // three launch pairs, each with its own last round of CTAs)
+    for (int beta = 0; beta < nd;) {
+        LimbJobs J = jobs(B, n - 1, 0);
+        const int first = beta;
+        for (; beta < nd; ++beta) {
+            const int d0 = beta * A, d1 = std::min(level, d0 + A);
+            const int nt = level - (d1 - d0) + K, slot0 = (beta - first) * ext_l;
+            // (the launch's second grid dimension holds the limbs of the batch)
+            if (beta > first && (J.n_limbs + nt > CKKS_MAX_PRIMES || slot0 + ext_l > 256 ||
+                                 (i64)B * (n - 1) * (J.n_limbs + nt) > 65535))
+                break;
+            for (int x = 0; x < ext_l; ++x) {
+                if (x >= d0 && x < d1) continue;
+                J.slot[J.n_limbs] = J.dslot[J.n_limbs] = (uint8_t)(slot0 + x);
+                J.prime[J.n_limbs++] = (uint8_t)(x < level ? x : C.L + (x - level));
+            }
         }
-        for (int i = 0; i < K; ++i, ++l) {
-            J.slot[l] = J.dslot[l] = (uint8_t)(level + i);
-            J.prime[l] = (uint8_t)(C.L + i);
-        }
-        LimbView v = view(ext + (size_t)beta * ext_l * N, ev.bstride, (i64)nd * ext_l * N);
+        LimbView v = view(ext + (size_t)first * ext_l * N, ev.bstride, (i64)nd * ext_l * N);
         LoadSpec L{};
         L.mode = LD_PLAIN;
         L.a = v;
