@@ -273,6 +273,21 @@ struct DotLimbs {
         s1 = mad_wide(a.hi, b.hi, s1);
         sx = mad_wide(a.sum, b.sum, sx);
     }
+    // (the sum + a multiple of q) / 2^(2 SB): Montgomery reduction by limbs, two
+    // steps of SB bits (R = 2^(2 SB)) that take one narrow and two wide
+    // multiplies each and no 64 x 64-bit product. q0, q1: q's limbs;
+    // nqi = -q^-1 mod 2^SB. In [0, sum / 2^(2 SB) + q + 1).
+    template <int SB>
+    CKKS_HD u64 redc(u32 q0, u32 q1, u32 nqi) const {
+        constexpr u32 M = (1u << SB) - 1;
+        const u64 x = sx - s0 - s1;
+        const u32 m0 = mad_lo(lo32(s0), nqi, 0u) & M;
+        const u64 a = mad_wide(m0, q0, s0) >> SB;
+        const u64 b = mad_wide(m0, q1, (u64)(lo32(x) & M)) + a;
+        const u32 m1 = mad_lo(lo32(b), nqi, 0u) & M;
+        const u64 c = mad_wide(m1, q0, b) >> SB;
+        return mad_wide(m1, q1, s1) + (x >> SB) + c;
+    }
     // SB = 30: brings the sums of up to 7 terms (or of a folded value, worth
     // one, and 6 terms) back to a value below 2 q 2^60 + 2^60: the middle sum's
     // high part and the high sum, reduced mod q, and two low limbs.

@@ -6,7 +6,8 @@
 //                 order the NTT's passes read them (twiddle_slot)
 //   N^-1          Shoup constants (INTT)
 //   ModUp BConv   per level and digit: N^-1 [(Q_beta/q_j)^-1]_{q_j} (applied
-//                 in the INTT epilogue) and [(Q_beta/q_j) mod x] R (Eq. 4)
+//                 in the INTT epilogue) and [(Q_beta/q_j) mod x] R (Eq. 4;
+//                 R = 2^60 when every prime is below 2^60)
 //   ModDown       N^-1 [phat_i^-1]_{p_i} and [p_i^-1]_{q_j} R (Eq. 5, 12)
 //   key fold      P^-1 R^2 mod q_j, R^2 mod p_i (Eq. 12: P^-1 inside the key)
 //   rescale       q_i^-1 mod q_j, and g^{mu,t}_eta of Eq. 16 per level, mu
@@ -15,6 +16,7 @@
 #include <new>
 
 #include "internal.h"
+#include "rns.h"
 
 namespace ckks {
 
@@ -172,6 +174,9 @@ int context_build(Context &C, const uint32_t log_n, const uint32_t L, const uint
             rfix[(size_t)x * 16 + e] = h_shoup(acc, m);
             acc = h_mul(acc, R, m);
         }
+        const u64 R60 = (1ull << 60) % m;
+        rfix[(size_t)x * 16 + kRfix60] = h_shoup(R60, m);
+        rfix[(size_t)x * 16 + kRfix60 + 1] = h_shoup(h_mul(R60, R60, m), m);
         u64 Pm = 1 % m;
         for (int i = 0; i < C.K; ++i) Pm = h_mul(Pm, p[i] % m, m);
         keyfold[x] = x < C.L ? h_mul(h_inv(Pm, m), r2[x], m) : r2[x];
@@ -214,7 +219,9 @@ int context_build(Context &C, const uint32_t log_n, const uint32_t L, const uint
                     u64 hx = 1 % m;
                     for (int j2 = d0; j2 < d1; ++j2)
                         if (j2 != j) hx = h_mul(hx, q[j2] % m, m);
-                    bcon[(((size_t)lv * C.dnum + b) * A + (j - d0)) * NP + x] = h_mul(hx, h_R(m), m);
+                    // Montgomery form: R = 2^60 for the products on limbs, else 2^64
+                    bcon[(((size_t)lv * C.dnum + b) * A + (j - d0)) * NP + x] =
+                        h_mul(hx, C.limbs30 ? (1ull << 60) % m : h_R(m), m);
                 }
             }
         }

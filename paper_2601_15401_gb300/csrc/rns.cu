@@ -433,8 +433,10 @@ __device__ __forceinline__ void bconv_block(const u64 *ctab, const u64 *y0, u64 
         int jj = i / n_t, ti = i % n_t;
         int x = ti < nq_t ? (ti < d0 ? ti : ti + na) : L + (ti - nq_t);
         const u64 c = ctab[(i64)jj * n_primes + x];
-        cs[ti * na + jj] = LIMB ? pack_limbs<30>(c) : c;
+        cs[ti * AMAX + jj] = LIMB ? pack_limbs<30>(c) : c;
     }
+    // the products run over AMAX sources, the ones the digit does not have as zeros
+    for (int i = threadIdx.x; i < (AMAX - na) * n_t; i += blockDim.x) cs[i / (AMAX - na) * AMAX + na + i % (AMAX - na)] = 0;
     __syncthreads();
     grid_dependency_wait();
     constexpr int V = CKKS_BCONV_VEC;
@@ -450,11 +452,14 @@ __device__ __forceinline__ void bconv_block(const u64 *ctab, const u64 *y0, u64 
             for (int v = 0; v < V; ++v) y[jj][v] = 0ull;
     }
     Limbs yl[LIMB ? AMAX : 1][V];
+    bool wide = false;  // sources of 2^53 or more: the sum needs more than one subtraction
     if constexpr (LIMB) {
 #pragma unroll
-        for (int jj = 0; jj < AMAX; ++jj)
+        for (int jj = 0; jj < AMAX; ++jj) {
 #pragma unroll
             for (int v = 0; v < V; ++v) yl[jj][v] = split_limbs<30>(y[jj][v]);
+            if (jj < na) wide = wide || !small_prime(mods[d0 + jj].q);
+        }
     }
     u64 *dst = dst0 + e;
     for (int ti = 0; ti < n_t; ++ti) {
@@ -464,8 +469,12 @@ __device__ __forceinline__ void bconv_block(const u64 *ctab, const u64 *y0, u64 
         // sum over the digit: hi stays below q because the digit's primes sum to < 2^64
         u64 r[V];
         if constexpr (LIMB) {
-            const u64 *ct = cs + ti * na;
-            u64 hi[V], lo[V];
+            // Products of at most kLimbTerms30 sources, each chunk reduced by
+            // limbs: sources of S = sum of the digit's primes < 2^64 leave
+            // r < S q / 2^60 + q < 17 q (below 1.1 q for eight sources under
+            // 2^53).
+            const u64 *ct = cs + ti * AMAX;
+            const u32 q0 = lo32(m.q) & 0x3fffffffu, q1 = (u32)(m.q >> 30), nqi = 0u - lo32(m.qinv);
 #pragma unroll
             for (int j0 = 0; j0 < AMAX; j0 += kLimbTerms30) {
                 DotLimbs acc[V];
@@ -473,28 +482,21 @@ __device__ __forceinline__ void bconv_block(const u64 *ctab, const u64 *y0, u64 
                 for (int v = 0; v < V; ++v) acc[v].zero();
 #pragma unroll
                 for (int k = 0; k < kLimbTerms30; ++k)
-                    if (j0 + k < AMAX && j0 + k < na) {
+                    if (j0 + k < AMAX) {
                         const Limbs c = packed_limbs(ct[j0 + k]);
 #pragma unroll
                         for (int v = 0; v < V; ++v) acc[v].mac(yl[j0 + k < AMAX ? j0 + k : 0][v], c);
                     }
 #pragma unroll
                 for (int v = 0; v < V; ++v) {
-                    u64 h, l;
-                    acc[v].template value<30>(h, l);
-                    if (j0 == 0) {
-                        hi[v] = h;
-                        lo[v] = l;
-                    } else {
-                        lo[v] += l;
-                        hi[v] += h + (lo[v] < l ? 1ull : 0ull);
-                    }
+                    u64 t = acc[v].template redc<30>(q0, q1, nqi);
+                    if (wide) t = reduce_near(t, m.q, m.canon);
+                    t = t >= m.q ? t - m.q : t;
+                    r[v] = j0 == 0 ? t : add_mod(r[v], t, m.q);
                 }
             }
-#pragma unroll
-            for (int v = 0; v < V; ++v) r[v] = redc_t<Q1>(hi[v], lo[v], m);
         } else {
-            const u64 *ct = cs + ti * na;
+            const u64 *ct = cs + ti * AMAX;
             Acc128Lazy acc[V];
 #pragma unroll
             for (int v = 0; v < V; ++v) acc[v].zero();
@@ -514,7 +516,7 @@ __device__ __forceinline__ void bconv_block(const u64 *ctab, const u64 *y0, u64 
 
 template <int AMAX, bool Q1, bool LIMB>
 __global__ void __launch_bounds__(CKKS_BCONV_MAX_THREADS, CKKS_BCONV_MINB) bconv_kernel(BconvArgs A) {
-    extern __shared__ u64 cs[];  // [n_targets][|digit|] Montgomery constants
+    extern __shared__ u64 cs[];  // [n_targets][AMAX] Montgomery constants
     const int job = blockIdx.y;
     const int b = blockIdx.z;
     const int t = job / A.n_digits;
@@ -534,6 +536,9 @@ __global__ void __launch_bounds__(CKKS_BCONV_MAX_THREADS, CKKS_BCONV_MINB) bconv
     const BconvJob J = jobs[blockIdx.y];
     bconv_block<AMAX, Q1, LIMB>(J.consts, J.y, J.ext, J.level, J.beta, alpha, L, K, n_primes, N, mods, cs);
 }
+
+// sources the kernel for digits of alpha primes is unrolled to
+static int bconv_sources(int alpha) { return alpha <= 4 ? 4 : alpha <= 8 ? 8 : alpha <= 12 ? 12 : 16; }
 
 template <bool Q1, bool LIMB>
 static void launch_bconv_sized(int alpha, dim3 grid, int thr, size_t smem, const BconvArgs &A, cudaStream_t st) {
@@ -556,7 +561,7 @@ static void launch_bconv_table_sized(const Context &C, dim3 grid, int thr, size_
 cudaError_t launch_bconv(const Context &C, const BconvArgs &A, cudaStream_t st) {
     const int thr = std::min(C.tune_bconv_threads, CKKS_BCONV_MAX_THREADS);
     dim3 grid((A.N + thr * CKKS_BCONV_VEC - 1) / (thr * CKKS_BCONV_VEC), A.n_t * A.n_digits, A.n_batch);
-    size_t smem = (size_t)A.alpha * (A.level + A.K) * sizeof(u64);
+    size_t smem = (size_t)bconv_sources(A.alpha) * (A.level + A.K) * sizeof(u64);
     count_kernel(C);
     count_op(C, OP_BCONV, (unsigned long long)A.n_t * A.n_digits * A.n_batch);
     // reads y' once, writes level + K - |digit| limbs per (t, digit)
@@ -584,7 +589,7 @@ cudaError_t launch_bconv_table(const Context &C, const BconvJob *jobs, int n_job
     if (n_jobs > 65535) return cudaErrorInvalidValue;
     const int thr = std::min(C.tune_bconv_threads, CKKS_BCONV_MAX_THREADS);
     dim3 grid((C.N + thr * CKKS_BCONV_VEC - 1) / (thr * CKKS_BCONV_VEC), (unsigned)n_jobs);
-    size_t smem = (size_t)C.alpha * (C.L + C.K) * sizeof(u64);
+    size_t smem = (size_t)bconv_sources(C.alpha) * (C.L + C.K) * sizeof(u64);
     count_kernel(C);
     count_op(C, OP_BCONV, (unsigned long long)n_jobs);
     ProfScope ps(C, KC_BCONV, bytes, st, macs);

@@ -8,6 +8,10 @@ struct Context;
 
 #define CKKS_MAX_CHILDREN 12
 
+// rfix entries of the products on limbs: R^1 and R^2 with R = 2^60 (the others,
+// e <= 12, are R^(e-1) with R = 2^64)
+constexpr int kRfix60 = 14;
+
 struct TensorArgs {
     int n_batch, level, N, m, log_n;
     LimbView child[CKKS_MAX_CHILDREN];   // limb j of poly a: ptr + b bstride + a pstride + j N

@@ -44,6 +44,14 @@ template <int SB> static void dots(u64 q, u64 qb, int terms, std::mt19937_64 &g)
     u64 hi, lo;
     d.value<SB>(hi, lo);
     check(hi == (u64)(sum >> 64) && lo == (u64)sum, "dot", q, qb, terms);
+    // Montgomery reduction of the sum by limbs modulo the prime qb: r 2^(2 SB) = sum
+    // (mod qb), r <= sum / 2^(2 SB) + qb
+    u64 inv = qb;
+    for (int i = 0; i < 6; ++i) inv *= 2 - qb * inv;
+    const u64 r = d.redc<SB>((u32)qb & ((1u << SB) - 1), (u32)(qb >> SB), 0u - (u32)inv);
+    const u128 R = ((u128)1 << (2 * SB)) % qb;
+    check((u64)((u128)(r % qb) * (u64)R % qb) == (u64)(sum % qb) && (u128)r <= (sum >> (2 * SB)) + qb + 1, "redc", q, qb,
+          terms);
 }
 int main() {
     std::mt19937_64 g(20);
