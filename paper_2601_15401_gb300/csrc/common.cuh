@@ -147,6 +147,33 @@ struct Acc128Lazy {
     __device__ __forceinline__ void add(u64 vhi, u64 vlo, u64) { add(vhi, vlo); }
 };
 
+// V adjacent words at p (16-byte loads / stores for even V; p 16-byte aligned)
+template <int V>
+__device__ __forceinline__ void load_span(const u64 *p, u64 (&o)[V]) {
+    if constexpr (V % 2 == 0) {
+#pragma unroll
+        for (int i = 0; i < V; i += 2) {
+            const ulonglong2 v = *reinterpret_cast<const ulonglong2 *>(p + i);
+            o[i] = v.x;
+            o[i + 1] = v.y;
+        }
+    } else {
+#pragma unroll
+        for (int i = 0; i < V; ++i) o[i] = p[i];
+    }
+}
+
+template <int V>
+__device__ __forceinline__ void store_span(u64 *p, const u64 (&v)[V]) {
+    if constexpr (V % 2 == 0) {
+#pragma unroll
+        for (int i = 0; i < V; i += 2) *reinterpret_cast<ulonglong2 *>(p + i) = make_ulonglong2(v[i], v[i + 1]);
+    } else {
+#pragma unroll
+        for (int i = 0; i < V; ++i) p[i] = v[i];
+    }
+}
+
 // Addressing of a set of limbs: limb (b, p, l) of a [batch][poly][limb][N]
 // view lives at ptr + b * bstride + p * pstride + slot[l] * N.
 struct LimbView {

@@ -16,7 +16,6 @@
 #include <new>
 
 #include "internal.h"
-#include "rns.h"
 
 namespace ckks {
 
@@ -174,9 +173,6 @@ int context_build(Context &C, const uint32_t log_n, const uint32_t L, const uint
             rfix[(size_t)x * 16 + e] = h_shoup(acc, m);
             acc = h_mul(acc, R, m);
         }
-        const u64 R60 = (1ull << 60) % m;
-        rfix[(size_t)x * 16 + kRfix60] = h_shoup(R60, m);
-        rfix[(size_t)x * 16 + kRfix60 + 1] = h_shoup(h_mul(R60, R60, m), m);
         u64 Pm = 1 % m;
         for (int i = 0; i < C.K; ++i) Pm = h_mul(Pm, p[i] % m, m);
         keyfold[x] = x < C.L ? h_mul(h_inv(Pm, m), r2[x], m) : r2[x];

@@ -40,33 +40,6 @@ static constexpr int kThreads = 256;
 #endif
 using TensorAcc = std::conditional<CKKS_TENSOR_LAZY != 0, Acc128Lazy, Acc128>::type;
 
-// V adjacent words at p (16-byte loads / stores for even V; p 16-byte aligned)
-template <int V>
-__device__ __forceinline__ void load_span(const u64 *p, u64 (&o)[V]) {
-    if constexpr (V % 2 == 0) {
-#pragma unroll
-        for (int i = 0; i < V; i += 2) {
-            const ulonglong2 v = *reinterpret_cast<const ulonglong2 *>(p + i);
-            o[i] = v.x;
-            o[i + 1] = v.y;
-        }
-    } else {
-#pragma unroll
-        for (int i = 0; i < V; ++i) o[i] = p[i];
-    }
-}
-
-template <int V>
-__device__ __forceinline__ void store_span(u64 *p, const u64 (&v)[V]) {
-    if constexpr (V % 2 == 0) {
-#pragma unroll
-        for (int i = 0; i < V; i += 2) *reinterpret_cast<ulonglong2 *>(p + i) = make_ulonglong2(v[i], v[i + 1]);
-    } else {
-#pragma unroll
-        for (int i = 0; i < V; ++i) p[i] = v[i];
-    }
-}
-
 // ---------------------------------------------------------------------------
 // tensor product: out = prod over children of (sum_l c_l s^l), coefficient-
 // wise in the NTT domain. Each child product is a Montgomery product, so the
@@ -318,7 +291,7 @@ cudaError_t launch_tensor(const Context &C, const TensorArgs &Ain, cudaStream_t 
     // children sorted by size, largest first (the smallest, last, takes the
     // R^(m-1) correction); a node shape with a fixed kernel takes it
     int code = tensor_sort_children(A);
-    if (!C.tune_tensor_fixed) code = -1;
+    if (!C.tune_tensor_fixed || (code >= kTensorSmallCode && !C.limbs30)) code = -1;
     int in_polys = 0, maxt = 0;
     bool vec2 = view_vec2(A.out);
     for (int c = 0; c < A.m; ++c) {
@@ -328,11 +301,12 @@ cudaError_t launch_tensor(const Context &C, const TensorArgs &Ain, cudaStream_t 
     }
     int out_polys = in_polys - A.m + 1;
     maxt = std::max(maxt, out_polys);
+    const bool vec2_any = vec2;
     vec2 = vec2 && maxt <= kTensorVecMaxT;
     const double coeffs = (double)A.n_batch * A.level * A.N;
     ProfScope ps(C, KC_TENSOR, (double)(in_polys + out_polys) * coeffs * sizeof(u64), st,
                  coeffs * tensor_products_per_coeff(A.child_polys, A.m));
-    if (code >= 0) return launch_tensor_fixed(C, A, code, st);
+    if (code >= 0) return launch_tensor_fixed(C, A, code, vec2_any, st);
     const i64 per = vec2 ? 2 * kThreads : kThreads;
     dim3 blocks((unsigned)(((i64)A.level * A.N + per - 1) / per), A.n_batch);
     if (vec2) {

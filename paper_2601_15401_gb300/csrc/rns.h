@@ -8,10 +8,6 @@ struct Context;
 
 #define CKKS_MAX_CHILDREN 12
 
-// rfix entries of the products on limbs: R^1 and R^2 with R = 2^60 (the others,
-// e <= 12, are R^(e-1) with R = 2^64)
-constexpr int kRfix60 = 14;
-
 struct TensorArgs {
     int n_batch, level, N, m, log_n;
     LimbView child[CKKS_MAX_CHILDREN];   // limb j of poly a: ptr + b bstride + a pstride + j N
@@ -124,13 +120,19 @@ struct TensorTableView {
 };
 
 cudaError_t launch_tensor(const Context &C, const TensorArgs &A, cudaStream_t st);
+// Codes of the small shapes (every child at most 3 terms): only in contexts
+// whose products run on limbs (limbs30).
+constexpr int kTensorSmallCode = 14;
 // Node shapes with exactly unrolled tensor kernels (children sorted by
 // tuple size, largest first; c = 0 for two children): two children of 4..7
 // terms (codes 0..9) except 6 and 4 (children of 5 and 3 inputs: no tree
 // within the depth rule has that node for k <= 16), three of 4 or 5 terms
-// (codes 10..13); -1 otherwise.
+// (codes 10..13); (2,2), (3,3), (2,2,2) and (3,3,2) (codes 14..17); -1
+// otherwise.
 __host__ __device__ inline int tensor_fixed_code(int m, int a, int b, int c) {
     if (m == 2 && b >= 4 && b <= a && a <= 7 && !(a == 6 && b == 4)) return (a - 4) * (a - 3) / 2 + (b - 4);
+    if (m == 2 && a == b && a <= 3) return kTensorSmallCode + a - 2;
+    if (m == 3 && a == b && a <= 3 && c == 2) return kTensorSmallCode + a;
     if (m == 3 && c >= 4 && c <= b && b <= a && a <= 5) return 10 + (a - 4) + (b - 4) + (c - 4);
     return -1;
 }
@@ -141,7 +143,7 @@ int tensor_sort_children(TensorJob &T);
 int tensor_sort_children(TensorArgs &A);
 // Uniform launch of a node of shape `code` (children sorted); the caller
 // counts and times it.
-cudaError_t launch_tensor_fixed(const Context &C, const TensorArgs &A, int code, cudaStream_t st);
+cudaError_t launch_tensor_fixed(const Context &C, const TensorArgs &A, int code, bool vec2, cudaStream_t st);
 // vec2: every entry's pointers are 16-byte aligned and its strides even
 // (tensor_job_vec2), so tuples of up to 5 terms may take two coefficients
 // per thread
@@ -150,7 +152,7 @@ cudaError_t launch_tensor_table(const Context &C, const TensorJob *jobs, int n_j
                                 bool vec2, double bytes, double ops, cudaStream_t st);
 // Table launch of nodes that all have the (sorted) shape `code`.
 cudaError_t launch_tensor_fixed_table(const Context &C, const TensorJob *jobs, int n_jobs, int code, int max_level,
-                                      double bytes, double ops, cudaStream_t st);
+                                      bool vec2, double bytes, double ops, cudaStream_t st);
 double tensor_products_per_coeff(const int *polys, int m);
 cudaError_t launch_rschain_table(const Context &C, const RsJob *jobs, int n_jobs, int max_polys, double bytes,
                                  cudaStream_t st);

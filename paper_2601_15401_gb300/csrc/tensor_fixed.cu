@@ -9,20 +9,20 @@
 // of the node issued before the first product, each output term stored as
 // soon as it is reduced. Shapes (tensor_fixed_code): two children of 4..7
 // terms, three of 4 or 5 terms — among them the roots and the larger inner
-// nodes of the paper's partitions for k = 6..12 (Table II).
+// nodes of the paper's partitions for k = 6..12 (Table II) — and, on limbs,
+// the small nodes: two or three ciphertexts, two children of 3 terms, alone or
+// with a ciphertext.
 //
 // Operands are reduced residues and no term sums more than 7 products, so
 // the 128-bit sums need no per-term reduction: B q^2 < q 2^64 for B <= 8
-// and q < 2^61 keeps the high word below q, as REDC requires.
+// and q < 2^61 keeps the high word below q, as REDC requires. With every
+// prime below 2^60 (LIMB) the products run on 30-bit limbs (DotLimbs, at most
+// 8 terms): three multiply-adds each.
 #include <utility>
 
 #include "common.cuh"
 #include "internal.h"
 #include "rns.h"
-
-#ifndef CKKS_TENSOR_PRESCALE
-#define CKKS_TENSOR_PRESCALE 1
-#endif
 
 namespace ckks {
 
@@ -30,92 +30,119 @@ namespace {
 
 constexpr int kThreads = 256;
 
-// z = x * y (polynomials in s of A and B terms), each term REDC-reduced
-template <int A, int B, bool Q1>
-__device__ __forceinline__ void conv_redc(const u64 (&x)[A], const u64 (&y)[B], u64 (&z)[A + B - 1], const ModQ m) {
-    static_assert(A >= B && B <= 8, "at most 8 products per term");
-#pragma unroll
-    for (int t = 0; t < A + B - 1; ++t) {
-        Acc128Lazy acc;
-        acc.zero();
-#pragma unroll
-        for (int b = 0; b < B; ++b)
-            if (t - b >= 0 && t - b < A) acc.mac(x[t - b], y[b]);
-        z[t] = redc_t<Q1>(acc.hi, acc.lo, m);
+// CTAs per SM the small shapes are compiled for (bound by HBM)
+#ifndef CKKS_TENSOR_SMALL_MINB
+#define CKKS_TENSOR_SMALL_MINB 3
+#endif
+
+// A residue as an operand of the dot products, itself or its limbs, and the
+// reduction of a sum of at most 8 products of residues. (The sums of limbs
+// are put together as 128-bit words for the REDC: reducing them by limbs, as
+// BConv does, took 155 against 137 us for two 4-term children, the final
+// subtractions costing more than the multiplies saved.)
+template <bool LIMB, bool Q1>
+struct Operand {
+    typedef u64 type;
+    typedef Acc128Lazy acc;
+    static __device__ __forceinline__ u64 make(u64 v) { return v; }
+    static __device__ __forceinline__ u64 reduce(const Acc128Lazy &a, const ModQ &m) { return redc_t<Q1>(a.hi, a.lo, m); }
+};
+template <bool Q1>
+struct Operand<true, Q1> {
+    typedef Limbs type;
+    typedef DotLimbs acc;
+    static __device__ __forceinline__ Limbs make(u64 v) { return split_limbs<30>(v); }
+    static __device__ __forceinline__ u64 reduce(const DotLimbs &a, const ModQ &m) {
+        u64 hi, lo;
+        a.value<30>(hi, lo);
+        return redc_t<Q1>(hi, lo, m);
     }
-}
+};
 
-// the same, each term stored at dst + t ds as soon as it is formed (with
-// CKKS_TENSOR_PRESCALE = 0 multiplied by the Shoup constant fix first)
-template <int A, int B, bool Q1>
-__device__ __forceinline__ void conv_redc_store(const u64 (&x)[A], const u64 (&y)[B], const ModQ m, const Shoup fix,
-                                                u64 *dst, i64 ds) {
+// term t of x * y (polynomials in s of A and B terms) at coefficient e, reduced
+template <int A, int B, int V, bool Q1, bool LIMB>
+__device__ __forceinline__ u64 conv_term(const typename Operand<LIMB, Q1>::type (&x)[A][V],
+                                         const typename Operand<LIMB, Q1>::type (&y)[B][V], int t, int e,
+                                         const ModQ m) {
     static_assert(A >= B && B <= 8, "at most 8 products per term");
+    typename Operand<LIMB, Q1>::acc acc;
+    acc.zero();
 #pragma unroll
-    for (int t = 0; t < A + B - 1; ++t) {
-        Acc128Lazy acc;
-        acc.zero();
-#pragma unroll
-        for (int b = 0; b < B; ++b)
-            if (t - b >= 0 && t - b < A) acc.mac(x[t - b], y[b]);
-        const u64 z = redc_t<Q1>(acc.hi, acc.lo, m);
-        dst[(i64)t * ds] = CKKS_TENSOR_PRESCALE ? z : shoup_t<Q1>(z, fix.w, fix.wp, m.q);
-    }
+    for (int b = 0; b < B; ++b)
+        if (t - b >= 0 && t - b < A) acc.mac(x[t - b][e], y[b][e]);
+    return Operand<LIMB, Q1>::reduce(acc, m);
 }
 
-template <int T>
-__device__ __forceinline__ void load_terms(const u64 *src, i64 ps, u64 (&o)[T]) {
+template <int T, int V>
+__device__ __forceinline__ void load_terms(const u64 *src, i64 ps, u64 (&o)[T][V]) {
 #pragma unroll
-    for (int a = 0; a < T; ++a) o[a] = src[(i64)a * ps];
+    for (int a = 0; a < T; ++a) load_span<V>(src + (i64)a * ps, o[a]);
 }
 
-// the terms of the last (smallest) child times R^(m-1)
-template <int T, bool Q1>
-__device__ __forceinline__ void prescale(u64 (&o)[T], const Shoup fix, u64 q) {
-    if (CKKS_TENSOR_PRESCALE)
-#pragma unroll
-        for (int a = 0; a < T; ++a) o[a] = shoup_t<Q1>(o[a], fix.w, fix.wp, q);
-}
-
-// One coefficient r (= limb j * N + coefficient) of a node with children of
-// A, B (and C; 0 for two children) terms: m - 1 Montgomery products, which
-// leave R^-(m-1), and R^(m-1) as a Shoup product by the per-prime constant
-// rfix[j][m] on the terms of the last child.
-template <int A, int B, int C, bool Q1, class View>
+// V adjacent coefficients r (= limb j * N + coefficient) of a node with
+// children of A, B (and C; 0 for two children) terms: m - 1 Montgomery
+// products, which leave R^-(m-1), and R^(m-1) as a Shoup product by a per-prime
+// constant on the terms of the last child.
+template <int A, int B, int C, int V, bool Q1, bool LIMB, class View>
 __device__ __forceinline__ void tensor_fixed_coeff(const View &v, i64 r, int j, const ModQ m, const Shoup *rfix) {
-    u64 x[A], y[B];
-    load_terms<A>(v.src(0) + r, v.pstride(0), x);
-    load_terms<B>(v.src(1) + r, v.pstride(1), y);
+    typedef Operand<LIMB, Q1> Op;
+    const Shoup fix = rfix[(i64)j * 16 + (C ? 3 : 2)];
+    constexpr int Z = A + B - 1, CC = C ? C : 1;
+    u64 x[A][V], y[B][V], w[CC][V];
+    load_terms<A, V>(v.src(0) + r, v.pstride(0), x);
+    load_terms<B, V>(v.src(1) + r, v.pstride(1), y);
+    if constexpr (C != 0) load_terms<C, V>(v.src(2) + r, v.pstride(2), w);
     u64 *dst = v.dst() + r;
     const i64 ds = v.dstride();
+    typename Op::type xo[A][V], yo[B][V];
+#pragma unroll
+    for (int e = 0; e < V; ++e) {
+#pragma unroll
+        for (int a = 0; a < A; ++a) xo[a][e] = Op::make(x[a][e]);
+#pragma unroll
+        for (int b = 0; b < B; ++b)
+            yo[b][e] = Op::make(C ? y[b][e] : shoup_t<Q1>(y[b][e], fix.w, fix.wp, m.q));
+    }
     if constexpr (C == 0) {
-        const Shoup fix = rfix[(i64)j * 16 + 2];
-        prescale<B, Q1>(y, fix, m.q);
-        conv_redc_store<A, B, Q1>(x, y, m, fix, dst, ds);
+#pragma unroll
+        for (int t = 0; t < Z; ++t) {
+            u64 o[V];
+#pragma unroll
+            for (int e = 0; e < V; ++e) o[e] = conv_term<A, B, V, Q1, LIMB>(xo, yo, t, e, m);
+            store_span<V>(dst + (i64)t * ds, o);
+        }
     } else {
-        const Shoup fix = rfix[(i64)j * 16 + 3];
-        u64 w[C];
-        load_terms<C>(v.src(2) + r, v.pstride(2), w);
-        u64 z[A + B - 1];
-        conv_redc<A, B, Q1>(x, y, z, m);
-        prescale<C, Q1>(w, fix, m.q);
-        conv_redc_store<A + B - 1, C, Q1>(z, w, m, fix, dst, ds);
+        typename Op::type zo[Z][V], wo[CC][V];
+#pragma unroll
+        for (int e = 0; e < V; ++e) {
+#pragma unroll
+            for (int t = 0; t < Z; ++t) zo[t][e] = Op::make(conv_term<A, B, V, Q1, LIMB>(xo, yo, t, e, m));
+#pragma unroll
+            for (int a = 0; a < CC; ++a) wo[a][e] = Op::make(shoup_t<Q1>(w[a][e], fix.w, fix.wp, m.q));
+        }
+#pragma unroll
+        for (int t = 0; t < Z + CC - 1; ++t) {
+            u64 o[V];
+#pragma unroll
+            for (int e = 0; e < V; ++e) o[e] = conv_term<Z, CC, V, Q1, LIMB>(zo, wo, t, e, m);
+            store_span<V>(dst + (i64)t * ds, o);
+        }
     }
 }
 
-template <int A, int B, int C, bool Q1>
-__global__ void __launch_bounds__(kThreads, 3) tensor_fixed_kernel(TensorArgs T) {
+template <int A, int B, int C, int V, bool Q1, bool LIMB>
+__global__ void __launch_bounds__(kThreads, A <= 3 ? CKKS_TENSOR_SMALL_MINB : A + B + C <= 8 ? 4 : 3) tensor_fixed_kernel(TensorArgs T) {
     grid_dependency_wait();
-    const i64 r = (i64)blockIdx.x * blockDim.x + threadIdx.x;  // limb * N + coefficient
+    const i64 r = ((i64)blockIdx.x * blockDim.x + threadIdx.x) * V;  // limb * N + coefficient
     if (r >= (i64)T.level * T.N) return;
     const int j = (int)(r >> T.log_n);
-    tensor_fixed_coeff<A, B, C, Q1>(TensorUniformView{T, (int)blockIdx.y}, r, j, T.mods[j], T.rfix);
+    tensor_fixed_coeff<A, B, C, V, Q1, LIMB>(TensorUniformView{T, (int)blockIdx.y}, r, j, T.mods[j], T.rfix);
 }
 
 // blockIdx.y = table entry (every entry of the launch has this shape); the
 // entry is staged in shared memory, one word per thread
-template <int A, int B, int C, bool Q1>
-__global__ void __launch_bounds__(kThreads, 3) tensor_fixed_table_kernel(const TensorJob *jobs, int N, int log_n,
+template <int A, int B, int C, int V, bool Q1, bool LIMB>
+__global__ void __launch_bounds__(kThreads, A <= 3 ? CKKS_TENSOR_SMALL_MINB : A + B + C <= 8 ? 4 : 3) tensor_fixed_table_kernel(const TensorJob *jobs, int N, int log_n,
                                                                         const ModQ *mods, const Shoup *rfix) {
     grid_dependency_wait();
     __shared__ TensorJob J;
@@ -127,10 +154,10 @@ __global__ void __launch_bounds__(kThreads, 3) tensor_fixed_table_kernel(const T
         for (int i = threadIdx.x; i < W; i += blockDim.x) dst[i] = src[i];
     }
     __syncthreads();
-    const i64 r = (i64)blockIdx.x * blockDim.x + threadIdx.x;
+    const i64 r = ((i64)blockIdx.x * blockDim.x + threadIdx.x) * V;
     if (r >= (i64)J.level * N) return;
     const int j = (int)(r >> log_n);
-    tensor_fixed_coeff<A, B, C, Q1>(TensorTableView{J}, r, j, mods[j], rfix);
+    tensor_fixed_coeff<A, B, C, V, Q1, LIMB>(TensorTableView{J}, r, j, mods[j], rfix);
 }
 
 // The shape of each code (tensor_fixed_code), as template arguments.
@@ -150,27 +177,53 @@ cudaError_t with_shape(int code, F &&f) {
     case 11: return f(std::integral_constant<int, 5>{}, std::integral_constant<int, 4>{}, std::integral_constant<int, 4>{});
     case 12: return f(std::integral_constant<int, 5>{}, std::integral_constant<int, 5>{}, std::integral_constant<int, 4>{});
     case 13: return f(std::integral_constant<int, 5>{}, std::integral_constant<int, 5>{}, std::integral_constant<int, 5>{});
+    case 14: return f(std::integral_constant<int, 2>{}, std::integral_constant<int, 2>{}, std::integral_constant<int, 0>{});
+    case 15: return f(std::integral_constant<int, 3>{}, std::integral_constant<int, 3>{}, std::integral_constant<int, 0>{});
+    case 16: return f(std::integral_constant<int, 2>{}, std::integral_constant<int, 2>{}, std::integral_constant<int, 2>{});
+    case 17: return f(std::integral_constant<int, 3>{}, std::integral_constant<int, 3>{}, std::integral_constant<int, 2>{});
     default: return cudaErrorInvalidValue;
     }
 }
 
-template <bool Q1>
-cudaError_t launch_uniform(const TensorArgs &T, int code, cudaStream_t st) {
-    dim3 blocks((unsigned)(((i64)T.level * T.N + kThreads - 1) / kThreads), T.n_batch);
+// Small tuples (up to 3 terms a child; only on limbs) take two adjacent
+// coefficients per thread where every pointer allows 16-byte accesses.
+template <int A, bool LIMB>
+constexpr bool kSmallShape = A <= 3 && LIMB;
+
+template <bool Q1, bool LIMB>
+cudaError_t launch_uniform(const TensorArgs &T, int code, bool vec2, cudaStream_t st) {
     return with_shape(code, [&](auto a, auto b, auto c) {
-        return launch_dependent(tensor_fixed_kernel<decltype(a)::value, decltype(b)::value, decltype(c)::value, Q1>,
-                                blocks, dim3(kThreads), 0, st, T);
+        constexpr int A = decltype(a)::value, B = decltype(b)::value, C = decltype(c)::value;
+        auto go = [&](auto kern, int V) {
+            const i64 per = (i64)kThreads * V;
+            dim3 blocks((unsigned)(((i64)T.level * T.N + per - 1) / per), T.n_batch);
+            return launch_dependent(kern, blocks, dim3(kThreads), 0, st, T);
+        };
+        if constexpr (A <= 3 && !LIMB) return cudaErrorInvalidValue;
+        else {
+            if constexpr (kSmallShape<A, LIMB>)
+                if (vec2) return go(tensor_fixed_kernel<A, B, C, 2, Q1, LIMB>, 2);
+            return go(tensor_fixed_kernel<A, B, C, 1, Q1, LIMB>, 1);
+        }
     });
 }
 
-template <bool Q1>
-cudaError_t launch_table(const Context &C, const TensorJob *jobs, int n_jobs, int code, int max_level,
+template <bool Q1, bool LIMB>
+cudaError_t launch_table(const Context &C_, const TensorJob *jobs, int n_jobs, int code, int max_level, bool vec2,
                          cudaStream_t st) {
-    dim3 blocks((unsigned)(((i64)max_level * C.N + kThreads - 1) / kThreads), (unsigned)n_jobs);
     return with_shape(code, [&](auto a, auto b, auto c) {
-        return launch_dependent(
-            tensor_fixed_table_kernel<decltype(a)::value, decltype(b)::value, decltype(c)::value, Q1>, blocks,
-            dim3(kThreads), 0, st, jobs, C.N, C.log_n, C.d_mods, C.d_rfix);
+        constexpr int A = decltype(a)::value, B = decltype(b)::value, C = decltype(c)::value;
+        auto go = [&](auto kern, int V) {
+            const i64 per = (i64)kThreads * V;
+            dim3 blocks((unsigned)(((i64)max_level * C_.N + per - 1) / per), (unsigned)n_jobs);
+            return launch_dependent(kern, blocks, dim3(kThreads), 0, st, jobs, C_.N, C_.log_n, C_.d_mods, C_.d_rfix);
+        };
+        if constexpr (A <= 3 && !LIMB) return cudaErrorInvalidValue;
+        else {
+            if constexpr (kSmallShape<A, LIMB>)
+                if (vec2) return go(tensor_fixed_table_kernel<A, B, C, 2, Q1, LIMB>, 2);
+            return go(tensor_fixed_table_kernel<A, B, C, 1, Q1, LIMB>, 1);
+        }
     });
 }
 
@@ -197,18 +250,20 @@ int tensor_sort_children(TensorArgs &A) {
     return tensor_fixed_code(A.m, A.child_polys[0], A.child_polys[1], A.m > 2 ? A.child_polys[2] : 0);
 }
 
-cudaError_t launch_tensor_fixed(const Context &C, const TensorArgs &A, int code, cudaStream_t st) {
-    return C.q1() ? launch_uniform<true>(A, code, st) : launch_uniform<false>(A, code, st);
+cudaError_t launch_tensor_fixed(const Context &C, const TensorArgs &A, int code, bool vec2, cudaStream_t st) {
+    if (!C.limbs30) return launch_uniform<false, false>(A, code, vec2, st);
+    return C.q1() ? launch_uniform<true, true>(A, code, vec2, st) : launch_uniform<false, true>(A, code, vec2, st);
 }
 
 cudaError_t launch_tensor_fixed_table(const Context &C, const TensorJob *jobs, int n_jobs, int code, int max_level,
-                                      double bytes, double ops, cudaStream_t st) {
+                                      bool vec2, double bytes, double ops, cudaStream_t st) {
     if (n_jobs <= 0) return cudaSuccess;
     if (n_jobs > 65535) return cudaErrorInvalidValue;
     count_kernel(C);
     ProfScope ps(C, KC_TENSOR, bytes, st, ops);
-    return C.q1() ? launch_table<true>(C, jobs, n_jobs, code, max_level, st)
-                  : launch_table<false>(C, jobs, n_jobs, code, max_level, st);
+    if (!C.limbs30) return launch_table<false, false>(C, jobs, n_jobs, code, max_level, vec2, st);
+    return C.q1() ? launch_table<true, true>(C, jobs, n_jobs, code, max_level, vec2, st)
+                  : launch_table<false, true>(C, jobs, n_jobs, code, max_level, vec2, st);
 }
 
 }  // namespace ckks

@@ -252,7 +252,8 @@ void build_product(Builder &B, const WaveProduct &w, Bump &ws) {
         int cls = maxt <= 3 ? 0 : maxt <= 4 ? 1 : maxt <= 5 ? 2 : maxt <= 7 ? 3 : maxt <= 9 ? 4 : 5;
         // children sorted by size, largest first (the smallest, last, takes
         // the R^(m-1) correction)
-        if (tensor_sort_children(T) >= 0 && C.tune_tensor_fixed) cls = 6;
+        const int code = tensor_sort_children(T);
+        if (code >= 0 && C.tune_tensor_fixed && (code < kTensorSmallCode || C.limbs30)) cls = 6;
         if (emit) {
             Stage &s = B.at(round, cls, SK_TENSOR);
             s.fixed = cls == 6;
@@ -574,7 +575,7 @@ cudaError_t enqueue(ckks_wave &W, char *ws /* the job tables */, cudaStream_t st
             if (s.fixed) {
                 for (const Stage::FixedRun &r : s.runs) {
                     e = launch_tensor_fixed_table(C, (const TensorJob *)(ws + s.off) + r.first, r.count, r.code,
-                                                  r.max_level, r.bytes, r.ops, st);
+                                                  r.max_level, s.vec2, r.bytes, r.ops, st);
                     if (e != cudaSuccess) break;
                 }
             } else
