@@ -130,7 +130,7 @@ int context_build(Context &C, const uint32_t log_n, const uint32_t L, const uint
     std::vector<Shoup> ninv(NP), one(NP);
     std::vector<u64> r2(NP), keyfold(NP);
     std::vector<Shoup> rfix((size_t)NP * 16);
-    std::vector<u64> cK((size_t)NP * CKKS_MAX_PRIMES, 0);
+    std::vector<u64> cK((size_t)NP * CKKS_MAX_PRIMES, 0), cK60(cK);
     std::vector<Shoup> invq((size_t)CKKS_MAX_PRIMES * CKKS_MAX_PRIMES);
     std::vector<Shoup> pscale(C.K);
     std::vector<Shoup> pgadget((size_t)C.dnum * NP);
@@ -177,7 +177,11 @@ int context_build(Context &C, const uint32_t log_n, const uint32_t L, const uint
         for (int i = 0; i < C.K; ++i) Pm = h_mul(Pm, p[i] % m, m);
         keyfold[x] = x < C.L ? h_mul(h_inv(Pm, m), r2[x], m) : r2[x];
         if (x < C.L) {
-            for (int i = 0; i < C.K; ++i) cK[(size_t)x * CKKS_MAX_PRIMES + i] = h_mul(h_inv(p[i] % m, m), R, m);
+            for (int i = 0; i < C.K; ++i) {
+                const u64 inv = h_inv(p[i] % m, m);
+                cK[(size_t)x * CKKS_MAX_PRIMES + i] = h_mul(inv, R, m);
+                cK60[(size_t)x * CKKS_MAX_PRIMES + i] = h_mul(inv, (1ull << 60) % m, m);
+            }
             for (int b = 0; b < C.dnum; ++b) {
                 bool in_digit = x / C.alpha == b;
                 pgadget[(size_t)b * NP + x] = h_shoup(in_digit ? Pm : 0, m);
@@ -261,6 +265,7 @@ int context_build(Context &C, const uint32_t log_n, const uint32_t L, const uint
         {one.data(), one.size() * sizeof(Shoup), (void **)&C.d_one},
         {pscale.data(), pscale.size() * sizeof(Shoup), (void **)&C.d_pscale},
         {cK.data(), cK.size() * sizeof(u64), (void **)&C.d_cK},
+        {cK60.data(), cK60.size() * sizeof(u64), (void **)&C.d_cK60},
         {r2.data(), r2.size() * sizeof(u64), (void **)&C.d_r2},
         {rfix.data(), rfix.size() * sizeof(Shoup), (void **)&C.d_rfix},
         {keyfold.data(), keyfold.size() * sizeof(u64), (void **)&C.d_keyfold},

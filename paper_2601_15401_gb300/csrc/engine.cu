@@ -394,11 +394,24 @@ static cudaError_t relin_core(const Context &C, Ws &ws, int B, int n, int level,
             // keys of the separate form add to C* in place
             LimbJobs J = jobs(B, 2, level);
             LoadSpec L{};
-            L.mode = LD_BCONVK;
-            L.b = zv;
-            L.mods = C.d_mods;
-            L.cK = C.d_cK;
-            L.K = K;
+            // The scaled BConv as a kernel of its own, into the ModUp outputs'
+            // buffer (the first key's, free after its products), where it is large enough:
+            // it reads the K limbs z once for all targets. Fused into the
+            // transform's load every target limb reads them again (768 limbs
+            // at N = 2^16, K = 8: 661 us, against 227 for a plain load).
+            const bool own = C.limbs30 && K <= 16 && nd * ext_l >= 2 * level;
+            if (own) {
+                const LimbView wv = view(ext, ev.bstride, (i64)level * N);
+                TRY(launch_moddown_conv(C, zv, wv, B, level, st));
+                L.mode = LD_PLAIN;
+                L.a = wv;
+            } else {
+                L.mode = LD_BCONVK;
+                L.b = zv;
+                L.mods = C.d_mods;
+                L.cK = C.d_cK;
+                L.K = K;
+            }
             StoreSpec S{};
             S.mode = ST_ADDSUB;
             S.dst = cstar;

@@ -129,6 +129,7 @@ struct Context {
     Shoup *d_one = nullptr;           // [L+K]   (1, floor(2^64/q)): x mod q for any x
     Shoup *d_pscale = nullptr;        // [K]     N^-1 [phat_i^-1]_{p_i}
     u64 *d_cK = nullptr;              // [L+K][64]: row j < L: [p_i^-1 R]_{q_j}
+    u64 *d_cK60 = nullptr;            // the same with R = 2^60 (products on limbs)
     u64 *d_r2 = nullptr;              // [L+K]   R^2 mod q
     Shoup *d_rfix = nullptr;          // [L+K][16] R^(e-1) mod q (Shoup), e >= 1
     u64 *d_keyfold = nullptr;         // [L+K]   Q limbs: P^-1 R^2, P limbs: R^2 (mod prime)
@@ -145,7 +146,7 @@ struct Context {
     Profiler prof;
     // launch tunables
     int tune_ntt_tile_cols = 4096;    // elements per CTA tile, column phases
-    int tune_ntt_tile_blocks = 4096;  // elements per CTA tile, block phases (at most kBlockTile are used)
+    int tune_ntt_tile_blocks = 4096;  // elements per CTA tile, block phases (at most kBlockTile, ntt.cu)
     int tune_bconv_threads = 256;
     int tune_mac_threads = 256;
     // forms of the rescaling (same results; for measuring the paper's
@@ -165,7 +166,7 @@ struct Context {
     // exactly unrolled kernels for that shape; 0 = the bounded generic kernels
     int tune_tensor_fixed = 1;
     // every prime (Q and P) is 1 (mod 2^32): the kernels can then take the
-    // cheaper forms of the Shoup product and of REDC (shoup_lazy_q1,
+    // cheaper forms of the Shoup product and of REDC (remainder_mad<true>,
     // redc_q1); set at creation. tune_q1 = 0 keeps the general forms.
     bool primes_q1 = false;
     // every prime is below 2^60: dot products run on 30-bit limbs (DotLimbs)

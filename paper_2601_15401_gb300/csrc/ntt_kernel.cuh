@@ -823,7 +823,10 @@ static inline cudaError_t dispatch_whole_n(const NttPhase &P, const LimbJobs *J,
             CKKS_MODES(LD_SIGNED, ST_REDUCE) CKKS_LAUNCH(LG, 0, WHOLE, LD_SIGNED, ST_REDUCE, 2, false);
         CKKS_MODES(LD_EQ17, ST_REDUCE) CKKS_LAUNCH(LG, 0, WHOLE, LD_EQ17, ST_REDUCE, 2, false);
         CKKS_MODES(LD_EQ17, ST_MRS) CKKS_LAUNCH(LG, 0, WHOLE, LD_EQ17, ST_MRS, 2, false);
-        CKKS_MODES(LD_BCONVK, ST_ADDSUB) CKKS_LAUNCH(LG, 0, WHOLE, LD_BCONVK, ST_ADDSUB, 2, false);
+        if constexpr (!TABLE) {
+            CKKS_MODES(LD_BCONVK, ST_ADDSUB) CKKS_LAUNCH(LG, 0, WHOLE, LD_BCONVK, ST_ADDSUB, 2, false);
+            CKKS_MODES(LD_PLAIN, ST_ADDSUB) CKKS_LAUNCH(LG, 0, WHOLE, LD_PLAIN, ST_ADDSUB, 2, false);
+        }
     } else {
         CKKS_MODES(LD_PLAIN, ST_SCALE) CKKS_LAUNCH(LG, 0, WHOLE, LD_PLAIN, ST_SCALE, 2, false);
         CKKS_MODES(LD_ADD, ST_MODDOWN) CKKS_LAUNCH(LG, 0, WHOLE, LD_ADD, ST_MODDOWN, 2, false);

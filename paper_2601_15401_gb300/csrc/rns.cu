@@ -392,21 +392,27 @@ __device__ __forceinline__ int key_limb_bits(u64 q, int key_digits) {
 // constant is one 8-byte word (its limbs' sum is added up again) and serves
 // CKKS_BCONV_VEC coefficients. Otherwise (a prime of 2^60 or more)
 // 64 x 64 -> 128-bit products.
+// One conversion: na source limbs (N apart from y0, primes from index src0)
+// to the Q limbs [0, d0) and [d0 + skip, level), then n_p P limbs; the
+// constant of (source jj, prime x) at ctab[jj cj + x cx].
+struct Conversion {
+    const u64 *ctab;
+    int cj, cx;
+    const u64 *y0;
+    int na, src0;
+    u64 *dst0;
+    int level, d0, skip, n_p, L;
+};
+
 template <int AMAX, bool Q1, bool LIMB>
-__device__ __forceinline__ void bconv_block(const u64 *ctab, const u64 *y0, u64 *dst0, int level, int beta,
-                                            int alpha, int L, int K, int n_primes, int N, const ModQ *mods,
-                                            u64 *cs) {
-    const int d0 = beta * alpha;
-    int d1 = d0 + alpha;
-    if (d1 > level) d1 = level;
-    const int na = d1 - d0;
-    // targets: Q limbs outside the digit, then every P limb
-    const int nq_t = level - na;
-    const int n_t = nq_t + K;
+__device__ __forceinline__ void bconv_block(const Conversion &B, int N, const ModQ *mods, u64 *cs) {
+    const int na = B.na, level = B.level;
+    const int nq_t = level - B.skip, n_t = nq_t + B.n_p;
+    auto slot_of = [&](int ti) { return ti < nq_t ? (ti < B.d0 ? ti : ti + B.skip) : level + (ti - nq_t); };
+    auto prime_of = [&](int ti) { return ti < nq_t ? (ti < B.d0 ? ti : ti + B.skip) : B.L + (ti - nq_t); };
     for (int i = threadIdx.x; i < na * n_t; i += blockDim.x) {
         int jj = i / n_t, ti = i % n_t;
-        int x = ti < nq_t ? (ti < d0 ? ti : ti + na) : L + (ti - nq_t);
-        const u64 c = ctab[(i64)jj * n_primes + x];
+        const u64 c = B.ctab[(i64)jj * B.cj + (i64)prime_of(ti) * B.cx];
         cs[ti * AMAX + jj] = LIMB ? pack_limbs<30>(c) : c;
     }
     // the products run over AMAX sources, the ones the digit does not have as zeros
@@ -416,11 +422,11 @@ __device__ __forceinline__ void bconv_block(const u64 *ctab, const u64 *y0, u64 
     constexpr int V = CKKS_BCONV_VEC;
     const int e = (blockIdx.x * blockDim.x + threadIdx.x) * V;
     if (e >= N) return;
-    const u64 *ysrc = y0 + e;
+    const u64 *ysrc = B.y0 + e;
     u64 y[AMAX][V];
 #pragma unroll
     for (int jj = 0; jj < AMAX; ++jj) {
-        if (jj < na) load_span<V>(ysrc + (i64)(d0 + jj) * N, y[jj]);
+        if (jj < na) load_span<V>(ysrc + (i64)jj * N, y[jj]);
         else
 #pragma unroll
             for (int v = 0; v < V; ++v) y[jj][v] = 0ull;
@@ -432,14 +438,13 @@ __device__ __forceinline__ void bconv_block(const u64 *ctab, const u64 *y0, u64 
         for (int jj = 0; jj < AMAX; ++jj) {
 #pragma unroll
             for (int v = 0; v < V; ++v) yl[jj][v] = split_limbs<30>(y[jj][v]);
-            if (jj < na) wide = wide || !small_prime(mods[d0 + jj].q);
+            if (jj < na) wide = wide || !small_prime(mods[B.src0 + jj].q);
         }
     }
-    u64 *dst = dst0 + e;
+    u64 *dst = B.dst0 + e;
     for (int ti = 0; ti < n_t; ++ti) {
-        const int slot = ti < nq_t ? (ti < d0 ? ti : ti + na) : level + (ti - nq_t);
-        const int x = ti < nq_t ? slot : L + (ti - nq_t);
-        const ModQ m = mods[x];
+        const int slot = slot_of(ti);
+        const ModQ m = mods[prime_of(ti)];
         // sum over the digit: hi stays below q because the digit's primes sum to < 2^64
         u64 r[V];
         if constexpr (LIMB) {
@@ -488,6 +493,13 @@ __device__ __forceinline__ void bconv_block(const u64 *ctab, const u64 *y0, u64 
     }
 }
 
+// ModUp of digit beta of d_t (limb 0 at y) into the (t, digit) output at ext
+__device__ __forceinline__ Conversion modup_conversion(const u64 *consts, const u64 *y, u64 *ext, int level, int beta,
+                                                       int alpha, int L, int K, int n_primes, int N) {
+    const int d0 = beta * alpha, d1 = d0 + alpha < level ? d0 + alpha : level;
+    return Conversion{consts, n_primes, 1, y + (i64)d0 * N, d1 - d0, d0, ext, level, d0, d1 - d0, K, L};
+}
+
 template <int AMAX, bool Q1, bool LIMB>
 __global__ void __launch_bounds__(CKKS_BCONV_MAX_THREADS, CKKS_BCONV_MINB) bconv_kernel(BconvArgs A) {
     extern __shared__ u64 cs[];  // [n_targets][AMAX] Montgomery constants
@@ -495,20 +507,34 @@ __global__ void __launch_bounds__(CKKS_BCONV_MAX_THREADS, CKKS_BCONV_MINB) bconv
     const int b = blockIdx.z;
     const int t = job / A.n_digits;
     const int beta = job % A.n_digits;
-    bconv_block<AMAX, Q1, LIMB>(A.consts + (i64)beta * A.alpha * A.n_primes,
-                      A.y.ptr + (i64)b * A.y.bstride + (i64)t * A.y.pstride,
-                      A.ext.ptr + (i64)b * A.ext.bstride + (i64)(t * A.n_digits + beta) * A.ext.pstride, A.level, beta,
-                      A.alpha, A.L, A.K, A.n_primes, A.N, A.mods, cs);
+    bconv_block<AMAX, Q1, LIMB>(
+        modup_conversion(A.consts + (i64)beta * A.alpha * A.n_primes,
+                         A.y.ptr + (i64)b * A.y.bstride + (i64)t * A.y.pstride,
+                         A.ext.ptr + (i64)b * A.ext.bstride + (i64)(t * A.n_digits + beta) * A.ext.pstride, A.level,
+                         beta, A.alpha, A.L, A.K, A.n_primes, A.N),
+        A.N, A.mods, cs);
 }
 
 // Table launch: blockIdx.y = (product, d_t, digit) entry.
 template <int AMAX, bool Q1, bool LIMB>
-__global__ void __launch_bounds__(CKKS_BCONV_MAX_THREADS, CKKS_BCONV_MINB) bconv_table_kernel(const BconvJob *jobs, int alpha, int L, int K,
-                                                           int n_primes, int N, const ModQ *mods) {
-    grid_dependency_wait();
+__global__ void __launch_bounds__(CKKS_BCONV_MAX_THREADS, CKKS_BCONV_MINB)
+    bconv_table_kernel(const BconvJob *jobs, int alpha, int L, int K, int n_primes, int N, const ModQ *mods) {
     extern __shared__ u64 cs[];
+    grid_dependency_wait();
     const BconvJob J = jobs[blockIdx.y];
-    bconv_block<AMAX, Q1, LIMB>(J.consts, J.y, J.ext, J.level, J.beta, alpha, L, K, n_primes, N, mods, cs);
+    bconv_block<AMAX, Q1, LIMB>(modup_conversion(J.consts, J.y, J.ext, J.level, J.beta, alpha, L, K, n_primes, N), N,
+                                mods, cs);
+}
+
+// Scaled BConv of ModDown (Eq. 12): the K limbs z of polynomial blockIdx.y of
+// batch element blockIdx.z into `level` Q limbs of out.
+template <int AMAX>
+__global__ void __launch_bounds__(CKKS_BCONV_MAX_THREADS, CKKS_BCONV_MINB)
+    moddown_conv_kernel(LimbView z, LimbView out, const u64 *cK, int level, int L, int K, int N, const ModQ *mods) {
+    extern __shared__ u64 cs[];
+    const Conversion B{cK, 1, CKKS_MAX_PRIMES, z.ptr + (i64)blockIdx.z * z.bstride + (i64)blockIdx.y * z.pstride, K, L,
+                       out.ptr + (i64)blockIdx.z * out.bstride + (i64)blockIdx.y * out.pstride, level, level, 0, 0, L};
+    bconv_block<AMAX, false, true>(B, N, mods, cs);
 }
 
 // sources the kernel for digits of alpha primes is unrolled to
@@ -530,6 +556,23 @@ static void launch_bconv_table_sized(const Context &C, dim3 grid, int thr, size_
     else if (a <= 8) launch_dependent(bconv_table_kernel<8, Q1, LIMB>, grid, dim3(thr), smem, st, jobs, a, C.L, C.K, np, C.N, C.d_mods);
     else if (a <= 12) launch_dependent(bconv_table_kernel<12, Q1, LIMB>, grid, dim3(thr), smem, st, jobs, a, C.L, C.K, np, C.N, C.d_mods);
     else launch_dependent(bconv_table_kernel<16, Q1, LIMB>, grid, dim3(thr), smem, st, jobs, a, C.L, C.K, np, C.N, C.d_mods);
+}
+
+cudaError_t launch_moddown_conv(const Context &C, LimbView z, LimbView out, int batch, int level, cudaStream_t st) {
+    const int thr = std::min(C.tune_bconv_threads, CKKS_BCONV_MAX_THREADS), per = thr * CKKS_BCONV_VEC;
+    dim3 grid((C.N + per - 1) / per, 2, batch);
+    const size_t smem = (size_t)bconv_sources(C.K) * level * sizeof(u64);
+    count_kernel(C);
+    ProfScope ps(C, KC_BCONV, 2.0 * batch * (C.K + level) * C.N * sizeof(u64), st, 2.0 * batch * C.K * level * (double)C.N);
+    auto go = [&](auto kern) {
+        return launch_dependent(kern, grid, dim3(thr), smem, st, z, out, C.d_cK60, level, C.L, C.K, C.N, C.d_mods);
+    };
+    switch (bconv_sources(C.K)) {
+    case 4: return go(moddown_conv_kernel<4>);
+    case 8: return go(moddown_conv_kernel<8>);
+    case 12: return go(moddown_conv_kernel<12>);
+    default: return go(moddown_conv_kernel<16>);
+    }
 }
 
 cudaError_t launch_bconv(const Context &C, const BconvArgs &A, cudaStream_t st) {

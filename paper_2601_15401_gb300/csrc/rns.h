@@ -162,6 +162,9 @@ cudaError_t launch_bconv_table(const Context &C, const BconvJob *jobs, int n_job
 cudaError_t launch_mac_table(const Context &C, const MacJob *jobs, const MacTarget *targets, int n_pairs,
                              int n_targets, const u64 *keys, double bytes, double macs, cudaStream_t st);
 cudaError_t launch_bconv(const Context &C, const BconvArgs &A, cudaStream_t st);
+// ModDown's scaled BConv of two polynomials: z [batch][2][K] -> out [batch][2][level]
+// (16-byte aligned); only with products on limbs (limbs30) and K <= 16
+cudaError_t launch_moddown_conv(const Context &C, LimbView z, LimbView out, int batch, int level, cudaStream_t st);
 cudaError_t launch_mac(const Context &C, const MacArgs &A, cudaStream_t st);
 cudaError_t launch_rschain(const Context &C, const RsChainArgs &A, cudaStream_t st);
 cudaError_t launch_keyprep(const Context &C, u64 *keys, long long n_rows, cudaStream_t st);
