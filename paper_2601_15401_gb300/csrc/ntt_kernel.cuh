@@ -32,10 +32,11 @@
 //     2^60 on the sums are folded every second stage); inverse sums are
 //     folded to |x| <= q at every stage.
 //
-// Twiddles: tw[prime][k] = (psi^brv(k), companion) for the forward,
-// psi^-brv(k) for the inverse. The stage with m groups uses tw[m + i] for
-// group i; in the block phase the global group index is b m_loc + i_loc and
-// m = N1 m_loc, so the index is m_loc (N1 + b) + i_loc.
+// Twiddles: psi^brv(k) with its companion for the forward, psi^-brv(k) for the
+// inverse. The stage with m groups uses k = m + i for group i; in the block
+// phase the global group index is b m_loc + i_loc and m = N1 m_loc, so
+// k = m_loc (N1 + b) + i_loc. The table holds them in the order the passes read
+// them (below).
 //
 // Element-wise work is fused into the global <-> shared copies: the load side
 // can add two limbs or form the rescale combination of Eq. 17; the store side
@@ -43,12 +44,17 @@
 // Eq. 11/12) or finish Algorithm 1 (A' = g A - B).
 //
 // Template parameters LM / SM fix the load / store mode at compile time
-// (-1: read from the launch's spec at run time). A fixed mode keeps only the
-// pointers and constants that mode uses alive, which is what lets the
-// specialised kernels fit three CTAs per SM. JOBS selects where a CTA finds
-// its limb: from the launch's uniform batch x polynomial x limb description
-// (LimbJobs), or from a device table of NttJob entries (limbs of different
-// products, levels and tree nodes in one launch).
+// (-1: read from the launch's spec at run time, N <= 2^8 only). A fixed mode
+// keeps only the pointers and constants that mode uses alive, which is what
+// lets the column kernels fit three or four CTAs per SM. A CTA finds its limb in
+// the launch's uniform batch x polynomial x limb description (LimbJobs) or in a
+// device table of NttJob entries (limbs of different products, levels and tree
+// nodes in one launch).
+//
+// Bound by the integer multiply pipe: 74-81 % busy in the four phases of 384
+// limbs at N = 2^16 (116 / 129 us forward columns / blocks, 122 / 140 inverse
+// blocks / columns; 163 / 172 / 166 / 188 with the exact-quotient butterflies and
+// run-time tiles before).
 #pragma once
 #include "common.cuh"
 #include "internal.h"
@@ -197,15 +203,11 @@ __device__ __forceinline__ u64 eq17_sub(u64 r, u64 s, u64 q) {
 // any signed 64-bit integer mod q (canonical); `one`: the constant 1
 template <bool Q1>
 __device__ __forceinline__ u64 signed_mod(u64 v, Shoup one, u64 q) {
-    // beyond the product's range (|v| < 2^63 - 2^33) v = 4 (v >> 2) + (v & 3)
-    const bool far = (i64)(v ^ (v << 1)) < 0;  // |v| >= 2^62
-    u64 r = shoup_t<Q1>(far ? (u64)((i64)v >> 2) : v, one.w, one.wp, q);
-    if (far) {
-        r = add_mod(r, r, q);
-        r = add_mod(r, r, q);
-        r = add_mod(r, shoup_t<Q1>(v & 3, one.w, one.wp, q), q);
-    }
-    return r;
+    // v = 4 (v >> 2) + (v & 3): v itself may be beyond the product's range
+    u64 r = shoup_t<Q1>((u64)((i64)v >> 2), one.w, one.wp, q);
+    r = add_mod(r, r, q);
+    r = add_mod(r, r, q);
+    return add_mod(r, shoup_t<Q1>(v & 3, one.w, one.wp, q), q);
 }
 
 // out[u] = sum_i z_i[u DIST] c_i R^-1 mod q over the K limbs z_i (N apart) of the
@@ -413,6 +415,37 @@ __device__ __forceinline__ void load_set(u64 (&x)[EL], const LoadCtx &lc, int e)
 #pragma unroll
             for (int k = 0; k < EL; ++k)
                 x[k] = eq17_sub<SMALL>(shoup_signed<Q1>(lc.a[e + k * DIST], g.w, g.wp, q), x[k], q);
+        }
+    } else if constexpr (LM == LD_SIGNED) {
+        // all words first: one test says whether every sum is within the
+        // product's range (|a|, |b| < 2^61, as errors and messages are), so the
+        // reductions run side by side (a test per word: 14.5 us for a secret's
+        // two limbs at N = 2^15)
+        const u64 q = lc.m.q;
+        const Shoup one = *lc.g;
+        u64 out = 0;
+#pragma unroll
+        for (int k = 0; k < EL; ++k) {
+            x[k] = lc.a[e + k * DIST];
+            out |= x[k] + (1ull << 61);
+        }
+        if (lc.b) {
+#pragma unroll
+            for (int k = 0; k < EL; ++k) {
+                const u64 y = lc.b[e + k * DIST];
+                out |= y + (1ull << 61);
+                x[k] += y;
+            }
+        }
+        if ((out >> 62) == 0) {
+#pragma unroll
+            for (int k = 0; k < EL; ++k) {
+                const u64 r = shoup_signed<Q1>(x[k], one.w, one.wp, q);
+                x[k] = SMALL ? r : lift_sign(r, q);
+            }
+        } else {
+#pragma unroll
+            for (int k = 0; k < EL; ++k) x[k] = load_elem<LM, SMALL, Q1>(lc, e + k * DIST);
         }
     } else if constexpr (LM == LD_BCONVK) {
         constexpr int G = EL >= CKKS_NTT_MODDOWN_GROUP ? CKKS_NTT_MODDOWN_GROUP : EL;
@@ -709,11 +742,11 @@ struct PhaseLaunch {
 #define CKKS_NTT_COL_MINB 4     // columns: 64 registers (871 vs 842 G butterflies/s with three CTAs, 736 with two)
 #endif
 #ifndef CKKS_NTT_COL_WIDE_MINB
-#define CKKS_NTT_COL_WIDE_MINB 4  // columns with an Eq. 17 or signed load (411 -> 393 us per k = 12, batch 8 launch
+#define CKKS_NTT_COL_WIDE_MINB 4  // columns with an Eq. 17 load (411 -> 393 us per k = 12, batch 8 launch
                                   // against three CTAs)
 #endif
 #ifndef CKKS_NTT_COL_MODDOWN_MINB
-#define CKKS_NTT_COL_MODDOWN_MINB 3  // columns whose store sums over the K z-limbs: 80 registers
+#define CKKS_NTT_COL_MODDOWN_MINB 3  // columns with a signed load or a store that sums over the K z-limbs: 80 registers
 #endif
 #ifndef CKKS_NTT_COL_BCONVK_MINB
 #define CKKS_NTT_COL_BCONVK_MINB 2  // columns whose load sums over the K z-limbs: 128 registers
@@ -774,7 +807,7 @@ static inline cudaError_t dispatch_cols(const NttPhase &P, const LimbJobs *J, co
         CKKS_MODES(LD_EQ17, ST_LAZY) CKKS_LAUNCH(LG, LG2, COLS, LD_EQ17, ST_LAZY, CKKS_NTT_COL_WIDE_MINB, Q1);
         CKKS_MODES(LD_BCONVK, ST_LAZY) CKKS_LAUNCH(LG, LG2, COLS, LD_BCONVK, ST_LAZY, CKKS_NTT_COL_BCONVK_MINB, Q1);
         if constexpr (!TABLE)
-            CKKS_MODES(LD_SIGNED, ST_LAZY) CKKS_LAUNCH(LG, LG2, COLS, LD_SIGNED, ST_LAZY, CKKS_NTT_COL_WIDE_MINB, Q1);
+            CKKS_MODES(LD_SIGNED, ST_LAZY) CKKS_LAUNCH(LG, LG2, COLS, LD_SIGNED, ST_LAZY, CKKS_NTT_COL_MODDOWN_MINB, Q1);
     } else {
         CKKS_MODES(LD_PLAIN, ST_SCALE) CKKS_LAUNCH(LG, LG2, COLS, LD_PLAIN, ST_SCALE, CKKS_NTT_COL_MINB, Q1);
         CKKS_MODES(LD_PLAIN, ST_MODDOWN) CKKS_LAUNCH(LG, LG2, COLS, LD_PLAIN, ST_MODDOWN, CKKS_NTT_COL_MODDOWN_MINB, Q1);
