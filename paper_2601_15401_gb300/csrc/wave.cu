@@ -488,8 +488,12 @@ int build(ckks_wave &W, char *scratch, std::vector<char> &tables) {
         if (s.kind == SK_NTT) {
             // limbs of one prime next to each other: neighbouring CTAs read
             // the same twiddles
-            std::stable_sort(s.ntt.begin(), s.ntt.end(),
-                             [](const NttJob &a, const NttJob &b) { return a.prime < b.prime; });
+            size_t at[CKKS_MAX_PRIMES + 1] = {0};
+            for (const NttJob &j : s.ntt) ++at[j.prime + 1];
+            for (int x = 0; x < CKKS_MAX_PRIMES; ++x) at[x + 1] += at[x];
+            std::vector<NttJob> sorted(s.ntt.size());
+            for (const NttJob &j : s.ntt) sorted[at[j.prime]++] = j;
+            s.ntt.swap(sorted);
             s.off = put(tables, s.ntt);
         }
         if (s.kind == SK_TENSOR && s.fixed) {
