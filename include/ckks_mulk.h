@@ -113,8 +113,8 @@ int ckks_keygen_evk(ckks_context *ctx, uint32_t t_max, const int64_t *s, const u
 /* ckks_evk_set_create: adopts a key buffer in the layout above for
  * t = 2..t_max; the buffer must be 16-byte aligned (CKKS_EINVAL otherwise:
  * the key MAC reads it with 16-byte loads). The buffer is converted IN
- * PLACE to the library's internal form (Montgomery form; P^-1 folded into
- * the Q rows, Eq. 12) and is borrowed until ckks_evk_set_destroy; do not
+ * PLACE to the library's internal form (Montgomery form, P^-1 folded into
+ * the Q rows, Eq. 12, each word split into two limbs) and is borrowed until ckks_evk_set_destroy; do not
  * read it as plain keys after. */
 int ckks_evk_set_create(ckks_context *ctx, uint32_t t_max, uint64_t *keys, void *stream, ckks_evk_set **out);
 void ckks_evk_set_destroy(ckks_evk_set *set);
@@ -446,10 +446,11 @@ int ckks_pull(void *dst, const void *src, size_t bytes, int blocks, void *stream
  * multiple of 32, at most 256) that each run ckks_peak_chains() independent
  * chains of `iters` operations of one kind on registers only, and write one
  * word per thread to `out` (device, blocks x threads words, caller-owned):
- *   kind 0  lazy Shoup product x w - floor(x w' / 2^64) q (w' = floor(w 2^64 / q))
- *   kind 1  lazy Cooley-Tukey butterfly of the NTT (Shoup product plus
- *           Harvey's additions and correction)
- *   kind 2  64 x 64 -> 128-bit multiply-accumulate
+ *   kind 0  lazy Shoup product x w - h q with a rounded signed quotient h
+ *   kind 1  lazy Cooley-Tukey butterfly of the NTT (a Shoup product and two
+ *           additions, in the form the transform runs for this q)
+ *   kind 2  multiply-accumulate of the dot products: on limbs for q < 2^60,
+ *           else a 64 x 64 -> 128-bit product
  *   kind 3  Montgomery product, R = 2^64
  *   kind 4  16 x 16 transpose of 64-bit values within each half-warp by
  *           warp shuffles (the exchange between two radix-16 NTT passes)
@@ -459,8 +460,9 @@ int ckks_pull(void *dst, const void *src, size_t bytes, int blocks, void *stream
  * (kinds 6 and 7 need q = 1 (mod 2^32), else CKKS_EINVAL before any launch;
  * kinds 4 and 5 run 16 values per thread and count one operation per
  * value moved: blocks x threads x 16 x iters; q, w, wp are not used)
- * q: odd modulus below 2^62; w, wp: host arrays of ckks_peak_chains() Shoup
- * pairs (w < q). The caller times the launch on `stream` with CUDA events:
+ * q: odd modulus below 2^62; w, wp: host arrays of ckks_peak_chains()
+ * constants w < q and companions floor(w 2^64 / q) (the companions the
+ * kernels use are derived from w and q). The caller times the launch on `stream` with CUDA events:
  * operations per second = blocks x threads x chains x iters / time
  * (kinds 0-3, 6, 7).
  * Returns CKKS_EINVAL for bad arguments, CKKS_ECUDA on a launch error. */
@@ -471,10 +473,12 @@ int ckks_peak_int(int kind, uint64_t q, const uint64_t *w, const uint64_t *wp, i
 /* Launch tunables of a context; results are the same for every value.
  * Chosen by the autotuner: "ntt_tile_cols" / "ntt_tile_blocks" = elements
  * per CTA tile of the NTT's column / block phases ("ntt_tile" sets both;
- * reading it gives the column value) (1024..8192,
- * power of two; default 4096), "bconv_threads" = threads per BConv block
- * (64..1024, multiple of 32; default 256), "mac_threads" = threads per
- * key-MAC block (same range).
+ * reading it gives the column value) (1024..8192, power of two; default
+ * 4096; the kernels use whole groups of 16 columns up to 4096 elements and at
+ * most 1024 elements of blocks, and transforms up to N = 2^12 no tile at all),
+ * "bconv_threads" = threads per BConv block (64..1024, multiple of 32;
+ * default 256), "mac_threads" = threads per key-MAC block (same range);
+ * both kernels run at most 256.
  * Forms of the rescaling, for measuring the paper's reformulations (every
  * rescaling form gives the same residues): "inner_rescale" 0 = Algorithm 1 (mu INTT
  * + (l - mu) NTT per polynomial, default), 1 = mu single rescales of Eq. 7,
@@ -505,10 +509,10 @@ int ckks_peak_int(int kind, uint64_t q, const uint64_t *w, const uint64_t *wp, i
  * Residues are the same either way; for other primes the value has no
  * effect.
  * Tensor product kernels (Eq. 13): "tensor_fixed" 1 (default) runs the
- * product of a tree node whose two or three children are all tuples of at
- * least four terms, in one of the compiled shapes (two children of 4..7
- * terms; three of 4 or 5), through a kernel unrolled for exactly that
- * shape; 0 sends every node to the kernels bounded by the largest tuple
+ * product of a tree node in one of the compiled shapes (two children of
+ * 4..7 terms; three of 4 or 5; in contexts with all primes below 2^60 also
+ * two or three ciphertexts, two tuples of 3 terms, and 3, 3 and 2 terms)
+ * through a kernel unrolled for exactly that shape; 0 sends every node to the kernels bounded by the largest tuple
  * size. Residues are the same either way. */
 int ckks_tune_set(ckks_context *ctx, const char *key, int value);
 int ckks_tune_get(const ckks_context *ctx, const char *key, int *value);

@@ -3,8 +3,9 @@
 //   kind 0  lazy Shoup product with the balanced companion (fused scalings)
 //   kind 1  lazy Cooley-Tukey butterfly in the form the NTT runs for this q
 //           (arith.cuh; the forward NTT's unit of work)
-//   kind 2  64 x 64 -> 128-bit multiply-accumulate (BConv, key MAC, tensor
-//           product dot products)
+//   kind 2  multiply-accumulate of the dot products (BConv, key MAC): on limbs
+//           for q < 2^60 (DotLimbs, both operands split beforehand), else a
+//           64 x 64 -> 128-bit product added with carry
 //   kind 3  Montgomery product with R = 2^64 (tensor product, key preparation)
 //   kind 4  the exchange between two radix-16 passes of a 256-point block
 //           (each of 16 threads holds 16 values; afterwards thread i holds
@@ -53,7 +54,8 @@ __device__ __forceinline__ void transpose16_shfl(u64 (&v)[16]) {
     }
 }
 
-// SMALL: the butterfly form of primes below 2^kSmallBits
+// SMALL: the butterfly form of primes below 2^kSmallBits; for KIND 2 the limb
+// form
 template <int KIND, bool SMALL = false>
 __global__ void __launch_bounds__(256) peak_kernel(PeakConsts P, int iters, u64 *out) {
     const u64 tid = (u64)blockIdx.x * blockDim.x + threadIdx.x;
@@ -67,6 +69,9 @@ __global__ void __launch_bounds__(256) peak_kernel(PeakConsts P, int iters, u64 
     Acc128Lazy acc[kChains];
 #pragma unroll
     for (int i = 0; i < kChains; ++i) acc[i].zero();
+    DotLimbs dot[kChains];
+#pragma unroll
+    for (int i = 0; i < kChains; ++i) dot[i].zero();
     const ModQ m{q, P.qinv, {0, 0}, 0};
     for (int it = 0; it < iters; ++it) {
 #pragma unroll
@@ -79,6 +84,9 @@ __global__ void __launch_bounds__(256) peak_kernel(PeakConsts P, int iters, u64 
                 ct_bfly<SMALL, true>(x[i], y[i], P.w[i], P.wp[i], q);
             } else if (KIND == 7) {
                 x[i] = shoup_signed<true>(x[i], P.w[i], P.wp[i], q);
+            } else if (KIND == 2 && SMALL) {
+                dot[i].mac(packed_limbs(x[i]), packed_limbs(P.w[i]));
+                x[i] += y[i];
             } else if (KIND == 2) {
                 acc[i].mac(x[i], P.w[i]);
                 x[i] += y[i];
@@ -89,7 +97,7 @@ __global__ void __launch_bounds__(256) peak_kernel(PeakConsts P, int iters, u64 
     }
     u64 r = 0;
 #pragma unroll
-    for (int i = 0; i < kChains; ++i) r ^= x[i] ^ y[i] ^ acc[i].hi ^ acc[i].lo;
+    for (int i = 0; i < kChains; ++i) r ^= x[i] ^ y[i] ^ acc[i].hi ^ acc[i].lo ^ dot[i].s0 ^ dot[i].s1 ^ dot[i].sx;
     out[tid] = r;
 }
 
@@ -149,7 +157,10 @@ extern "C" int ckks_peak_int(int kind, uint64_t q, const uint64_t *w, const uint
         if (small_prime(q)) peak_kernel<1, true><<<blocks, threads, 0, st>>>(P, iters, (u64 *)out);
         else peak_kernel<1><<<blocks, threads, 0, st>>>(P, iters, (u64 *)out);
         break;
-    case 2: peak_kernel<2><<<blocks, threads, 0, st>>>(P, iters, (u64 *)out); break;
+    case 2:
+        if (q >> 60) peak_kernel<2><<<blocks, threads, 0, st>>>(P, iters, (u64 *)out);
+        else peak_kernel<2, true><<<blocks, threads, 0, st>>>(P, iters, (u64 *)out);
+        break;
     case 3: peak_kernel<3><<<blocks, threads, 0, st>>>(P, iters, (u64 *)out); break;
     case 6:
         if (small_prime(q)) peak_kernel<6, true><<<blocks, threads, 0, st>>>(P, iters, (u64 *)out);
