@@ -6,9 +6,9 @@
 //   step 2), key preparation (P^-1 folded into the Q limbs, Eq. 12) and key
 //   generation (Eq. 2, 9, 14).
 //
-// All are memory-bound streams over [batch][poly][limb][N]; each thread owns
-// one coefficient and loops over what the formula sums, keeping partial sums
-// in 128-bit accumulators reduced once (Montgomery REDC).
+// Each thread owns one or two coefficients of [batch][poly][limb][N] and loops
+// over what the formula sums, keeping partial sums in limb or 128-bit
+// accumulators reduced once (Montgomery).
 #include "common.cuh"
 #include "internal.h"
 #include "rns.h"
@@ -353,7 +353,11 @@ cudaError_t launch_tensor_table(const Context &C, const TensorJob *jobs, int n_j
 // Coefficients per thread of the key MAC of single products / of pairs of
 // products (CKKS_MAC_PAIR, rns.h: two products of the same shape share each
 // term's key loads), its largest block (the "mac_threads" tunable is cut to
-// it) and the CTAs of that size per SM it is compiled for.
+// it) and the CTAs of that size per SM it is compiled for. The kernel is bound
+// by HBM (4.9 TB/s for a k = 12 product, batch 4, multiply pipe 60 % busy), so
+// warps in flight count: 64 registers and one coefficient of a pair 1225 us
+// for batch 8, two at 80 or 128 registers 1240 / 1232; a single product 86
+// against 91 / 111 us (128-bit products, four coefficients: 111).
 #ifndef CKKS_MAC_VEC
 #define CKKS_MAC_VEC 2
 #endif
@@ -370,8 +374,11 @@ cudaError_t launch_tensor_table(const Context &C, const TensorJob *jobs, int n_j
 __device__ __forceinline__ int key_limb_bits(u64 q, int key_digits) {
     return small_prime(q) && 11 * key_digits <= kLimbTerms27 ? 27 : 30;
 }
+
 // Coefficients per thread of BConv, its largest block (the "bconv_threads"
-// tunable is cut to it) and the CTAs of that size per SM it is compiled for.
+// tunable is cut to it) and the CTAs of that size per SM it is compiled for
+// (k = 12, batch 8: 2009 us with three, 2188 with two; one coefficient per
+// thread 2239).
 #ifndef CKKS_BCONV_VEC
 #define CKKS_BCONV_VEC 2
 #endif
@@ -383,11 +390,12 @@ __device__ __forceinline__ int key_limb_bits(u64 q, int key_digits) {
 // One CTA: the constants of (level, digit) staged in shared memory, then
 // CKKS_BCONV_VEC adjacent coefficients per thread (16-byte loads and stores
 // for two). y: limb 0 of the prescaled d_t; dst: slot 0 of the (t, digit)
-// ModUp output. Bound by the integer multiply pipe: |digit| products per
-// target and coefficient.
+// ModUp output. Bound by the integer multiply pipe (81 % busy): |digit| products
+// per target and coefficient (k = 12, batch 4: 957 us; 1231 with 128-bit
+// products).
 // LIMB: the sources' limbs stay in registers, the constants hold their own
 // limbs in shared memory, a product is three multiply-adds; sums of more than
-// kLimbTerms30 sources are added as 128-bit words. Every lane reads the same
+// kLimbTerms30 sources are reduced in parts and added. Every lane reads the same
 // constant, but shared memory still returns 32 lanes' worth of bytes, so a
 // constant is one 8-byte word (its limbs' sum is added up again) and serves
 // CKKS_BCONV_VEC coefficients. Otherwise (a prime of 2^60 or more)

@@ -30,7 +30,8 @@ namespace {
 
 constexpr int kThreads = 256;
 
-// CTAs per SM the small shapes are compiled for (bound by HBM)
+// CTAs per SM the small shapes are compiled for (three ciphertexts: 118.6 us
+// with three, 121 with four)
 #ifndef CKKS_TENSOR_SMALL_MINB
 #define CKKS_TENSOR_SMALL_MINB 3
 #endif
