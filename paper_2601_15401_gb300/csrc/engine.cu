@@ -739,7 +739,7 @@ int run_mul2_ws(const Context &C, int level, int B, LimbView a, LimbView b, Limb
 
 cudaError_t run_tensor(const Context &C, int B, int level, int m, const LimbView *in, const int *polys,
                        LimbView out, cudaStream_t st) {
-    TensorArgs T;
+    TensorArgs T{};
     T.n_batch = B;
     T.level = level;
     T.N = C.N;

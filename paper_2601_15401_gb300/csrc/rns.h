@@ -1,6 +1,7 @@
 // Argument blocks of the coefficient-wise RNS kernels (rns.cu).
 #pragma once
 #include "common.cuh"
+#include "tensor_shapes.h"
 
 namespace ckks {
 
@@ -120,22 +121,6 @@ struct TensorTableView {
 };
 
 cudaError_t launch_tensor(const Context &C, const TensorArgs &A, cudaStream_t st);
-// Codes of the small shapes (every child at most 3 terms): only in contexts
-// whose products run on limbs (limbs30).
-constexpr int kTensorSmallCode = 14;
-// Node shapes with exactly unrolled tensor kernels (children sorted by
-// tuple size, largest first; c = 0 for two children): two children of 4..7
-// terms (codes 0..9) except 6 and 4 (children of 5 and 3 inputs: no tree
-// within the depth rule has that node for k <= 16), three of 4 or 5 terms
-// (codes 10..13); (2,2), (3,3), (2,2,2) and (3,3,2) (codes 14..17); -1
-// otherwise.
-__host__ __device__ inline int tensor_fixed_code(int m, int a, int b, int c) {
-    if (m == 2 && b >= 4 && b <= a && a <= 7 && !(a == 6 && b == 4)) return (a - 4) * (a - 3) / 2 + (b - 4);
-    if (m == 2 && a == b && a <= 3) return kTensorSmallCode + a - 2;
-    if (m == 3 && a == b && a <= 3 && c == 2) return kTensorSmallCode + a;
-    if (m == 3 && c >= 4 && c <= b && b <= a && a <= 5) return 10 + (a - 4) + (b - 4) + (c - 4);
-    return -1;
-}
 // The node's children sorted by tuple size, largest first (the product is
 // commutative, so the order does not change the result); the shape code of
 // the sorted node, -1 when no fixed kernel covers it.

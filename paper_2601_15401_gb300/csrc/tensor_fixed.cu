@@ -7,7 +7,7 @@
 // size, largest first (the product is commutative and every step returns
 // canonical residues, so the order does not change the result), every load
 // of the node issued before the first product, each output term stored as
-// soon as it is reduced. Shapes (tensor_fixed_code): two children of 4..7
+// soon as it is reduced. Shapes (kTensorShapes): two children of 4..7
 // terms, three of 4 or 5 terms — among them the roots and the larger inner
 // nodes of the paper's partitions for k = 6..12 (Table II) — and, on limbs,
 // the small nodes: two or three ciphertexts, two children of 3 terms, alone or
@@ -161,28 +161,16 @@ __global__ void __launch_bounds__(kThreads, A <= 3 ? CKKS_TENSOR_SMALL_MINB : A 
     tensor_fixed_coeff<A, B, C, V, Q1, LIMB>(TensorTableView{J}, r, j, mods[j], rfix);
 }
 
-// The shape of each code (tensor_fixed_code), as template arguments.
-template <class F>
+// f(A, B, C) with the shape of `code` (kTensorShapes) as integral constants
+template <int I = 0, class F>
 cudaError_t with_shape(int code, F &&f) {
-    switch (code) {
-    case 0: return f(std::integral_constant<int, 4>{}, std::integral_constant<int, 4>{}, std::integral_constant<int, 0>{});
-    case 1: return f(std::integral_constant<int, 5>{}, std::integral_constant<int, 4>{}, std::integral_constant<int, 0>{});
-    case 2: return f(std::integral_constant<int, 5>{}, std::integral_constant<int, 5>{}, std::integral_constant<int, 0>{});
-    case 4: return f(std::integral_constant<int, 6>{}, std::integral_constant<int, 5>{}, std::integral_constant<int, 0>{});
-    case 5: return f(std::integral_constant<int, 6>{}, std::integral_constant<int, 6>{}, std::integral_constant<int, 0>{});
-    case 6: return f(std::integral_constant<int, 7>{}, std::integral_constant<int, 4>{}, std::integral_constant<int, 0>{});
-    case 7: return f(std::integral_constant<int, 7>{}, std::integral_constant<int, 5>{}, std::integral_constant<int, 0>{});
-    case 8: return f(std::integral_constant<int, 7>{}, std::integral_constant<int, 6>{}, std::integral_constant<int, 0>{});
-    case 9: return f(std::integral_constant<int, 7>{}, std::integral_constant<int, 7>{}, std::integral_constant<int, 0>{});
-    case 10: return f(std::integral_constant<int, 4>{}, std::integral_constant<int, 4>{}, std::integral_constant<int, 4>{});
-    case 11: return f(std::integral_constant<int, 5>{}, std::integral_constant<int, 4>{}, std::integral_constant<int, 4>{});
-    case 12: return f(std::integral_constant<int, 5>{}, std::integral_constant<int, 5>{}, std::integral_constant<int, 4>{});
-    case 13: return f(std::integral_constant<int, 5>{}, std::integral_constant<int, 5>{}, std::integral_constant<int, 5>{});
-    case 14: return f(std::integral_constant<int, 2>{}, std::integral_constant<int, 2>{}, std::integral_constant<int, 0>{});
-    case 15: return f(std::integral_constant<int, 3>{}, std::integral_constant<int, 3>{}, std::integral_constant<int, 0>{});
-    case 16: return f(std::integral_constant<int, 2>{}, std::integral_constant<int, 2>{}, std::integral_constant<int, 2>{});
-    case 17: return f(std::integral_constant<int, 3>{}, std::integral_constant<int, 3>{}, std::integral_constant<int, 2>{});
-    default: return cudaErrorInvalidValue;
+    if constexpr (I < kTensorShapeCount) {
+        if (code == I)
+            return f(std::integral_constant<int, kTensorShapes[I].a>{}, std::integral_constant<int, kTensorShapes[I].b>{},
+                     std::integral_constant<int, kTensorShapes[I].c>{});
+        return with_shape<I + 1>(code, f);
+    } else {
+        return cudaErrorInvalidValue;
     }
 }
 
