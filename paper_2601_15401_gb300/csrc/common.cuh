@@ -37,7 +37,9 @@ __device__ __forceinline__ void grid_dependency_wait() { asm volatile("griddepco
 
 // Launches a kernel whose every CTA calls grid_dependency_wait as a dependent
 // of the work before it on the stream: the gap between two launches shrinks
-// (one product at N = 2^10: 58.4 -> 40.7 us for nine launches).
+// (one product at N = 2^10: 58.4 -> 40.7 us for nine launches). Callers return
+// its result: a refused launch leaves nothing behind in the thread's
+// last-error slot, where the next valid call would find it.
 template <typename... P, typename... A>
 static inline cudaError_t launch_dependent(void (*kern)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t st,
                                            A... args) {
@@ -51,7 +53,9 @@ static inline cudaError_t launch_dependent(void (*kern)(P...), dim3 grid, dim3 b
     at[0].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = at;
     cfg.numAttrs = 1;
-    return cudaLaunchKernelEx(&cfg, kern, P(args)...);
+    const cudaError_t e = cudaLaunchKernelEx(&cfg, kern, P(args)...);
+    if (e != cudaSuccess) cudaGetLastError();
+    return e;
 }
 
 __device__ __forceinline__ u64 mulhi64(u64 a, u64 b) { return __umul64hi(a, b); }

@@ -188,12 +188,10 @@ cudaError_t dft(const Context &C, const double2 *in, double2 *tmp, double2 *out,
     const size_t sm2 = (size_t)(kTC * N2 + N2 / 2 + 1) * sizeof(double2);
     const int tc = N2 < kTC ? N2 : kTC, tr = N1 < kTC ? N1 : kTC;
     count_kernel(C);
-    launch_dependent(fft_cols_kernel, dim3(N2 / tc, batch), dim3(kThr), sm1, st, in, tmp, lg1, lg2, sign, T);
-    cudaError_t e = cudaGetLastError();
+    cudaError_t e = launch_dependent(fft_cols_kernel, dim3(N2 / tc, batch), dim3(kThr), sm1, st, in, tmp, lg1, lg2, sign, T);
     if (e != cudaSuccess) return e;
     count_kernel(C);
-    launch_dependent(fft_rows_kernel, dim3(N1 / tr, batch), dim3(kThr), sm2, st, tmp, out, lg1, lg2, sign, T);
-    return cudaGetLastError();
+    return launch_dependent(fft_rows_kernel, dim3(N1 / tr, batch), dim3(kThr), sm2, st, tmp, out, lg1, lg2, sign, T);
 }
 
 size_t embed_ws(const Context &C, uint32_t batch) { return (2 * (size_t)batch + 2) * C.N * sizeof(double2); }
@@ -201,8 +199,7 @@ size_t embed_ws(const Context &C, uint32_t batch) { return (2 * (size_t)batch + 
 // the roots table at the end of the workspace, filled on `st`
 cudaError_t roots(const Context &C, double2 *T, cudaStream_t st) {
     count_kernel(C);
-    launch_dependent(roots_kernel, dim3((2 * C.N + kThr - 1) / kThr), dim3(kThr), 0, st, T, C.N);
-    return cudaGetLastError();
+    return launch_dependent(roots_kernel, dim3((2 * C.N + kThr - 1) / kThr), dim3(kThr), 0, st, T, C.N);
 }
 
 }  // namespace
@@ -229,14 +226,12 @@ int ckks_encode(ckks_context *ctx, const double *z, uint32_t batch, double scale
     cudaError_t err = roots(C, T, st);
     if (err == cudaSuccess) {
         count_kernel(C);
-        launch_dependent(scatter_kernel, dim3((C.N / 2 + kThr - 1) / kThr, batch), dim3(kThr), 0, st, z, A, C.N, scale);
-        err = cudaGetLastError();
+        err = launch_dependent(scatter_kernel, dim3((C.N / 2 + kThr - 1) / kThr, batch), dim3(kThr), 0, st, z, A, C.N, scale);
     }
     if (err == cudaSuccess) err = dft(C, A, Bf, A, (int)batch, -1, T, st);
     if (err == cudaSuccess) {
         count_kernel(C);
-        launch_dependent(untwist_round_kernel, dim3((C.N + kThr - 1) / kThr, batch), dim3(kThr), 0, st, A, (long long *)m, C.N, T);
-        err = cudaGetLastError();
+        err = launch_dependent(untwist_round_kernel, dim3((C.N + kThr - 1) / kThr, batch), dim3(kThr), 0, st, A, (long long *)m, C.N, T);
     }
     if (err != cudaSuccess) {
         const_cast<Context &>(C).sticky.store((int)err);
@@ -259,14 +254,12 @@ int ckks_decode(ckks_context *ctx, const double *m, uint32_t batch, double scale
     cudaError_t err = roots(C, T, st);
     if (err == cudaSuccess) {
         count_kernel(C);
-        launch_dependent(twist_kernel, dim3((C.N + kThr - 1) / kThr, batch), dim3(kThr), 0, st, m, A, C.N, T);
-        err = cudaGetLastError();
+        err = launch_dependent(twist_kernel, dim3((C.N + kThr - 1) / kThr, batch), dim3(kThr), 0, st, m, A, C.N, T);
     }
     if (err == cudaSuccess) err = dft(C, A, Bf, A, (int)batch, +1, T, st);
     if (err == cudaSuccess) {
         count_kernel(C);
-        launch_dependent(slots_kernel, dim3((C.N / 2 + kThr - 1) / kThr, batch), dim3(kThr), 0, st, A, z, C.N, 1.0 / scale);
-        err = cudaGetLastError();
+        err = launch_dependent(slots_kernel, dim3((C.N / 2 + kThr - 1) / kThr, batch), dim3(kThr), 0, st, A, z, C.N, 1.0 / scale);
     }
     if (err != cudaSuccess) {
         const_cast<Context &>(C).sticky.store((int)err);

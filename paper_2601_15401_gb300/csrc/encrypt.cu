@@ -200,8 +200,7 @@ int ckks_encrypt_batch(ckks_context *ctx, const int64_t *m, const int64_t *v, co
         err = transform_signed(C, (int)cb, 3, (int)level, sa, sb, w, st);
         if (err == cudaSuccess) {
             count_kernel(C);
-            launch_dependent(enc_batch_kernel, dim3(blocks((i64)level * N), cb), dim3(kThr), 0, st, W, (const u64 *)pk, (i64)C.L * N, (u64 *)out[b0].data, os, ps, (int)level, C.N, C.d_mods, C.d_r2);
-            err = cudaGetLastError();
+            err = launch_dependent(enc_batch_kernel, dim3(blocks((i64)level * N), cb), dim3(kThr), 0, st, W, (const u64 *)pk, (i64)C.L * N, (u64 *)out[b0].data, os, ps, (int)level, C.N, C.d_mods, C.d_r2);
         }
     }
     if (err != cudaSuccess) {
@@ -250,8 +249,7 @@ int ckks_decrypt_batch(ckks_context *ctx, const ckks_tuple *ct, uint32_t batch, 
     cudaError_t err = transform_signed(C, 1, 1, limbs, sa, sb, LimbView{S, 0, (i64)limbs * N}, st);
     if (err == cudaSuccess) {
         count_kernel(C);
-        launch_dependent(dec_batch_kernel, dim3(blocks((i64)limbs * N), batch), dim3(kThr), 0, st, (const u64 *)ct[0].data, cs, (i64)ct[0].poly_stride * N, S, P, limbs, C.N, C.d_mods, C.d_r2);
-        err = cudaGetLastError();
+        err = launch_dependent(dec_batch_kernel, dim3(blocks((i64)limbs * N), batch), dim3(kThr), 0, st, (const u64 *)ct[0].data, cs, (i64)ct[0].poly_stride * N, S, P, limbs, C.N, C.d_mods, C.d_r2);
     }
     if (err == cudaSuccess) {
         LimbView v{P, (i64)limbs * N, (i64)limbs * N};
@@ -265,8 +263,7 @@ int ckks_decrypt_batch(ckks_context *ctx, const ckks_tuple *ct, uint32_t batch, 
             one_q1 = make_shoup(1, q1);
         }
         count_kernel(C);
-        launch_dependent(crt2_kernel, dim3(blocks(N), batch), dim3(kThr), 0, st, P, out, limbs, C.N, q0, q1, inv, one_q1);
-        err = cudaGetLastError();
+        err = launch_dependent(crt2_kernel, dim3(blocks(N), batch), dim3(kThr), 0, st, P, out, limbs, C.N, q0, q1, inv, one_q1);
     }
     if (err != cudaSuccess) {
         const_cast<Context &>(C).sticky.store((int)err);

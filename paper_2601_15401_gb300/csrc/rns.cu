@@ -254,30 +254,32 @@ double tensor_products_per_coeff(const int *polys, int m) {
 constexpr int kTensorVecMaxT = CKKS_TENSOR_VEC_MAXT;
 
 template <bool Q1, int V>
-static void launch_tensor_sized(int maxt, dim3 blocks, const TensorArgs &A, cudaStream_t st) {
-    if (maxt <= 3) launch_dependent(tensor_kernel<3, Q1, V>, blocks, dim3(kThreads), 0, st, A);
-    else if (maxt <= 4) launch_dependent(tensor_kernel<4, Q1, V>, blocks, dim3(kThreads), 0, st, A);
-    else if (maxt <= 5 && (V == 1 || kTensorVecMaxT >= 5)) launch_dependent(tensor_kernel<5, Q1, V>, blocks, dim3(kThreads), 0, st, A);
+static cudaError_t launch_tensor_sized(int maxt, dim3 blocks, const TensorArgs &A, cudaStream_t st) {
+    if (maxt <= 3) return launch_dependent(tensor_kernel<3, Q1, V>, blocks, dim3(kThreads), 0, st, A);
+    else if (maxt <= 4) return launch_dependent(tensor_kernel<4, Q1, V>, blocks, dim3(kThreads), 0, st, A);
+    else if (maxt <= 5 && (V == 1 || kTensorVecMaxT >= 5)) return launch_dependent(tensor_kernel<5, Q1, V>, blocks, dim3(kThreads), 0, st, A);
     else if constexpr (V == 1) {
-        if (maxt <= 7) launch_dependent(tensor_kernel<7, Q1, 1>, blocks, dim3(kThreads), 0, st, A);
-        else if (maxt <= 9) launch_dependent(tensor_kernel<9, Q1, 1>, blocks, dim3(kThreads), 0, st, A);
-        else launch_dependent(tensor_kernel<CKKS_MAX_TUPLE, Q1, 1>, blocks, dim3(kThreads), 0, st, A);
+        if (maxt <= 7) return launch_dependent(tensor_kernel<7, Q1, 1>, blocks, dim3(kThreads), 0, st, A);
+        else if (maxt <= 9) return launch_dependent(tensor_kernel<9, Q1, 1>, blocks, dim3(kThreads), 0, st, A);
+        else return launch_dependent(tensor_kernel<CKKS_MAX_TUPLE, Q1, 1>, blocks, dim3(kThreads), 0, st, A);
     }
+    return cudaErrorInvalidValue;  // no kernel of two coefficients for tuples this large
 }
 
 template <bool Q1, int V>
-static void launch_tensor_table_sized(const Context &C, int maxt, dim3 blocks, const TensorJob *jobs,
+static cudaError_t launch_tensor_table_sized(const Context &C, int maxt, dim3 blocks, const TensorJob *jobs,
                                       cudaStream_t st) {
 #define CKKS_TT(MT, VV) launch_dependent(tensor_table_kernel<MT, Q1, VV>, blocks, dim3(kThreads), 0, st, jobs, C.N, C.log_n, C.d_mods, C.d_rfix)
-    if (maxt <= 3) CKKS_TT(3, V);
-    else if (maxt <= 4) CKKS_TT(4, V);
-    else if (maxt <= 5 && (V == 1 || kTensorVecMaxT >= 5)) CKKS_TT(5, V);
+    if (maxt <= 3) return CKKS_TT(3, V);
+    else if (maxt <= 4) return CKKS_TT(4, V);
+    else if (maxt <= 5 && (V == 1 || kTensorVecMaxT >= 5)) return CKKS_TT(5, V);
     else if constexpr (V == 1) {
-        if (maxt <= 7) CKKS_TT(7, 1);
-        else if (maxt <= 9) CKKS_TT(9, 1);
-        else CKKS_TT(CKKS_MAX_TUPLE, 1);
+        if (maxt <= 7) return CKKS_TT(7, 1);
+        else if (maxt <= 9) return CKKS_TT(9, 1);
+        else return CKKS_TT(CKKS_MAX_TUPLE, 1);
     }
 #undef CKKS_TT
+    return cudaErrorInvalidValue;
 }
 
 static bool view_vec2(const LimbView &v) {
@@ -310,13 +312,11 @@ cudaError_t launch_tensor(const Context &C, const TensorArgs &Ain, cudaStream_t 
     const i64 per = vec2 ? 2 * kThreads : kThreads;
     dim3 blocks((unsigned)(((i64)A.level * A.N + per - 1) / per), A.n_batch);
     if (vec2) {
-        if (C.q1()) launch_tensor_sized<true, 2>(maxt, blocks, A, st);
-        else launch_tensor_sized<false, 2>(maxt, blocks, A, st);
-    } else {
-        if (C.q1()) launch_tensor_sized<true, 1>(maxt, blocks, A, st);
-        else launch_tensor_sized<false, 1>(maxt, blocks, A, st);
+        if (C.q1()) return launch_tensor_sized<true, 2>(maxt, blocks, A, st);
+        return launch_tensor_sized<false, 2>(maxt, blocks, A, st);
     }
-    return cudaGetLastError();
+    if (C.q1()) return launch_tensor_sized<true, 1>(maxt, blocks, A, st);
+    return launch_tensor_sized<false, 1>(maxt, blocks, A, st);
 }
 
 bool tensor_job_vec2(const TensorJob &T) {
@@ -335,13 +335,11 @@ cudaError_t launch_tensor_table(const Context &C, const TensorJob *jobs, int n_j
     count_kernel(C);
     ProfScope ps(C, KC_TENSOR, bytes, st, ops);
     if (vec2) {
-        if (C.q1()) launch_tensor_table_sized<true, 2>(C, maxt, blocks, jobs, st);
-        else launch_tensor_table_sized<false, 2>(C, maxt, blocks, jobs, st);
-    } else {
-        if (C.q1()) launch_tensor_table_sized<true, 1>(C, maxt, blocks, jobs, st);
-        else launch_tensor_table_sized<false, 1>(C, maxt, blocks, jobs, st);
+        if (C.q1()) return launch_tensor_table_sized<true, 2>(C, maxt, blocks, jobs, st);
+        return launch_tensor_table_sized<false, 2>(C, maxt, blocks, jobs, st);
     }
-    return cudaGetLastError();
+    if (C.q1()) return launch_tensor_table_sized<true, 1>(C, maxt, blocks, jobs, st);
+    return launch_tensor_table_sized<false, 1>(C, maxt, blocks, jobs, st);
 }
 
 // ---------------------------------------------------------------------------
@@ -549,21 +547,21 @@ __global__ void __launch_bounds__(CKKS_BCONV_MAX_THREADS, CKKS_BCONV_MINB)
 static int bconv_sources(int alpha) { return alpha <= 4 ? 4 : alpha <= 8 ? 8 : alpha <= 12 ? 12 : 16; }
 
 template <bool Q1, bool LIMB>
-static void launch_bconv_sized(int alpha, dim3 grid, int thr, size_t smem, const BconvArgs &A, cudaStream_t st) {
-    if (alpha <= 4) launch_dependent(bconv_kernel<4, Q1, LIMB>, grid, dim3(thr), smem, st, A);
-    else if (alpha <= 8) launch_dependent(bconv_kernel<8, Q1, LIMB>, grid, dim3(thr), smem, st, A);
-    else if (alpha <= 12) launch_dependent(bconv_kernel<12, Q1, LIMB>, grid, dim3(thr), smem, st, A);
-    else launch_dependent(bconv_kernel<16, Q1, LIMB>, grid, dim3(thr), smem, st, A);
+static cudaError_t launch_bconv_sized(int alpha, dim3 grid, int thr, size_t smem, const BconvArgs &A, cudaStream_t st) {
+    if (alpha <= 4) return launch_dependent(bconv_kernel<4, Q1, LIMB>, grid, dim3(thr), smem, st, A);
+    if (alpha <= 8) return launch_dependent(bconv_kernel<8, Q1, LIMB>, grid, dim3(thr), smem, st, A);
+    if (alpha <= 12) return launch_dependent(bconv_kernel<12, Q1, LIMB>, grid, dim3(thr), smem, st, A);
+    return launch_dependent(bconv_kernel<16, Q1, LIMB>, grid, dim3(thr), smem, st, A);
 }
 
 template <bool Q1, bool LIMB>
-static void launch_bconv_table_sized(const Context &C, dim3 grid, int thr, size_t smem, const BconvJob *jobs,
+static cudaError_t launch_bconv_table_sized(const Context &C, dim3 grid, int thr, size_t smem, const BconvJob *jobs,
                                      cudaStream_t st) {
     const int np = C.L + C.K, a = C.alpha;
-    if (a <= 4) launch_dependent(bconv_table_kernel<4, Q1, LIMB>, grid, dim3(thr), smem, st, jobs, a, C.L, C.K, np, C.N, C.d_mods);
-    else if (a <= 8) launch_dependent(bconv_table_kernel<8, Q1, LIMB>, grid, dim3(thr), smem, st, jobs, a, C.L, C.K, np, C.N, C.d_mods);
-    else if (a <= 12) launch_dependent(bconv_table_kernel<12, Q1, LIMB>, grid, dim3(thr), smem, st, jobs, a, C.L, C.K, np, C.N, C.d_mods);
-    else launch_dependent(bconv_table_kernel<16, Q1, LIMB>, grid, dim3(thr), smem, st, jobs, a, C.L, C.K, np, C.N, C.d_mods);
+    if (a <= 4) return launch_dependent(bconv_table_kernel<4, Q1, LIMB>, grid, dim3(thr), smem, st, jobs, a, C.L, C.K, np, C.N, C.d_mods);
+    if (a <= 8) return launch_dependent(bconv_table_kernel<8, Q1, LIMB>, grid, dim3(thr), smem, st, jobs, a, C.L, C.K, np, C.N, C.d_mods);
+    if (a <= 12) return launch_dependent(bconv_table_kernel<12, Q1, LIMB>, grid, dim3(thr), smem, st, jobs, a, C.L, C.K, np, C.N, C.d_mods);
+    return launch_dependent(bconv_table_kernel<16, Q1, LIMB>, grid, dim3(thr), smem, st, jobs, a, C.L, C.K, np, C.N, C.d_mods);
 }
 
 cudaError_t launch_moddown_conv(const Context &C, LimbView z, LimbView out, int batch, int level, cudaStream_t st) {
@@ -599,13 +597,9 @@ cudaError_t launch_bconv(const Context &C, const BconvArgs &A, cudaStream_t st) 
     }
     macs *= (double)A.n_t * A.n_batch * A.N;
     ProfScope ps(C, KC_BCONV, ((double)A.n_t * A.level + limbs_out) * A.n_batch * A.N * sizeof(u64), st, macs);
-    if (C.limbs30) {
-        if (C.q1()) launch_bconv_sized<true, true>(A.alpha, grid, thr, smem, A, st);
-        else launch_bconv_sized<false, true>(A.alpha, grid, thr, smem, A, st);
-    } else {
-        launch_bconv_sized<false, false>(A.alpha, grid, thr, smem, A, st);
-    }
-    return cudaGetLastError();
+    if (!C.limbs30) return launch_bconv_sized<false, false>(A.alpha, grid, thr, smem, A, st);
+    if (C.q1()) return launch_bconv_sized<true, true>(A.alpha, grid, thr, smem, A, st);
+    return launch_bconv_sized<false, true>(A.alpha, grid, thr, smem, A, st);
 }
 
 cudaError_t launch_bconv_table(const Context &C, const BconvJob *jobs, int n_jobs, double bytes, double macs,
@@ -618,13 +612,9 @@ cudaError_t launch_bconv_table(const Context &C, const BconvJob *jobs, int n_job
     count_kernel(C);
     count_op(C, OP_BCONV, (unsigned long long)n_jobs);
     ProfScope ps(C, KC_BCONV, bytes, st, macs);
-    if (C.limbs30) {
-        if (C.q1()) launch_bconv_table_sized<true, true>(C, grid, thr, smem, jobs, st);
-        else launch_bconv_table_sized<false, true>(C, grid, thr, smem, jobs, st);
-    } else {
-        launch_bconv_table_sized<false, false>(C, grid, thr, smem, jobs, st);
-    }
-    return cudaGetLastError();
+    if (!C.limbs30) return launch_bconv_table_sized<false, false>(C, grid, thr, smem, jobs, st);
+    if (C.q1()) return launch_bconv_table_sized<true, true>(C, grid, thr, smem, jobs, st);
+    return launch_bconv_table_sized<false, true>(C, grid, thr, smem, jobs, st);
 }
 
 // ---------------------------------------------------------------------------
@@ -779,14 +769,14 @@ __global__ void __launch_bounds__(CKKS_MAC_MAX_THREADS, CKKS_MAC_MINB) mac_kerne
 }
 
 template <int P, int V>
-static void launch_mac_part(const Context &C, const MacArgs &A, int b_first, int n_groups, cudaStream_t st) {
+static cudaError_t launch_mac_part(const Context &C, const MacArgs &A, int b_first, int n_groups, cudaStream_t st) {
     const int thr = std::min(C.tune_mac_threads, CKKS_MAC_MAX_THREADS);
     const int chunks = (A.N + thr * V - 1) / (thr * V);
     const long long blocks = (long long)chunks * (A.level + A.K) * n_groups;
     count_kernel(C);
-    if (!C.limbs30) launch_dependent(mac_kernel<false, P, V, false>, dim3((unsigned)blocks), dim3(thr), 0, st, A, b_first, n_groups);
-    else if (C.q1()) launch_dependent(mac_kernel<true, P, V, true>, dim3((unsigned)blocks), dim3(thr), 0, st, A, b_first, n_groups);
-    else launch_dependent(mac_kernel<false, P, V, true>, dim3((unsigned)blocks), dim3(thr), 0, st, A, b_first, n_groups);
+    if (!C.limbs30) return launch_dependent(mac_kernel<false, P, V, false>, dim3((unsigned)blocks), dim3(thr), 0, st, A, b_first, n_groups);
+    if (C.q1()) return launch_dependent(mac_kernel<true, P, V, true>, dim3((unsigned)blocks), dim3(thr), 0, st, A, b_first, n_groups);
+    return launch_dependent(mac_kernel<false, P, V, true>, dim3((unsigned)blocks), dim3(thr), 0, st, A, b_first, n_groups);
 }
 
 cudaError_t launch_mac(const Context &C, const MacArgs &A, cudaStream_t st) {
@@ -799,9 +789,11 @@ cudaError_t launch_mac(const Context &C, const MacArgs &A, cudaStream_t st) {
     ProfScope ps(C, KC_MAC, bytes, st, macs);
     // pairs of batch elements share the key loads; an odd last one alone
     const int pairs = CKKS_MAC_PAIR ? A.n_batch / 2 : 0;
-    if (pairs > 0) launch_mac_part<2, CKKS_MAC_VEC_PAIR>(C, A, 0, pairs, st);
-    if (A.n_batch - 2 * pairs > 0) launch_mac_part<1, CKKS_MAC_VEC>(C, A, 2 * pairs, A.n_batch - 2 * pairs, st);
-    return cudaGetLastError();
+    cudaError_t e = cudaSuccess;
+    if (pairs > 0) e = launch_mac_part<2, CKKS_MAC_VEC_PAIR>(C, A, 0, pairs, st);
+    if (e == cudaSuccess && A.n_batch - 2 * pairs > 0)
+        e = launch_mac_part<1, CKKS_MAC_VEC>(C, A, 2 * pairs, A.n_batch - 2 * pairs, st);
+    return e;
 }
 
 // Table launch of the key MAC: blockIdx.x = accumulator limb (products
@@ -851,11 +843,10 @@ static cudaError_t launch_mac_table_part(const Context &C, const MacJob *jobs, c
     const i64 kps = (i64)(C.L + C.K) * C.N;
 #define CKKS_MACT(Q, LB) \
     launch_dependent(mac_table_kernel<Q, P, V, LB>, grid, dim3(thr), 0, st, jobs, targets, keys, kps, C.dnum, C.alpha, C.L, C.N, C.d_mods)
-    if (!C.limbs30) CKKS_MACT(false, false);
-    else if (C.q1()) CKKS_MACT(true, true);
-    else CKKS_MACT(false, true);
+    if (!C.limbs30) return CKKS_MACT(false, false);
+    if (C.q1()) return CKKS_MACT(true, true);
+    return CKKS_MACT(false, true);
 #undef CKKS_MACT
-    return cudaGetLastError();
 }
 
 cudaError_t launch_mac_table(const Context &C, const MacJob *jobs, const MacTarget *targets, int n_pairs,
@@ -941,8 +932,7 @@ cudaError_t launch_rschain(const Context &C, const RsChainArgs &A, cudaStream_t 
     i64 total = (i64)A.n_batch * A.n_polys * A.N;
     count_kernel(C);
     ProfScope ps(C, KC_RSCHAIN, 2.0 * A.n_batch * A.n_polys * A.mu * A.N * sizeof(u64), st);
-    launch_dependent(rschain_kernel, dim3((unsigned)((total + kThreads - 1) / kThreads)), dim3(kThreads), 0, st, A);
-    return cudaGetLastError();
+    return launch_dependent(rschain_kernel, dim3((unsigned)((total + kThreads - 1) / kThreads)), dim3(kThreads), 0, st, A);
 }
 
 cudaError_t launch_rschain_table(const Context &C, const RsJob *jobs, int n_jobs, int max_polys, double bytes,
@@ -952,8 +942,7 @@ cudaError_t launch_rschain_table(const Context &C, const RsJob *jobs, int n_jobs
     count_kernel(C);
     ProfScope ps(C, KC_RSCHAIN, bytes, st);
     dim3 grid((unsigned)(((i64)max_polys * C.N + kThreads - 1) / kThreads), (unsigned)n_jobs);
-    launch_dependent(rschain_table_kernel, grid, dim3(kThreads), 0, st, jobs, C.N, C.d_mods, C.d_one, C.d_invq);
-    return cudaGetLastError();
+    return launch_dependent(rschain_table_kernel, grid, dim3(kThreads), 0, st, jobs, C.N, C.d_mods, C.d_one, C.d_invq);
 }
 
 // ---------------------------------------------------------------------------
@@ -1046,8 +1035,7 @@ cudaError_t launch_add_limbs(const Context &C, LimbView dst, LimbView src, int b
     if (total == 0 || batch == 0) return cudaSuccess;
     count_kernel(C);
     dim3 grid((unsigned)((total + kThreads - 1) / kThreads), (unsigned)batch);
-    launch_dependent(add_limbs_kernel, grid, dim3(kThreads), 0, st, dst, src, polys, level, C.N, C.d_mods);
-    return cudaGetLastError();
+    return launch_dependent(add_limbs_kernel, grid, dim3(kThreads), 0, st, dst, src, polys, level, C.N, C.d_mods);
 }
 
 // ek0 = E - a S + [P G_beta]_x S^t,  ek1 = a   (all L + K limbs, NTT domain)
