@@ -3,6 +3,7 @@
 #include <atomic>
 #include <cstdint>
 #include <string>
+#include <type_traits>
 #include <vector>
 
 #include "common.cuh"
@@ -174,6 +175,17 @@ struct Context {
     int tune_q1 = 1;
     bool q1() const { return primes_q1 && tune_q1 != 0; }
 };
+
+// f(q1, limb) with the forms of a context's dot products (key MAC, BConv, fixed
+// tensor shapes) as integral constants: sums on limbs where every prime is
+// below 2^60, else as 128-bit words, either with the REDC for primes
+// = 1 (mod 2^32) where all are (two 7-term children as 128-bit products, 24
+// limbs at N = 2^16: 90.6 us with it, 95.2 without).
+template <class F>
+inline auto with_product_form(const Context &C, F &&f) {
+    if (C.limbs30) return C.q1() ? f(std::true_type{}, std::true_type{}) : f(std::false_type{}, std::true_type{});
+    return C.q1() ? f(std::true_type{}, std::false_type{}) : f(std::false_type{}, std::false_type{});
+}
 
 // Records CUDA events around one launch on its stream when the hook is on;
 // `bytes` is the launch's algorithmic traffic (each input and output limb

@@ -597,9 +597,9 @@ cudaError_t launch_bconv(const Context &C, const BconvArgs &A, cudaStream_t st) 
     }
     macs *= (double)A.n_t * A.n_batch * A.N;
     ProfScope ps(C, KC_BCONV, ((double)A.n_t * A.level + limbs_out) * A.n_batch * A.N * sizeof(u64), st, macs);
-    if (!C.limbs30) return launch_bconv_sized<false, false>(A.alpha, grid, thr, smem, A, st);
-    if (C.q1()) return launch_bconv_sized<true, true>(A.alpha, grid, thr, smem, A, st);
-    return launch_bconv_sized<false, true>(A.alpha, grid, thr, smem, A, st);
+    return with_product_form(C, [&](auto q1, auto limb) {
+        return launch_bconv_sized<q1.value, limb.value>(A.alpha, grid, thr, smem, A, st);
+    });
 }
 
 cudaError_t launch_bconv_table(const Context &C, const BconvJob *jobs, int n_jobs, double bytes, double macs,
@@ -612,9 +612,9 @@ cudaError_t launch_bconv_table(const Context &C, const BconvJob *jobs, int n_job
     count_kernel(C);
     count_op(C, OP_BCONV, (unsigned long long)n_jobs);
     ProfScope ps(C, KC_BCONV, bytes, st, macs);
-    if (!C.limbs30) return launch_bconv_table_sized<false, false>(C, grid, thr, smem, jobs, st);
-    if (C.q1()) return launch_bconv_table_sized<true, true>(C, grid, thr, smem, jobs, st);
-    return launch_bconv_table_sized<false, true>(C, grid, thr, smem, jobs, st);
+    return with_product_form(C, [&](auto q1, auto limb) {
+        return launch_bconv_table_sized<q1.value, limb.value>(C, grid, thr, smem, jobs, st);
+    });
 }
 
 // ---------------------------------------------------------------------------
@@ -774,9 +774,10 @@ static cudaError_t launch_mac_part(const Context &C, const MacArgs &A, int b_fir
     const int chunks = (A.N + thr * V - 1) / (thr * V);
     const long long blocks = (long long)chunks * (A.level + A.K) * n_groups;
     count_kernel(C);
-    if (!C.limbs30) return launch_dependent(mac_kernel<false, P, V, false>, dim3((unsigned)blocks), dim3(thr), 0, st, A, b_first, n_groups);
-    if (C.q1()) return launch_dependent(mac_kernel<true, P, V, true>, dim3((unsigned)blocks), dim3(thr), 0, st, A, b_first, n_groups);
-    return launch_dependent(mac_kernel<false, P, V, true>, dim3((unsigned)blocks), dim3(thr), 0, st, A, b_first, n_groups);
+    return with_product_form(C, [&](auto q1, auto limb) {
+        return launch_dependent(mac_kernel<q1.value, P, V, limb.value>, dim3((unsigned)blocks), dim3(thr), 0, st, A,
+                                b_first, n_groups);
+    });
 }
 
 cudaError_t launch_mac(const Context &C, const MacArgs &A, cudaStream_t st) {
@@ -841,12 +842,10 @@ static cudaError_t launch_mac_table_part(const Context &C, const MacJob *jobs, c
     count_kernel(C);
     dim3 grid((unsigned)n, (unsigned)chunks);
     const i64 kps = (i64)(C.L + C.K) * C.N;
-#define CKKS_MACT(Q, LB) \
-    launch_dependent(mac_table_kernel<Q, P, V, LB>, grid, dim3(thr), 0, st, jobs, targets, keys, kps, C.dnum, C.alpha, C.L, C.N, C.d_mods)
-    if (!C.limbs30) return CKKS_MACT(false, false);
-    if (C.q1()) return CKKS_MACT(true, true);
-    return CKKS_MACT(false, true);
-#undef CKKS_MACT
+    return with_product_form(C, [&](auto q1, auto limb) {
+        return launch_dependent(mac_table_kernel<q1.value, P, V, limb.value>, grid, dim3(thr), 0, st, jobs, targets,
+                                keys, kps, C.dnum, C.alpha, C.L, C.N, C.d_mods);
+    });
 }
 
 cudaError_t launch_mac_table(const Context &C, const MacJob *jobs, const MacTarget *targets, int n_pairs,

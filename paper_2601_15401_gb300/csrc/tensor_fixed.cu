@@ -30,11 +30,12 @@ namespace {
 
 constexpr int kThreads = 256;
 
-// CTAs per SM the small shapes are compiled for (three ciphertexts: 118.6 us
-// with three, 121 with four)
-#ifndef CKKS_TENSOR_SMALL_MINB
-#define CKKS_TENSOR_SMALL_MINB 3
-#endif
+// CTAs per SM a shape is compiled for: four for two 4-term children on limbs,
+// three for all others (three ciphertexts on limbs: 118.6 us with three, 121
+// with four; two 4-term children as 128-bit products, 24 limbs at N = 2^16:
+// 43.1 us with three, 44.0 with four).
+template <int A, int B, int C, bool LIMB>
+constexpr int kFixedMinb = LIMB && A > 3 && A + B + C <= 8 ? 4 : 3;
 
 // A residue as an operand of the dot products, itself or its limbs, and the
 // reduction of a sum of at most 8 products of residues. (The sums of limbs
@@ -132,7 +133,7 @@ __device__ __forceinline__ void tensor_fixed_coeff(const View &v, i64 r, int j, 
 }
 
 template <int A, int B, int C, int V, bool Q1, bool LIMB>
-__global__ void __launch_bounds__(kThreads, A <= 3 ? CKKS_TENSOR_SMALL_MINB : A + B + C <= 8 ? 4 : 3) tensor_fixed_kernel(TensorArgs T) {
+__global__ void __launch_bounds__(kThreads, kFixedMinb<A, B, C, LIMB>) tensor_fixed_kernel(TensorArgs T) {
     grid_dependency_wait();
     const i64 r = ((i64)blockIdx.x * blockDim.x + threadIdx.x) * V;  // limb * N + coefficient
     if (r >= (i64)T.level * T.N) return;
@@ -143,7 +144,7 @@ __global__ void __launch_bounds__(kThreads, A <= 3 ? CKKS_TENSOR_SMALL_MINB : A 
 // blockIdx.y = table entry (every entry of the launch has this shape); the
 // entry is staged in shared memory, one word per thread
 template <int A, int B, int C, int V, bool Q1, bool LIMB>
-__global__ void __launch_bounds__(kThreads, A <= 3 ? CKKS_TENSOR_SMALL_MINB : A + B + C <= 8 ? 4 : 3) tensor_fixed_table_kernel(const TensorJob *jobs, int N, int log_n,
+__global__ void __launch_bounds__(kThreads, kFixedMinb<A, B, C, LIMB>) tensor_fixed_table_kernel(const TensorJob *jobs, int N, int log_n,
                                                                         const ModQ *mods, const Shoup *rfix) {
     grid_dependency_wait();
     __shared__ TensorJob J;
@@ -240,8 +241,9 @@ int tensor_sort_children(TensorArgs &A) {
 }
 
 cudaError_t launch_tensor_fixed(const Context &C, const TensorArgs &A, int code, bool vec2, cudaStream_t st) {
-    if (!C.limbs30) return launch_uniform<false, false>(A, code, vec2, st);
-    return C.q1() ? launch_uniform<true, true>(A, code, vec2, st) : launch_uniform<false, true>(A, code, vec2, st);
+    return with_product_form(C, [&](auto q1, auto limb) {
+        return launch_uniform<q1.value, limb.value>(A, code, vec2, st);
+    });
 }
 
 cudaError_t launch_tensor_fixed_table(const Context &C, const TensorJob *jobs, int n_jobs, int code, int max_level,
@@ -250,9 +252,9 @@ cudaError_t launch_tensor_fixed_table(const Context &C, const TensorJob *jobs, i
     if (n_jobs > 65535) return cudaErrorInvalidValue;
     count_kernel(C);
     ProfScope ps(C, KC_TENSOR, bytes, st, ops);
-    if (!C.limbs30) return launch_table<false, false>(C, jobs, n_jobs, code, max_level, vec2, st);
-    return C.q1() ? launch_table<true, true>(C, jobs, n_jobs, code, max_level, vec2, st)
-                  : launch_table<false, true>(C, jobs, n_jobs, code, max_level, vec2, st);
+    return with_product_form(C, [&](auto q1, auto limb) {
+        return launch_table<q1.value, limb.value>(C, jobs, n_jobs, code, max_level, vec2, st);
+    });
 }
 
 }  // namespace ckks
