@@ -52,6 +52,11 @@ int twiddle_slot(int logN, int k) {
 // phase of 384 limbs at N = 2^16: 143 / 145 us with 64 threads, 144 / 146 with
 // 128, 163 / 156 with 256).
 constexpr int kBlockTile = 1024;
+// Limbs per CTA of the transforms of N <= 2^8, one per warp (2048 limbs of
+// 2^7 / 2^8 points forward: 8.6 / 9.7 us with four, 10.1 / 11.6 with one, of
+// which some 8 us are the call's own; with run-time modes and shared memory for
+// as many blocks as a warp could hold, 10.1 / 12.3).
+constexpr int kTinyLimbs = 4;
 
 // Geometry of one phase: CTAs per limb, threads and shared memory per CTA. A
 // thread takes 16 points; the tile tunables set the elements per CTA (at
@@ -69,6 +74,7 @@ static int phase_geometry(const Context &C, bool cols, NttPhase &P, PhaseLaunch 
     P.tw_inv = C.d_tw_inv;
     const int logn = cols ? log_n1 : log_n2, n = 1 << logn;
     const int sets = n >= 16 ? n / 16 : 1;  // threads per sub-problem
+    G.limbs = 1;
     G.shape = cols ? COLS : logn > 8 ? WHOLE : BLOCKS;
     if (G.shape == COLS) {
         const int group = 16 * sets;
@@ -85,10 +91,13 @@ static int phase_geometry(const Context &C, bool cols, NttPhase &P, PhaseLaunch 
         int threads = std::min(C.tune_ntt_tile_blocks, kBlockTile) / 16;
         threads = std::max(32, std::min(threads, P.N1 * sets));
         const int blocks = threads / sets;
+        if (P.N1 == 1) G.limbs = kTinyLimbs, threads = 32 * kTinyLimbs;
         G.tiles = (P.N1 + blocks - 1) / blocks;
         G.threads = threads;
         // per warp: its blocks (one pad word per 16) and their n - 1 twiddles each (Geo::warp_bytes)
-        G.smem = (size_t)blocks * ((n + n / 16) * sizeof(u64) + (n - 1) * sizeof(ulonglong2));
+        // or its limb's (N <= 2^8)
+        if (P.N1 == 1) G.smem = kTinyLimbs * (((n + n / 16 + 1) & ~1) * sizeof(u64) + (n - 1) * sizeof(ulonglong2));
+        else G.smem = (size_t)blocks * ((n + n / 16) * sizeof(u64) + (n - 1) * sizeof(ulonglong2));
     }
     return logn;
 }

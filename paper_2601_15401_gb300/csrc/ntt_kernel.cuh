@@ -322,9 +322,10 @@ struct Geo {
     static constexpr int group = SH == COLS ? 16 * sets : sets;     // threads per tile unit (16 columns / one block)
     static constexpr int unit = SH == COLS ? 16 * n : n + n / 16;   // shared words per tile unit
     static constexpr int stride = SH == COLS ? 1 << LOGN2 : 1;      // elements between neighbouring points in memory
-    static constexpr int warp_blocks = SH == BLOCKS ? 32 / sets : 1;  // blocks per warp (whole: the limb)
+    // blocks per warp (one where the block is the whole limb, N <= 2^8)
+    static constexpr int warp_blocks = SH == BLOCKS && LOGN2 != 0 ? 32 / sets : 1;
     // bytes of a warp's part of a block-phase CTA: its blocks, then their n - 1 twiddles each
-    static constexpr int warp_data = warp_blocks * unit;    // words (even)
+    static constexpr int warp_data = (warp_blocks * unit + 1) & ~1;  // words (even: the twiddles take 16-byte copies)
     static constexpr int warp_bytes = warp_data * 8 + warp_blocks * (n - 1) * 16;
     // shared offset of point pt relative to the thread's sub-problem; additive
     // over disjoint bit ranges of pt
@@ -608,13 +609,13 @@ __device__ __forceinline__ void phase_tile(u64 *sm, const NttPhase &P, const ulo
         // a warp and its blocks, or the CTA and its limb
         constexpr int BW = G::warp_blocks;
         constexpr int T = SH == WHOLE ? G::sets : 32;
-        constexpr int W = BW * n / T;                     // words per lane
+        constexpr int W = (BW * n + T - 1) / T;           // words per lane
         constexpr int U = W < 8 ? W : 8;
         constexpr int PF = FWD ? 0 : NP - 1, PL = FWD ? NP - 1 : 0;
-        // with LOGN2 = 0 the launch may have fewer blocks than a warp takes
+        // a limb of N <= 2^8 may be less than a word per lane, or a set
         constexpr bool FULL = LOGN2 != 0 || SH == WHOLE;
         const int lane = SH == WHOLE ? tid : tid & 31;
-        const int b0 = SH == WHOLE ? 0 : tile * (blockDim.x / G::sets) + (tid / 32) * BW;  // first block in the limb
+        const int b0 = !FULL || SH == WHOLE ? 0 : tile * (blockDim.x / G::sets) + (tid / 32) * BW;  // first block in the limb
         u64 *wsm = SH == WHOLE ? sm : reinterpret_cast<u64 *>(reinterpret_cast<char *>(sm) + (tid / 32) * G::warp_bytes);
         ulonglong2 *wtw = reinterpret_cast<ulonglong2 *>(wsm + G::warp_data);
         ln.blk = SH == WHOLE ? 0 : lane / G::sets;
@@ -701,8 +702,12 @@ __device__ __forceinline__ void phase_tile(u64 *sm, const NttPhase &P, const ulo
 template <int LOGN, int LOGN2, bool FWD, int SH, int LM, int SM, int MINB, bool Q1>
 __global__ void __launch_bounds__(256, MINB) ntt_phase_kernel(NttPhase P, LimbJobs J, LoadSpec L, StoreSpec S) {
     extern __shared__ __align__(16) u64 sm[];
-    int b, p, l;
-    decode_job(J, blockIdx.y, b, p, l);
+    int b, p, l, job = blockIdx.y;
+    if constexpr (SH == BLOCKS && LOGN2 == 0) {  // N <= 2^8: a limb per warp
+        job = job * (blockDim.x / 32) + threadIdx.x / 32;
+        if (job >= J.n_batch * J.n_polys * J.n_limbs) return;
+    }
+    decode_job(J, job, b, p, l);
     const int prime = J.prime[l];
     const ModQ m = P.mods[prime];
     const ulonglong2 *tw = (FWD ? P.tw_fwd : P.tw_inv) + (i64)prime * P.N;
@@ -733,6 +738,7 @@ __global__ void __launch_bounds__(256, MINB) ntt_phase_table_kernel(NttPhase P, 
 // ---------------------------------------------------------------------------
 struct PhaseLaunch {
     int tiles, threads, shape;
+    int limbs;  // limbs per CTA
     size_t smem;
     cudaStream_t st;
 };
@@ -767,7 +773,9 @@ static inline cudaError_t launch_uniform(const NttPhase &P, const LimbJobs &J, c
     auto kern = ntt_phase_kernel<LOGN, LOGN2, FWD, SH, LM, SM, MINB, Q1>;
     cudaError_t e = allow_smem(kern, G.smem);
     if (e != cudaSuccess) return e;
-    dim3 grid(G.tiles, J.n_batch * J.n_polys * J.n_limbs);
+    const int limbs = J.n_batch * J.n_polys * J.n_limbs;
+    if (limbs > 65535) return cudaErrorInvalidConfiguration;  // the grid's second dimension, one limb each
+    dim3 grid(G.tiles, (limbs + G.limbs - 1) / G.limbs);
     return launch_dependent(kern, grid, dim3(G.threads), G.smem, G.st, P, J, L, S);
 }
 
@@ -791,7 +799,8 @@ static inline cudaError_t launch_table(const NttPhase &P, const NttJob *jobs, in
 //   two phases (N >= 2^13): dispatch_two, with the products in the form Q1
 //   selects (N >= 2^14);
 //   one phase (2^9 <= N <= 2^12): dispatch_whole;
-//   N <= 2^8: dispatch_tiny, run-time modes.
+//   N <= 2^8: dispatch_tiny, the plain transforms with a kernel of their own,
+//   the others run-time modes.
 #define CKKS_LAUNCH(LG, LG2, SHv, LMv, SMv, MB, Q)                                                   \
     do {                                                                                             \
         if constexpr (TABLE) return launch_table<LG, LG2, FWD, SHv, LMv, SMv, MB, Q>(P, jobs, n_jobs, L, S, G); \
@@ -886,14 +895,23 @@ static inline cudaError_t dispatch_tiny(int logn, const NttPhase &P, const LimbJ
     constexpr bool TABLE = false;
     const NttJob *jobs = nullptr;
     const int n_jobs = 0;
+#define CKKS_TINY(LG)                                                                             \
+    case LG:                                                                                      \
+        if constexpr (FWD) {                                                                      \
+            CKKS_MODES(LD_PLAIN, ST_REDUCE) CKKS_LAUNCH(LG, 0, BLOCKS, LD_PLAIN, ST_REDUCE, 2, false); \
+        } else {                                                                                  \
+            CKKS_MODES(LD_PLAIN, ST_SCALE) CKKS_LAUNCH(LG, 0, BLOCKS, LD_PLAIN, ST_SCALE, 2, false); \
+        }                                                                                         \
+        CKKS_LAUNCH(LG, 0, BLOCKS, -1, -1, 2, false)
     switch (logn) {
-    case 4: CKKS_LAUNCH(4, 0, BLOCKS, -1, -1, 2, false);
-    case 5: CKKS_LAUNCH(5, 0, BLOCKS, -1, -1, 2, false);
-    case 6: CKKS_LAUNCH(6, 0, BLOCKS, -1, -1, 2, false);
-    case 7: CKKS_LAUNCH(7, 0, BLOCKS, -1, -1, 2, false);
-    case 8: CKKS_LAUNCH(8, 0, BLOCKS, -1, -1, 2, false);
+        CKKS_TINY(4);
+        CKKS_TINY(5);
+        CKKS_TINY(6);
+        CKKS_TINY(7);
+        CKKS_TINY(8);
     default: return cudaErrorInvalidValue;
     }
+#undef CKKS_TINY
 }
 #undef CKKS_LAUNCH
 #undef CKKS_MODES
