@@ -472,13 +472,14 @@ int ckks_peak_int(int kind, uint64_t q, const uint64_t *w, const uint64_t *wp, i
 
 /* Launch tunables of a context; results are the same for every value.
  * Chosen by the autotuner: "ntt_tile_cols" / "ntt_tile_blocks" = elements
- * per CTA tile of the NTT's column / block phases ("ntt_tile" sets both;
- * reading it gives the column value) (1024..8192, power of two; default
- * 4096; the kernels use whole groups of 16 columns up to 4096 elements and at
- * most 1024 elements of blocks, and transforms up to N = 2^12 no tile at all),
- * "bconv_threads" = threads per BConv block (64..1024, multiple of 32;
- * default 256), "mac_threads" = threads per key-MAC block (same range);
- * both kernels run at most 256.
+ * per CTA tile of the NTT's column / block phases (powers of two, 1024..8192,
+ * default 4096, / 512..8192, default 1024; "ntt_tile" sets both, 1024..8192,
+ * and reading it gives the column value). A tile is whole groups of 16 columns
+ * or whole warps of blocks and at most 4096 elements: at N = 2^16 every column
+ * tile is 4096 elements, at 2^14 and 2^15 2048 or 4096; transforms up to
+ * N = 2^12 have no tile. "bconv_threads" = threads per BConv block (64..1024,
+ * multiple of 32; default 256), "mac_threads" = threads per key-MAC block
+ * (same range); both kernels run at most 256.
  * Forms of the rescaling, for measuring the paper's reformulations (every
  * rescaling form gives the same residues): "inner_rescale" 0 = Algorithm 1 (mu INTT
  * + (l - mu) NTT per polynomial, default), 1 = mu single rescales of Eq. 7,

@@ -712,7 +712,7 @@ static int *tune_slot(ckks_context *ctx, const char *key, int &lo, int &hi) {
         hi = 8192;
         return &ctx->c.tune_ntt_tile_cols;
     }
-    if (!strcmp(key, "ntt_tile_blocks")) { lo = 1024; hi = 8192; return &ctx->c.tune_ntt_tile_blocks; }
+    if (!strcmp(key, "ntt_tile_blocks")) { lo = 512; hi = 8192; return &ctx->c.tune_ntt_tile_blocks; }
     if (!strcmp(key, "bconv_threads")) { lo = 64; hi = 1024; return &ctx->c.tune_bconv_threads; }
     if (!strcmp(key, "mac_threads")) { lo = 64; hi = 1024; return &ctx->c.tune_mac_threads; }
     if (!strcmp(key, "inner_rescale")) { lo = 0; hi = 2; return &ctx->c.tune_inner_rescale; }

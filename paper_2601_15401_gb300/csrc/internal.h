@@ -7,6 +7,7 @@
 #include <vector>
 
 #include "common.cuh"
+#include "phase_shape.h"
 
 namespace ckks {
 
@@ -146,8 +147,8 @@ struct Context {
     std::atomic<int> sticky{0};
     Profiler prof;
     // launch tunables
-    int tune_ntt_tile_cols = 4096;    // elements per CTA tile, column phases
-    int tune_ntt_tile_blocks = 4096;  // elements per CTA tile, block phases (at most kBlockTile, ntt.cu)
+    int tune_ntt_tile_cols = 4096;            // elements per CTA tile, column phases (phase_shape.h)
+    int tune_ntt_tile_blocks = kBlockTile;    // elements per CTA tile, block phases
     int tune_bconv_threads = 256;
     int tune_mac_threads = 256;
     // forms of the rescaling (same results; for measuring the paper's
@@ -213,7 +214,6 @@ inline void count_op(const Context &C, int op, unsigned long long n = 1) {
 inline void count_kernel(const Context &C) { count_op(C, OP_KERNELS, 1); }
 
 // ntt.cu
-void ntt_geometry(int logN, int &log_n1, int &log_n2);
 int twiddle_slot(int logN, int k);  // table position of twiddle k
 // phase launch over a device table of NttJob (ntt_launch.cu); jobs: device
 // array of n_jobs entries

@@ -10,13 +10,6 @@
 
 namespace ckks {
 
-// Geometry of the phases for a given log N: log_n1 = 0 (one phase) up to
-// N = 2^12, the largest limb one CTA holds.
-void ntt_geometry(int logN, int &log_n1, int &log_n2) {
-    if (logN <= kWholeMax) { log_n1 = 0; log_n2 = logN; }
-    else { log_n1 = logN / 2; log_n2 = logN - log_n1; }
-}
-
 // Table position of forward / inverse twiddle k (psi^(+-)brv(k)) in the order
 // the passes read it (ntt_kernel.cuh): k = m_glob + i, m_glob = 2^s, is stage s
 // of the transform; its first log_n1 stages run in the column phase, the
@@ -46,22 +39,6 @@ int twiddle_slot(int logN, int k) {
     return (n_sub << start) + ((b * ((1 << len) - 1) + (1 << ep) - 1 + j) << start) + g;
 }
 
-// Elements per CTA of the block phases, at most. Their warps do not wait for
-// each other, so a CTA is only the unit in which shared memory is given out:
-// two-warp CTAs start as soon as two warps have ended (forward / inverse block
-// phase of 384 limbs at N = 2^16: 143 / 145 us with 64 threads, 144 / 146 with
-// 128, 163 / 156 with 256).
-constexpr int kBlockTile = 1024;
-// Limbs per CTA of the transforms of N <= 2^8, one per warp (2048 limbs of
-// 2^7 / 2^8 points forward: 8.6 / 9.7 us with four, 10.1 / 11.6 with one, of
-// which some 8 us are the call's own; with run-time modes and shared memory for
-// as many blocks as a warp could hold, 10.1 / 12.3).
-constexpr int kTinyLimbs = 4;
-
-// Geometry of one phase: CTAs per limb, threads and shared memory per CTA. A
-// thread takes 16 points; the tile tunables set the elements per CTA (at
-// least one group of 16 columns or one warp of blocks, at most 256 threads
-// for columns and kBlockTile elements for blocks).
 static int phase_geometry(const Context &C, bool cols, NttPhase &P, PhaseLaunch &G) {
     int log_n1, log_n2;
     ntt_geometry(C.log_n, log_n1, log_n2);
@@ -72,34 +49,8 @@ static int phase_geometry(const Context &C, bool cols, NttPhase &P, PhaseLaunch 
     P.mods = C.d_mods;
     P.tw_fwd = C.d_tw_fwd;
     P.tw_inv = C.d_tw_inv;
-    const int logn = cols ? log_n1 : log_n2, n = 1 << logn;
-    const int sets = n >= 16 ? n / 16 : 1;  // threads per sub-problem
-    G.limbs = 1;
-    G.shape = cols ? COLS : logn > 8 ? WHOLE : BLOCKS;
-    if (G.shape == COLS) {
-        const int group = 16 * sets;
-        int groups = C.tune_ntt_tile_cols / (16 * n);
-        groups = std::max(1, std::min(groups, std::min(256 / group, P.N2 / 16)));
-        G.tiles = P.N2 / 16 / groups;
-        G.threads = groups * group;
-        G.smem = (size_t)groups * 16 * n * sizeof(u64) + (size_t)n * sizeof(ulonglong2);
-    } else if (G.shape == WHOLE) {
-        G.tiles = 1;
-        G.threads = sets;
-        G.smem = (size_t)(n + n / 16) * sizeof(u64) + (size_t)(n - 1) * sizeof(ulonglong2);
-    } else {
-        int threads = std::min(C.tune_ntt_tile_blocks, kBlockTile) / 16;
-        threads = std::max(32, std::min(threads, P.N1 * sets));
-        const int blocks = threads / sets;
-        if (P.N1 == 1) G.limbs = kTinyLimbs, threads = 32 * kTinyLimbs;
-        G.tiles = (P.N1 + blocks - 1) / blocks;
-        G.threads = threads;
-        // per warp: its blocks (one pad word per 16) and their n - 1 twiddles each (Geo::warp_bytes)
-        // or its limb's (N <= 2^8)
-        if (P.N1 == 1) G.smem = kTinyLimbs * (((n + n / 16 + 1) & ~1) * sizeof(u64) + (n - 1) * sizeof(ulonglong2));
-        else G.smem = (size_t)blocks * ((n + n / 16) * sizeof(u64) + (n - 1) * sizeof(ulonglong2));
-    }
-    return logn;
+    G.s = phase_shape(C.log_n, cols, C.tune_ntt_tile_cols, C.tune_ntt_tile_blocks);
+    return G.s.logn;
 }
 
 // One phase. phase 0 = the first phase executed (forward: columns; inverse:

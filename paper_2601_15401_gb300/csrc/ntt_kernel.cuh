@@ -58,6 +58,7 @@
 #pragma once
 #include "common.cuh"
 #include "internal.h"
+#include "phase_shape.h"
 
 namespace ckks {
 
@@ -305,10 +306,8 @@ __device__ __forceinline__ void store_elem(const StoreCtx &c, int e, u64 v, bool
 // The geometry is fixed at compile time: every address within a thread's
 // point set is one base plus constant offsets.
 //   whole:   N <= 2^12 takes one launch for all stages: one CTA of n / 16
-//            threads holds a limb (N >= 2^9), or a warp holds one or more
-//            (a block phase with N1 = 1).
-enum Shape { COLS = 0, BLOCKS = 1, WHOLE = 2 };
-constexpr int kWholeMax = 12;  // log2 of the largest limb one CTA transforms
+//            threads holds a limb (N >= 2^9), or a warp does (a block phase
+//            with N1 = 1, kTinyLimbs warps per CTA).
 
 // elements whose sums over the K z-limbs run together
 #ifndef CKKS_NTT_MODDOWN_GROUP
@@ -700,7 +699,7 @@ __device__ __forceinline__ void phase_tile(u64 *sm, const NttPhase &P, const ulo
 // flattened dimension (limb * tiles + tile) for table launches
 // ---------------------------------------------------------------------------
 template <int LOGN, int LOGN2, bool FWD, int SH, int LM, int SM, int MINB, bool Q1>
-__global__ void __launch_bounds__(256, MINB) ntt_phase_kernel(NttPhase P, LimbJobs J, LoadSpec L, StoreSpec S) {
+__global__ void __launch_bounds__(kPhaseThreads, MINB) ntt_phase_kernel(NttPhase P, LimbJobs J, LoadSpec L, StoreSpec S) {
     extern __shared__ __align__(16) u64 sm[];
     int b, p, l, job = blockIdx.y;
     if constexpr (SH == BLOCKS && LOGN2 == 0) {  // N <= 2^8: a limb per warp
@@ -718,7 +717,7 @@ __global__ void __launch_bounds__(256, MINB) ntt_phase_kernel(NttPhase P, LimbJo
 }
 
 template <int LOGN, int LOGN2, bool FWD, int SH, int LM, int SM, int MINB, bool Q1>
-__global__ void __launch_bounds__(256, MINB) ntt_phase_table_kernel(NttPhase P, const NttJob *jobs, int tiles,
+__global__ void __launch_bounds__(kPhaseThreads, MINB) ntt_phase_table_kernel(NttPhase P, const NttJob *jobs, int tiles,
                                                                     LoadSpec L, StoreSpec S) {
     extern __shared__ __align__(16) u64 sm[];
     grid_dependency_wait();  // the job table may have been written just before
@@ -737,9 +736,7 @@ __global__ void __launch_bounds__(256, MINB) ntt_phase_table_kernel(NttPhase P, 
 // host-side launch of one instantiation
 // ---------------------------------------------------------------------------
 struct PhaseLaunch {
-    int tiles, threads, shape;
-    int limbs;  // limbs per CTA
-    size_t smem;
+    PhaseShape s;
     cudaStream_t st;
 };
 
@@ -771,24 +768,24 @@ template <int LOGN, int LOGN2, bool FWD, int SH, int LM, int SM, int MINB, bool 
 static inline cudaError_t launch_uniform(const NttPhase &P, const LimbJobs &J, const LoadSpec &L,
                                          const StoreSpec &S, const PhaseLaunch &G) {
     auto kern = ntt_phase_kernel<LOGN, LOGN2, FWD, SH, LM, SM, MINB, Q1>;
-    cudaError_t e = allow_smem(kern, G.smem);
+    cudaError_t e = allow_smem(kern, G.s.smem);
     if (e != cudaSuccess) return e;
     const int limbs = J.n_batch * J.n_polys * J.n_limbs;
     if (limbs > 65535) return cudaErrorInvalidConfiguration;  // the grid's second dimension, one limb each
-    dim3 grid(G.tiles, (limbs + G.limbs - 1) / G.limbs);
-    return launch_dependent(kern, grid, dim3(G.threads), G.smem, G.st, P, J, L, S);
+    dim3 grid(G.s.tiles, (limbs + G.s.limbs - 1) / G.s.limbs);
+    return launch_dependent(kern, grid, dim3(G.s.threads), G.s.smem, G.st, P, J, L, S);
 }
 
 template <int LOGN, int LOGN2, bool FWD, int SH, int LM, int SM, int MINB, bool Q1>
 static inline cudaError_t launch_table(const NttPhase &P, const NttJob *jobs, int n_jobs, const LoadSpec &L,
                                        const StoreSpec &S, const PhaseLaunch &G) {
     auto kern = ntt_phase_table_kernel<LOGN, LOGN2, FWD, SH, LM, SM, MINB, Q1>;
-    cudaError_t e = allow_smem(kern, G.smem);
+    cudaError_t e = allow_smem(kern, G.s.smem);
     if (e != cudaSuccess) return e;
-    const long long blocks = (long long)n_jobs * G.tiles;
+    const long long blocks = (long long)n_jobs * G.s.tiles;
     if (blocks <= 0) return cudaSuccess;
     if (blocks > 0x7FFFFFFFll) return cudaErrorInvalidValue;
-    return launch_dependent(kern, dim3((unsigned)blocks), dim3(G.threads), G.smem, G.st, P, jobs, G.tiles, L, S);
+    return launch_dependent(kern, dim3((unsigned)blocks), dim3(G.s.threads), G.s.smem, G.st, P, jobs, G.s.tiles, L, S);
 }
 
 // Dispatch of one direction (FWD) and job source (TABLE) over the shape, log2
@@ -843,7 +840,7 @@ static inline cudaError_t dispatch_two(int logn, const NttPhase &P, const LimbJo
                                        int n_jobs, const LoadSpec &L, const StoreSpec &S, const PhaseLaunch &G) {
 #define CKKS_COLS(LG, LG2) \
     if (logn == LG && P.log_n2 == LG2) return dispatch_cols<FWD, TABLE, Q1, LG, LG2>(P, J, jobs, n_jobs, L, S, G)
-    if (G.shape == COLS) {
+    if (G.s.shape == COLS) {
         if constexpr (!Q1) CKKS_COLS(6, 7);
         CKKS_COLS(7, 7);
         CKKS_COLS(7, 8);

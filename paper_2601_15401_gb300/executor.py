@@ -267,14 +267,39 @@ def one_per_launch(contexts, requests, executor: BatchExecutor):
 # autotuner
 # ---------------------------------------------------------------------------
 TUNE_SPACE = {
-    "ntt_tile_cols": [2048, 4096, 8192],
-    "ntt_tile_blocks": [1024, 2048, 4096],
-    "bconv_threads": [128, 256, 512],
-    "mac_threads": [128, 256, 512],
+    "ntt_tile_cols": [1024, 2048, 4096],
+    "ntt_tile_blocks": [512, 1024, 2048, 4096],
+    "bconv_threads": [64, 128, 256],
+    "mac_threads": [64, 128, 256],
 }
 # the library's defaults (Context in csrc/internal.h): the reference every
 # candidate's output is compared with
-TUNE_DEFAULTS = {"ntt_tile_cols": 4096, "ntt_tile_blocks": 4096, "bconv_threads": 256, "mac_threads": 256}
+TUNE_DEFAULTS = {"ntt_tile_cols": 4096, "ntt_tile_blocks": 1024, "bconv_threads": 256, "mac_threads": 256}
+
+
+def _tile_launch(name: str, value: int, log_n: int) -> int:
+    """What a tile size makes of the NTT's launches at a ring degree (the rule
+    of csrc/phase_shape.h): column groups / threads per CTA, 0 where a transform
+    is one launch without tiles."""
+    if log_n <= 12:
+        return 0
+    log_n1 = log_n // 2
+    if name == "ntt_tile_cols":
+        n = 1 << log_n1
+        return max(1, min(value // (16 * n), 256 // n, (1 << (log_n - log_n1)) // 16))
+    return max(32, min(value // 16, 256, (1 << log_n) // 16))
+
+
+def tune_values(name: str, log_n: int) -> list:
+    """The values of TUNE_SPACE[name] that are different launches at ring
+    degree 2^log_n; the default stands for its own."""
+    if not name.startswith("ntt_tile"):
+        return TUNE_SPACE[name]
+    default = TUNE_DEFAULTS[name]
+    one = {_tile_launch(name, default, log_n): default}
+    for v in TUNE_SPACE[name]:
+        one.setdefault(_tile_launch(name, v, log_n), v)
+    return sorted(one.values())
 
 
 def _cache_path() -> str:
@@ -293,7 +318,8 @@ def tune_key(ctx: Context) -> str:
 def autotune(ctx: Context, evk, k: int = 8, batch: int = 4, reps: int = 3, cache: str | None = None,
              force: bool = False) -> dict:
     """Pick each tunable by timing a batched k-input product (coordinate
-    descent over TUNE_SPACE, CUDA events), store the choice in a JSON cache
+    descent over the values of TUNE_SPACE that
+    are different launches at this N, CUDA events), store the choice in a JSON cache
     keyed by GPU, N, the prime-chain shape and the library's source hash, and
     apply it to `ctx`.
 
@@ -357,7 +383,10 @@ def autotune(ctx: Context, evk, k: int = 8, batch: int = 4, reps: int = 3, cache
 
     choice = dict(TUNE_DEFAULTS)
     trials, rejected = {}, []
-    for name, values in TUNE_SPACE.items():
+    for name in TUNE_SPACE:
+        values = tune_values(name, ctx.log_n)
+        if len(values) == 1:  # one launch whatever the value: the default
+            continue
         best = None
         for v in values:
             ctx.tune_set(name, v)
