@@ -813,11 +813,22 @@ def run_reference(args, rank, world):
             "e2e": {"value": v, "unit": UNIT, "h2d_bytes_per_step": 0, "d2h_bytes_per_step": 0}}
 
 
-KERNEL_SOURCES = {
-    "ntt": ["ntt.cu", "ntt_kernel.cuh", "ntt_uf.cu", "ntt_ui.cu", "ntt_tf.cu", "ntt_ti.cu", "ntt_uf1.cu", "ntt_ui1.cu",
-            "ntt_tf1.cu", "ntt_ti1.cu", "arith.cuh", "common.cuh", "internal.h"],
-    "rns": ["rns.cu", "tensor_fixed.cu", "rns.h", "arith.cuh", "common.cuh", "internal.h"],
-}
+def kernel_sources(group: str) -> list:
+    """Sources of a group of kernel classes: its translation units ("ntt": every
+    ntt*.cu that the build compiles) and the library headers they include,
+    directly or not."""
+    import re
+    from paper_2601_15401_gb300.build import SOURCES
+    csrc = os.path.join(ROOT, "paper_2601_15401_gb300", "csrc")
+    todo = [f for f in SOURCES if f.startswith("ntt")] if group == "ntt" else ["rns.cu", "tensor_fixed.cu"]
+    files = set()
+    while todo:
+        f = todo.pop()
+        if f in files or not os.path.exists(os.path.join(csrc, f)):
+            continue
+        files.add(f)
+        todo += re.findall(r'^\s*#\s*include\s+"([^"]+)"', open(os.path.join(csrc, f)).read(), re.M)
+    return sorted(files)
 
 
 def source_hash(kernel_class: str = "ntt") -> str:
@@ -827,7 +838,7 @@ def source_hash(kernel_class: str = "ntt") -> str:
     h = hashlib.sha256()
     csrc = os.path.join(ROOT, "paper_2601_15401_gb300", "csrc")
     group = "ntt" if kernel_class.startswith("ntt") else "rns"
-    for f in KERNEL_SOURCES[group]:
+    for f in kernel_sources(group):
         h.update(open(os.path.join(csrc, f), "rb").read())
     return h.hexdigest()[:16]
 
