@@ -1,6 +1,6 @@
 // Negacyclic NTT / INTT phase kernels over 64-bit NTT-friendly primes
-// (device code; instantiated by ntt_[ut][fi][1].cu and ntt_whole_[ut].cu, the
-// host logic is in ntt.cu).
+// (device code; instantiated by ntt_[ut][fi][1].cu and ntt_whole_[ut][fi].cu, the
+// host logic is in ntt.cu and phase_shape.h).
 //
 // The transform is the evaluation map A[i] = sum_j a_j psi^((2 brv(i)+1) j)
 // (bit-reversed order), computed with Cooley-Tukey butterflies forward and
@@ -494,7 +494,7 @@ struct Lane {
 };
 
 template <int LOGN, int LOGN2, bool FWD, int SH, int LM, int SM, bool SMALL, bool Q1, int I>
-__device__ __forceinline__ void run_passes(const Lane &ln, u64 q, const LoadCtx &lc, const StoreCtx &sc, int N1) {
+__device__ __forceinline__ void run_passes(const Lane &ln, u64 q, const LoadCtx &lc, const StoreCtx &sc) {
     constexpr int NP = Pass<LOGN, 0>::NP;
     if constexpr (I < NP) {
         typedef Geo<LOGN, LOGN2, SH> G;
@@ -550,7 +550,7 @@ __device__ __forceinline__ void run_passes(const Lane &ln, u64 q, const LoadCtx 
             }
         }
         if constexpr (!gout && last) pass_sync<SH>();
-        run_passes<LOGN, LOGN2, FWD, SH, LM, SM, SMALL, Q1, I + 1>(ln, q, lc, sc, N1);
+        run_passes<LOGN, LOGN2, FWD, SH, LM, SM, SMALL, Q1, I + 1>(ln, q, lc, sc);
     }
 }
 
@@ -603,7 +603,7 @@ __device__ __forceinline__ void phase_tile(u64 *sm, const NttPhase &P, const ulo
         // pass's loads are in flight
         for (int i = tid; i < n; i += blockDim.x) tws[i] = tw[i];
         grid_dependency_wait();
-        run_passes<LOGN, LOGN2, FWD, SH, LM, SM, SMALL, Q1, 0>(ln, q, lc, sc, P.N1);
+        run_passes<LOGN, LOGN2, FWD, SH, LM, SM, SMALL, Q1, 0>(ln, q, lc, sc);
     } else {
         // a warp and its blocks, or the CTA and its limb
         constexpr int BW = G::warp_blocks;
@@ -652,7 +652,7 @@ __device__ __forceinline__ void phase_tile(u64 *sm, const NttPhase &P, const ulo
                 }
             }
         }
-        run_passes<LOGN, LOGN2, FWD, SH, LM, SM, SMALL, Q1, 0>(ln, q, lc, sc, P.N1);
+        run_passes<LOGN, LOGN2, FWD, SH, LM, SM, SMALL, Q1, 0>(ln, q, lc, sc);
         if constexpr (RT) {
 #pragma unroll 1
             for (int idx = lane; idx < W * T; idx += T)
@@ -789,8 +789,8 @@ static inline cudaError_t launch_table(const NttPhase &P, const NttJob *jobs, in
 }
 
 // Dispatch of one direction (FWD) and job source (TABLE) over the shape, log2
-// n and the modes. Every pair of modes the library uses has its own kernel
-// (a kernel with run-time modes kept every mode's pointers alive and its code
+// n and the modes. Every pair of modes the library uses has its own kernel, for
+// tables those that waves use (a kernel with run-time modes kept every mode's pointers alive and its code
 // did not fit the instruction cache: 12-18 us a launch at N = 2^10 against
 // 5-7): a phase that fuses a mode has the plain mode on its other side.
 //   two phases (N >= 2^13): dispatch_two, with the products in the form Q1
@@ -811,9 +811,10 @@ static inline cudaError_t dispatch_cols(const NttPhase &P, const LimbJobs *J, co
     if constexpr (FWD) {
         CKKS_MODES(LD_PLAIN, ST_LAZY) CKKS_LAUNCH(LG, LG2, COLS, LD_PLAIN, ST_LAZY, CKKS_NTT_COL_MINB, Q1);
         CKKS_MODES(LD_EQ17, ST_LAZY) CKKS_LAUNCH(LG, LG2, COLS, LD_EQ17, ST_LAZY, CKKS_NTT_COL_WIDE_MINB, Q1);
-        CKKS_MODES(LD_BCONVK, ST_LAZY) CKKS_LAUNCH(LG, LG2, COLS, LD_BCONVK, ST_LAZY, CKKS_NTT_COL_BCONVK_MINB, Q1);
-        if constexpr (!TABLE)
+        if constexpr (!TABLE) {
+            CKKS_MODES(LD_BCONVK, ST_LAZY) CKKS_LAUNCH(LG, LG2, COLS, LD_BCONVK, ST_LAZY, CKKS_NTT_COL_BCONVK_MINB, Q1);
             CKKS_MODES(LD_SIGNED, ST_LAZY) CKKS_LAUNCH(LG, LG2, COLS, LD_SIGNED, ST_LAZY, CKKS_NTT_COL_MODDOWN_MINB, Q1);
+        }
     } else {
         CKKS_MODES(LD_PLAIN, ST_SCALE) CKKS_LAUNCH(LG, LG2, COLS, LD_PLAIN, ST_SCALE, CKKS_NTT_COL_MINB, Q1);
         CKKS_MODES(LD_PLAIN, ST_MODDOWN) CKKS_LAUNCH(LG, LG2, COLS, LD_PLAIN, ST_MODDOWN, CKKS_NTT_COL_MODDOWN_MINB, Q1);
@@ -827,7 +828,8 @@ static inline cudaError_t dispatch_blocks(const NttPhase &P, const LimbJobs *J, 
     if constexpr (FWD) {
         CKKS_MODES(LD_PLAIN, ST_REDUCE) CKKS_LAUNCH(LG, LG, BLOCKS, LD_PLAIN, ST_REDUCE, CKKS_NTT_BLOCK_MINB, Q1);
         CKKS_MODES(LD_PLAIN, ST_MRS) CKKS_LAUNCH(LG, LG, BLOCKS, LD_PLAIN, ST_MRS, CKKS_NTT_BLOCK_MINB, Q1);
-        CKKS_MODES(LD_PLAIN, ST_ADDSUB) CKKS_LAUNCH(LG, LG, BLOCKS, LD_PLAIN, ST_ADDSUB, CKKS_NTT_BLOCK_MINB, Q1);
+        if constexpr (!TABLE)
+            CKKS_MODES(LD_PLAIN, ST_ADDSUB) CKKS_LAUNCH(LG, LG, BLOCKS, LD_PLAIN, ST_ADDSUB, CKKS_NTT_BLOCK_MINB, Q1);
     } else {
         CKKS_MODES(LD_PLAIN, ST_LAZY) CKKS_LAUNCH(LG, LG, BLOCKS, LD_PLAIN, ST_LAZY, CKKS_NTT_BLOCK_MINB, Q1);
         CKKS_MODES(LD_ADD, ST_LAZY) CKKS_LAUNCH(LG, LG, BLOCKS, LD_ADD, ST_LAZY, CKKS_NTT_BLOCK_MINB, Q1);
@@ -869,7 +871,8 @@ static inline cudaError_t dispatch_whole_n(const NttPhase &P, const LimbJobs *J,
     } else {
         CKKS_MODES(LD_PLAIN, ST_SCALE) CKKS_LAUNCH(LG, 0, WHOLE, LD_PLAIN, ST_SCALE, 2, false);
         CKKS_MODES(LD_ADD, ST_MODDOWN) CKKS_LAUNCH(LG, 0, WHOLE, LD_ADD, ST_MODDOWN, 2, false);
-        CKKS_MODES(LD_PLAIN, ST_MODDOWN) CKKS_LAUNCH(LG, 0, WHOLE, LD_PLAIN, ST_MODDOWN, 2, false);
+        if constexpr (!TABLE)
+            CKKS_MODES(LD_PLAIN, ST_MODDOWN) CKKS_LAUNCH(LG, 0, WHOLE, LD_PLAIN, ST_MODDOWN, 2, false);
     }
     return cudaErrorInvalidValue;
 }
@@ -915,7 +918,7 @@ static inline cudaError_t dispatch_tiny(int logn, const NttPhase &P, const LimbJ
 
 // One translation unit per direction, job source (u: uniform, t: table) and
 // product form (ntt_*1.cu: primes = 1 (mod 2^32)) so that they compile in
-// parallel; ntt_whole.cu holds the one-phase kernels.
+// parallel; ntt_whole_*.cu hold the one-phase kernels.
 #define CKKS_DECL(name)                                                                              \
     cudaError_t name(int logn, const NttPhase &P, const LimbJobs *J, const NttJob *jobs, int n_jobs, \
                      const LoadSpec &L, const StoreSpec &S, const PhaseLaunch &G)
