@@ -306,11 +306,11 @@ def run_ours(args, rank, world, local_rank):
         achieved_ops = st["int_ops"] / (st["total_ms"] / 1e3) / 1e9
         roofline = {"bound": "alu", "kernel": dom[0],
                     "achieved": round(achieved_ops, 2), "peak": round(unit_peak / 1e9, 2) if unit_peak else None,
-                    "unit": "G Shoup products/s" if dom[0].startswith("ntt") else "G 128-bit MACs/s",
+                    "unit": "G Shoup products/s" if dom[0].startswith("ntt") else "G dot-product terms/s",
                     "frac": round(achieved_ops * 1e9 / unit_peak, 4) if unit_peak else None,
                     "traffic": traffic,
                     "peak_source": "measured in this run (ckks_peak_int: register-only stream of lazy NTT butterflies "
-                                   "/ 128-bit MACs over every SM, CUDA events, best of 5), the integer-multiply "
+                                   "/ dot-product terms on limbs over every SM, CUDA events, best of 5), the integer-multiply "
                                    "roofline of this GPU for the operation the kernel is built from"
                                    + (", the butterfly in the Shoup form for primes = 1 mod 2^32 that the kernels run"
                                       if q1_forms else ""),
@@ -429,12 +429,13 @@ def op_unit(kernel_class: str) -> str:
     if kernel_class.startswith("ntt"):
         return "butterfly"
     if kernel_class in ("bconv", "key_mac", "tensor"):
-        return "mac128"
+        return "dot_term"
     return ""
 
 
 def measure_int_peaks(G, params, q1: bool) -> dict:
-    """Rate of the lazy NTT butterfly and of the 128-bit MAC on this GPU
+    """Rate of the lazy NTT butterfly and of one term of a dot product (on limbs
+    for q < 2^60; the binding's name for it is "mac128") on this GPU
     (register-only kernels over every SM; operations/s), taken at the same
     point of the run as the timed steps. The butterfly is measured in the
     form the NTT kernels run (q1: the Shoup product for q = 1 mod 2^32);
@@ -445,7 +446,7 @@ def measure_int_peaks(G, params, q1: bool) -> dict:
 
     def rate(u):
         return max(G.peak_int(u, q, blocks=sms * per_sm, threads=256, iters=2048) for per_sm in (8, 16))
-    out = {"butterfly": rate("butterfly_q1" if q1 else "butterfly"), "mac128": rate("mac128")}
+    out = {"butterfly": rate("butterfly_q1" if q1 else "butterfly"), "dot_term": rate("mac128")}
     if q1:
         out["butterfly_general_form"] = rate("butterfly")
     return out

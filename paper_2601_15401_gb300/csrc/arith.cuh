@@ -203,7 +203,7 @@ CKKS_HD Canon make_canon(u64 q) {
     return c;
 }
 
-// u - floor(u / q) q or one q more, u < 256 q < 2^64 (unsigned): in [0, 2q).
+// u - floor(u / q) q or one q more, u < 256 q (unsigned 64-bit): in [0, 2q).
 CKKS_HD u64 reduce_near(u64 u, u64 q, Canon c) {
     const u32 k = ((u32)(u >> (c.shifts & 63)) * c.mul) >> (c.shifts >> 8);
     const u64 nq = 0ull - q;
@@ -295,7 +295,9 @@ struct DotLimbs {
         u64 x = sx - s0 - s1;
         x += s0 >> 30;
         s0 &= (1u << 30) - 1;
-        // s1 + (x >> 30) < 7 2^60 + 2^35: below 256 q for q >= 2^53
+        // operands are below q, their high limbs at most q / 2^30, so the high
+        // sum is at most 7 q^2 / 2^60 (after a fold 2 q + 6 q^2 / 2^60) and the
+        // middle one's high part 14 q / 2^30 + 8: below 256 q for every q < 2^60
         s1 = reduce_near(s1 + (x >> 30), q, c);
         x &= (1u << 30) - 1;
         sx = x + s0 + s1;

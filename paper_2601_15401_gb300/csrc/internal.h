@@ -128,7 +128,7 @@ struct Context {
     ulonglong2 *d_tw_fwd = nullptr;   // [L+K][N]
     ulonglong2 *d_tw_inv = nullptr;   // [L+K][N]
     Shoup *d_ninv = nullptr;          // [L+K]   N^-1
-    Shoup *d_one = nullptr;           // [L+K]   (1, floor(2^64/q)): x mod q for any x
+    Shoup *d_one = nullptr;           // [L+K]   1 as a product's constant: x mod q for signed |x| < 2^63 - 2^33
     Shoup *d_pscale = nullptr;        // [K]     N^-1 [phat_i^-1]_{p_i}
     u64 *d_cK = nullptr;              // [L+K][64]: row j < L: [p_i^-1 R]_{q_j}
     u64 *d_cK60 = nullptr;            // the same with R = 2^60 (products on limbs)
@@ -215,7 +215,7 @@ inline void count_kernel(const Context &C) { count_op(C, OP_KERNELS, 1); }
 
 // ntt.cu
 int twiddle_slot(int logN, int k);  // table position of twiddle k
-// phase launch over a device table of NttJob (ntt_launch.cu); jobs: device
+// phase launch over a device table of NttJob; jobs: device
 // array of n_jobs entries
 cudaError_t launch_ntt_phase_table(const Context &C, bool fwd, bool cols, const NttJob *jobs, int n_jobs,
                                    const LoadSpec &L, const StoreSpec &S, double alg_bytes, double ops,

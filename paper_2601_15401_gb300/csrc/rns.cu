@@ -355,7 +355,9 @@ cudaError_t launch_tensor_table(const Context &C, const TensorJob *jobs, int n_j
 // by HBM (4.9 TB/s for a k = 12 product, batch 4, multiply pipe 60 % busy), so
 // warps in flight count: 64 registers and one coefficient of a pair 1225 us
 // for batch 8, two at 80 or 128 registers 1240 / 1232; a single product 86
-// against 91 / 111 us (128-bit products, four coefficients: 111).
+// against 91 / 111 us (128-bit products, four coefficients: 111). At 64
+// registers the limb forms spill: 8 bytes a thread for pairs in a uniform
+// launch, about 100 for single products and in table launches.
 #ifndef CKKS_MAC_VEC
 #define CKKS_MAC_VEC 2
 #endif
@@ -376,7 +378,9 @@ __device__ __forceinline__ int key_limb_bits(u64 q, int key_digits) {
 // Coefficients per thread of BConv, its largest block (the "bconv_threads"
 // tunable is cut to it) and the CTAs of that size per SM it is compiled for
 // (k = 12, batch 8: 2009 us with three, 2188 with two; one coefficient per
-// thread 2239).
+// thread 2239). Digits of 13 to 16 primes spill some 110 bytes a thread;
+// two-input products with digits of 12 and 16 at N = 2^15, batch 4, take 545 and
+// 606 us (825 and 908 with the unspilled 128-bit kernels).
 #ifndef CKKS_BCONV_VEC
 #define CKKS_BCONV_VEC 2
 #endif
@@ -389,8 +393,11 @@ __device__ __forceinline__ int key_limb_bits(u64 q, int key_digits) {
 // CKKS_BCONV_VEC adjacent coefficients per thread (16-byte loads and stores
 // for two). y: limb 0 of the prescaled d_t; dst: slot 0 of the (t, digit)
 // ModUp output. Bound by the integer multiply pipe (81 % busy): |digit| products
-// per target and coefficient (k = 12, batch 4: 957 us; 1231 with 128-bit
-// products).
+// per target and coefficient, rounded up to AMAX (k = 12, batch 4: 957 us; 1231
+// with 128-bit products). A short last digit multiplies zeros: with digits of
+// eight 1.26x the products it needs at level 13, at most 2.27x (level 9); a
+// two-input product of level 9 at N = 2^15, batch 4, takes 241 us all the same
+// (391 with 128-bit products that skip them).
 // LIMB: the sources' limbs stay in registers, the constants hold their own
 // limbs in shared memory, a product is three multiply-adds; sums of more than
 // kLimbTerms30 sources are reduced in parts and added. Every lane reads the same

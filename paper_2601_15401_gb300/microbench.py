@@ -8,8 +8,8 @@ profiler captures (one kernel class at a time, a few GB on the device).
   python -m paper_2601_15401_gb300.microbench --op peak
 
 --op peak measures the GPU's rate of each integer operation of the hot path
-(lazy Shoup product, lazy NTT butterfly, 64 x 64 -> 128-bit MAC, Montgomery
-product) with register-only kernels over a sweep of grid sizes, for a 50-bit
+(lazy Shoup product, lazy NTT butterfly, one term of a dot product in the form
+the kernels run for the prime, Montgomery product) with register-only kernels over a sweep of grid sizes, for a 50-bit
 and a 60-bit prime: the integer roofline the NTT / BConv / MAC fractions are
 taken against.
 
