@@ -73,6 +73,9 @@ def test_the_search_times_each_launch_once(shapes):
             assert len(set(launches)) == len(launches)
             assert set(launches) == set(accepted.values())
             assert E.TUNE_DEFAULTS[name] in values
+    # a difference within two timings of one launch does not move a tunable
+    assert E.pick({128: 1.0, 256: 1.009}, 256) == 256 and E.pick({128: 1.0, 256: 1.02}, 256) == 128
+    assert E.pick({}, 256) == 256 and E.pick({128: 2.0, 64: 1.0}, 256) == 64
     # the other tunables: every value within what the kernels run
     for name in ("bconv_threads", "mac_threads"):
         assert E.tune_values(name, 16) == E.TUNE_SPACE[name] and max(E.TUNE_SPACE[name]) <= 256
